@@ -1154,14 +1154,25 @@ static int shape_hint(int c) {
 struct TuneEntry {
   int shape;            // index into kTuneShapes
   float us[kNShapes];   // time of each candidate, microseconds; 0 if not a candidate
+  float gram_us;        // time of the Gram form on the same phase; 0 if not timed
+  bool pinned;          // set by the caller (rss_autotune_set): this shape and no other
 };
 static std::mutex g_tune_m;
 static std::map<std::tuple<int, int, int>, TuneEntry> g_tune;
 
-template <typename T, typename Launch>
-static void tuned_id_launch(Factor<T> &F, int bmax, int nbox, Launch &&launch) {
+// gram: the exact-Gram form of the ID (id_gram.cu), when the factor may take
+// it; timed once per key beside the Householder shapes and used where it is
+// faster than all of them (a 512^2 grid's leaf phase of 1024 boxes 0.27 ms
+// against 1.2 ms, its phases of 4-64 boxes 0.09 against 0.4 ms), unless the
+// caller pinned a shape.  The widths that have no key take it by rule.
+template <typename T, typename Launch, typename Gram>
+static void tuned_id_launch(Factor<T> &F, int bmax, int nbox, Launch &&launch, bool have_gram, Gram &&gram) {
   const bool tunable = bmax > 0 && bmax <= 256 && !(F.flags & RSS_FLAG_NO_AUTOTUNE);
   if (!tunable) {
+    if (have_gram) {
+      gram();
+      return;
+    }
     set_id_groups(0);
     launch();
     return;
@@ -1170,44 +1181,56 @@ static void tuned_id_launch(Factor<T> &F, int bmax, int nbox, Launch &&launch) {
   while ((2 << bucket) <= nbox) bucket++;
   const int width = bmax <= 64 ? 64 : (bmax <= 128 ? 128 : 256);
   const auto key = std::make_tuple((int)sizeof(T), width, bucket);
-  int shape = -1;
+  TuneEntry te{-1, {}, 0.f, false};
   {
     std::lock_guard<std::mutex> lk(g_tune_m);
     auto it = g_tune.find(key);
-    if (it != g_tune.end()) shape = it->second.shape;
+    if (it != g_tune.end()) te = it->second;
   }
-  if (shape < 0) {
-    TuneEntry te{-1, {}};
+  const bool time_gram = have_gram && !te.pinned && te.gram_us == 0.f;
+  if (te.shape < 0 || time_gram) {
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
-    float best = 0.f;
-    for (int ci = 0; ci < kNShapes; ci++) {
-      const int tpc = kTuneShapes[ci][0], g = kTuneShapes[ci][1], ctas = kTuneShapes[ci][2];
-      if (!shape_fits(width, tpc, g, kTuneShapes[ci][3])) continue;  // the kernels' thread limits
-      if (ctas > 1 && width == 256 && tpc != 2) continue;  // the widest class: two threads per column
-      set_id_groups(shape_hint(ci));
+    auto timed = [&](auto &&fn) {
       float ms = 0.f;
       for (int rep = 0; rep < 2; rep++) {  // the second launch is timed
         CK(cudaEventRecord(e0, F.st));
-        launch();
+        fn();
         CK(cudaEventRecord(e1, F.st));
         CK(cudaEventSynchronize(e1));
         CK(cudaEventElapsedTime(&ms, e0, e1));
       }
-      te.us[ci] = std::max(1e3f * ms, 1e-3f);
-      if (te.shape < 0 || ms < best) {
-        best = ms;
-        te.shape = ci;
+      return std::max(1e3f * ms, 1e-3f);
+    };
+    if (te.shape < 0) {
+      float best = 0.f;
+      for (int ci = 0; ci < kNShapes; ci++) {
+        const int tpc = kTuneShapes[ci][0], g = kTuneShapes[ci][1], ctas = kTuneShapes[ci][2];
+        if (!shape_fits(width, tpc, g, kTuneShapes[ci][3])) continue;  // the kernels' thread limits
+        if (ctas > 1 && width == 256 && tpc != 2) continue;  // the widest class: two threads per column
+        set_id_groups(shape_hint(ci));
+        te.us[ci] = timed(launch);
+        if (te.shape < 0 || te.us[ci] < best) {
+          best = te.us[ci];
+          te.shape = ci;
+        }
       }
     }
+    if (time_gram) te.gram_us = timed(gram);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     std::lock_guard<std::mutex> lk(g_tune_m);
     auto ins = g_tune.insert({key, te});
-    shape = ins.first->second.shape;  // another thread may have tuned the key first
+    TuneEntry &have = ins.first->second;  // another thread may have tuned the key first
+    if (have.gram_us == 0.f && !have.pinned) have.gram_us = te.gram_us;
+    te = have;
   }
-  set_id_groups(shape_hint(shape));
+  if (have_gram && !te.pinned && te.gram_us < te.us[te.shape]) {
+    gram();
+    return;
+  }
+  set_id_groups(shape_hint(te.shape));
   launch();
   set_id_groups(0);
 }
@@ -1643,7 +1666,7 @@ template <typename T> static void run_factor(Factor<T> &F) {
   // only E is kept
   const bool symm = (F.flags & RSS_FLAG_SYMMETRIC_STORAGE) != 0;
   std::unordered_map<int64_t, int> child_b;  // (problem, node) -> sum of its children's b
-  DBuf gid, gel, gtri, gcnt;                 // per-phase ID and elimination scratch, grown as needed
+  DBuf gid, gel, gtri, gcnt, ggram;          // per-phase ID and elimination scratch, grown as needed
   if (F.mlp) F.d_ovf_used.alloc(sizeof(unsigned long long), st);
   // stages: (depth, weak).  RS-S: the strong step at depths maxdepth .. 2.
   // RS-WS (Sec. 3.4, Algorithm 2): at each depth a weak pass over the boxes,
@@ -1962,6 +1985,18 @@ template <typename T> static void run_factor(Factor<T> &F) {
       ims = IdMultiScratch{nullptr, 0, slots, ptr<int>(gcnt), kid_ctas};
     }
     set_id_multi(ims);
+    // the ID from the exact Gram matrix (FP32 factor, tolerances above its
+    // quantisation): partial sums of the largest phase
+    bool have_gram = false;
+    if constexpr (std::is_same<T, float>::value) {
+      have_gram = !large && F.eps >= ID_GRAM_EPS && H.bmax <= ID_GRAM_BMAX;
+      if (have_gram) {
+        int64_t need = 0;
+        for (auto &p : ph) need = std::max(need, id_gram_scratch_bytes(p.second, H.bmax, ring_max + F.px.np));
+        have_gram = need <= ID_GRAM_SCRATCH;
+        if (have_gram) grow(ggram, (size_t)need, st, 1);
+      }
+    }
     F.prof.host(KC_HOST_LEVEL, now_ms() - th0);
     for (auto &p : ph) {
       const int *bl = ptr<int>(d_list) + p.first;
@@ -1970,7 +2005,12 @@ template <typename T> static void run_factor(Factor<T> &F) {
                      ptr<T>(F.d_proxy), F.eps, ptr<T>(gid), id_stride, id_smem, st, ptr<int>(F.d_err));
       };
       int pi = F.prof.begin(KC_ID, st, base + p.first, p.second);
-      tuned_id_launch(F, large ? -H.bmax : H.bmax, p.second, id_launch);
+      auto gram_launch = [&] {
+        if constexpr (std::is_same<T, float>::value)
+          launch_id_gram(view, ptr<FBox<T>>(F.d_boxes), bl, p.second, H.bmax, ring_max, F.P, F.K, F.px,
+                         ptr<T>(F.d_proxy), F.eps, ggram.p, st, ptr<int>(F.d_err));
+      };
+      tuned_id_launch(F, large ? -H.bmax : H.bmax, p.second, id_launch, have_gram, gram_launch);
       check_launch("id");
       F.prof.end(pi, st);
       pi = F.prof.begin(KC_ELIM, st, base + p.first, p.second);
@@ -3474,7 +3514,7 @@ rss_status rss_autotune_set(int elem_bytes, int width, int phase_class, int tpc,
         (width == 256 && ctas > 1 && tpc != 2))
       throw Fail{RSS_EINVAL, "rss_autotune_set: bad arguments"};
     std::lock_guard<std::mutex> lk(g_tune_m);
-    TuneEntry te{shape, {}};
+    TuneEntry te{shape, {}, 0.f, true};
     g_tune[std::make_tuple(elem_bytes, width, phase_class)] = te;
   });
 }

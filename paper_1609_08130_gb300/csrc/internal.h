@@ -118,6 +118,17 @@ struct IdMultiScratch {
   int kid_ctas = 0;
 };
 void set_id_multi(const IdMultiScratch &m);
+// The FP32 factor's ID from the exact Gram matrix of its rows (id_gram.cu):
+// tolerances from ID_GRAM_EPS up (five times the quantisation), boxes up to
+// ID_GRAM_BMAX wide (one CTA's threads run the pivoted Cholesky), scratch
+// (id_gram_scratch_bytes for a phase of nbox boxes, m rows) up to 4 GB.
+constexpr double ID_GRAM_EPS = 5e-7;
+constexpr int ID_GRAM_BMAX = 512;
+constexpr int64_t ID_GRAM_SCRATCH = (int64_t)4 << 30;
+int64_t id_gram_scratch_bytes(int nbox, int bmax, int m);
+void launch_id_gram(const LevelDev<float> &lv, FBox<float> *boxes, const int *box_list, int nbox, int bmax,
+                    int ring_max, const Points &P, const KernelParams &K, const ProxyParams &px,
+                    const float *proxy_unit, double eps, void *scratch, cudaStream_t st, int *err);
 template <typename T>
 void launch_elim(const LevelDev<T> &lv, FBox<T> *boxes, const int *box_list, int nbox, int bmax,
                  T *scratch, int64_t scratch_stride, const Overflow<T> &ovf, cudaStream_t st, int *err, int njmax);

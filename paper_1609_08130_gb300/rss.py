@@ -16,7 +16,7 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 _CSRC = os.path.join(_HERE, "csrc")
 _INC = os.path.join(os.path.dirname(_HERE), "include")
 LIB_PATH = os.path.join(_HERE, "librss.so")
-SOURCES = ["api.cu", "kernels.cu", "refine.cu", "mlp.cu", "logdet.cu", "schur_tc.cu", "tree.cu"]
+SOURCES = ["api.cu", "kernels.cu", "refine.cu", "mlp.cu", "logdet.cu", "schur_tc.cu", "tree.cu", "id_gram.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_103a,code=sm_103a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-shared"]
 
@@ -42,13 +42,13 @@ def _nvcc():
 def build(force: bool = False) -> str:
     """Compile librss.so in-tree for sm_103a (translation units in parallel)."""
     srcs = [os.path.join(_CSRC, s) for s in SOURCES]
-    deps = srcs + [os.path.join(_CSRC, h) for h in ("common.cuh", "internal.h", "tc.cuh")] + \
+    deps = srcs + [os.path.join(_CSRC, h) for h in ("common.cuh", "internal.h", "tc.cuh", "df.cuh")] + \
         [os.path.join(_INC, "rss.h")]
     if not force and os.path.exists(LIB_PATH) and \
             os.path.getmtime(LIB_PATH) >= max(os.path.getmtime(d) for d in deps):
         return LIB_PATH
     tmp = LIB_PATH + f".tmp{os.getpid()}"
-    cmd = [_nvcc(), *NVCC_FLAGS, "--threads", "4", "-o", tmp, *srcs]
+    cmd = [_nvcc(), *NVCC_FLAGS, "--threads", "8", "-o", tmp, *srcs]
     subprocess.check_call(cmd)
     os.replace(tmp, LIB_PATH)
     return LIB_PATH
