@@ -912,6 +912,7 @@ template <typename T> struct Factor : FactorBase {
   mutable bool grid_ready = false, grid_f32_ready = false;
   int mv_ntile = 0;
   DBuf d_mv_ts, d_mv_te, d_mv_sb, d_mv_se;
+  DBuf d_mv_split;  // the points in FP32 parts (direct summation only)
   // rank proposal: the network (borrowed during rss_factor only), the
   // features of every box (MLP_NFEAT each, box order) and storage accounting
   // solve sweeps: work items (box, chunk) of every phase, per-box counters,
@@ -1431,6 +1432,11 @@ template <typename T> static void run_factor(Factor<T> &F) {
   F.d_err.alloc(sizeof(int), st);
   CK(cudaMemsetAsync(F.d_err.p, 0, sizeof(int), st));
   detect_grid(F);
+  if (F.grid_side == 0 && n > 0) {
+    F.d_mv_split.alloc((size_t)matvec_split_bytes(n, dim), st);
+    matvec_split(F.P.x, n, dim, F.d_mv_split.p, st);
+    check_launch("point parts");
+  }
   {
     // proxy surface template (Sec. 3.2): unit circle with n_p equispaced
     // angles in 2D, Fibonacci sphere with n_p points in 3D
@@ -2429,12 +2435,19 @@ template <typename T> static void apply_A_impl(const Factor<T> &F, const double 
     }
     grid_op_apply(F.G, x, y, nrhs, F.st, f32);
   } else if (f32) {
-    launch_matvec_f32(F.P, F.K, ptr<int64_t>(F.d_perm), x, y, F.n, nrhs, F.mv_ntile, ptr<int64_t>(F.d_mv_ts),
-                      ptr<int64_t>(F.d_mv_te), ptr<int64_t>(F.d_mv_sb), ptr<int64_t>(F.d_mv_se), F.st);
+    launch_matvec_f32(F.dim, F.K, F.P.wdof, ptr<int64_t>(F.d_perm), x, y, F.n, nrhs, F.mv_ntile,
+                      ptr<int64_t>(F.d_mv_ts), ptr<int64_t>(F.d_mv_te), ptr<int64_t>(F.d_mv_sb),
+                      ptr<int64_t>(F.d_mv_se), F.d_mv_split.p, F.st);
   } else {
-    launch_matvec(ptr<double>(F.d_x), F.dim, F.K, F.P.wdof, ptr<int64_t>(F.d_perm), x, y, F.n, nrhs, F.mv_ntile,
-                  ptr<int64_t>(F.d_mv_ts), ptr<int64_t>(F.d_mv_te), ptr<int64_t>(F.d_mv_sb), ptr<int64_t>(F.d_mv_se),
-                  F.st);
+    // at most 32 columns at a time, so that the scratch stays a small part of
+    // the caller's vectors; stream-ordered, so calls do not share it
+    DBuf xbuf;
+    xbuf.alloc((size_t)matvec_x_bytes(F.n, std::min(nrhs, 32), F.mv_ntile), F.st);
+    for (int c = 0; c < nrhs; c += 32)
+      launch_matvec(ptr<double>(F.d_x), F.dim, F.K, F.P.wdof, ptr<int64_t>(F.d_perm), x + (int64_t)c * F.n,
+                    y + (int64_t)c * F.n, F.n, std::min(nrhs - c, 32), F.mv_ntile, ptr<int64_t>(F.d_mv_ts),
+                    ptr<int64_t>(F.d_mv_te), ptr<int64_t>(F.d_mv_sb), ptr<int64_t>(F.d_mv_se), F.d_mv_split.p,
+                    xbuf.p, F.st);
   }
   check_launch("residual operator");
 }

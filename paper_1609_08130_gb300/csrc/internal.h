@@ -187,16 +187,22 @@ template <typename T> int64_t elim_ws_elems(int bmax);
 template <typename T>
 void launch_permute(int dir, const int64_t *perm, const double *in, T *out_or_in, double *out,
                     int64_t n, int nrhs, cudaStream_t st);
+// y = A x by direct summation in pairs of FP32 numbers (matvec.cu), FP64 in
+// and out.  split: the points' parts (matvec_split, matvec_split_bytes); xbuf:
+// matvec_x_bytes of scratch.
+int64_t matvec_split_bytes(int64_t n, int dim);
+int64_t matvec_x_bytes(int64_t n, int nrhs, int ntile);
+void matvec_split(const double *x_tree, int64_t n, int dim, void *split, cudaStream_t st);
 void launch_matvec(const double *x_tree, int dim, const KernelParams &K, const double *wdof, const int64_t *perm,
                    const double *xin, double *yout, int64_t n, int nrhs, int ntile, const int64_t *tstart,
-                   const int64_t *tend, const int64_t *sbeg, const int64_t *send, cudaStream_t st);
-// The same product with the kernel evaluated and summed in FP32 (the
-// points' distances from their depth-20 cells and offsets, as the FP32
-// factor's blocks; each tile of 256 sources summed in FP32, the tiles in
-// FP64): the operator of the inner GMRES of the refinement.
-void launch_matvec_f32(const Points &P, const KernelParams &K, const int64_t *perm, const double *xin,
+                   const int64_t *tend, const int64_t *sbeg, const int64_t *send, const void *split, void *xbuf,
+                   cudaStream_t st);
+// The same product with the kernel evaluated in FP32 and at most 256 terms
+// summed in FP32, those sums in FP64: the operator of the inner GMRES of the
+// refinement.
+void launch_matvec_f32(int dim, const KernelParams &K, const double *wdof, const int64_t *perm, const double *xin,
                        double *yout, int64_t n, int nrhs, int ntile, const int64_t *tstart, const int64_t *tend,
-                       const int64_t *sbeg, const int64_t *send, cudaStream_t st);
+                       const int64_t *sbeg, const int64_t *send, const void *split, cudaStream_t st);
 
 // FP64 operator x -> A x for points on an s^d grid of cell centres, by FFT
 // convolution on the circulant of side L = 2s (refine.cu).
