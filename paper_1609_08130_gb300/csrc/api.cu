@@ -917,7 +917,10 @@ template <typename T> struct Factor : FactorBase {
   // features of every box (MLP_NFEAT each, box order) and storage accounting
   // solve sweeps: work items (box, chunk) of every phase, per-box counters,
   // partial sums of the backward sweep
-  DBuf d_wbox, d_wchunk, d_wcnt, d_pbuf, d_poff;
+  DBuf d_wbox, d_wchunk, d_poff;
+  mutable DBuf d_wcnt, d_pbuf;
+  mutable int work_groups = 1;  // column groups d_wcnt and d_pbuf hold
+  int64_t pbuf_elems = 0;       // partial sums of one group
   const struct MlpModel *mlp = nullptr;
   std::vector<float> feats;
   int64_t reserved_T = 0, used_T = 0, ovf_used = 0;  // elements of T
@@ -2139,7 +2142,9 @@ template <typename T> static void run_factor(Factor<T> &F) {
     upload(F.d_poff, poff, st);
     F.d_wcnt.alloc(sizeof(int) * std::max<size_t>(F.h_boxes.size(), 1), st);
     CK(cudaMemsetAsync(F.d_wcnt.p, 0, sizeof(int) * std::max<size_t>(F.h_boxes.size(), 1), st));
-    F.d_pbuf.alloc(sizeof(T) * std::max<int64_t>(poff.back(), 1), st);
+    F.pbuf_elems = std::max<int64_t>(poff.back(), 1);
+    F.work_groups = 1;
+    F.d_pbuf.alloc(sizeof(T) * F.pbuf_elems, st);
   }
 
   // top blocks: every problem's DOFs still active (Sec. 3.3.3), dense LU
@@ -2244,19 +2249,43 @@ template <typename F> static rss_status guard(F &&fn) {
   }
 }
 
-// One phase of a sweep: the chunked solve kernels when they apply, else the
-// one-CTA-per-box kernel (apply sweeps, more than four right-hand sides, the
-// forced large-box path).
+// Counters and partial sums for `groups` groups of columns.
+template <typename T> static void ensure_groups(const Factor<T> &F, int groups) {
+  if (F.work_groups >= groups) return;
+  const size_t nb = sizeof(int) * std::max<size_t>(F.h_boxes.size(), 1) * groups;
+  F.d_wcnt.alloc(nb, F.st);
+  CK(cudaMemsetAsync(F.d_wcnt.p, 0, nb, F.st));
+  F.d_pbuf.alloc(sizeof(T) * (size_t)F.pbuf_elems * groups, F.st);
+  F.work_groups = groups;
+  F.work_gen++;  // captured sweeps hold the old buffers
+}
+
+// Whether the chunked kernels take groups of nr <= 4 columns of this phase
+// (else one CTA per box: the forced large-box path, boxes of over a thousand
+// DOFs).
+template <typename T> static bool chunked(const Phase &p, int nr) {
+  return nr <= 4 && p.njmax >= 0 && sweep_chunk_smem(p.bmax, nr, sizeof(T)) <= (size_t)(200 << 10);
+}
+// Columns per group of a call: all of them up to four, else four when every
+// phase takes groups, else one wide group.
+template <typename T> static int group_columns(const Factor<T> &F, int nrhs) {
+  if (nrhs <= 4) return nrhs;
+  for (const Phase &p : F.phases)
+    if (!chunked<T>(p, 4)) return nrhs;
+  return 4;
+}
+
+// One phase of a sweep over `groups` groups of nr columns.
 template <typename T>
-static void sweep_phase(const Factor<T> &F, int mode, const Phase &p, T *v, int nrhs, cudaStream_t st) {
-  const bool solve = mode == SWEEP_SOLVE_FWD || mode == SWEEP_SOLVE_BWD;
-  if (solve && nrhs <= 4 && p.njmax >= 0 && sweep_chunk_smem(p.bmax, nrhs, sizeof(T)) <= (size_t)(200 << 10)) {
-    launch_sweep_chunks<T>(mode, ptr<FBox<T>>(F.d_boxes), ptr<int>(F.d_wbox) + p.wfirst, ptr<int>(F.d_wchunk) + p.wfirst,
-                           p.wcount, v, nrhs, p.bmax, ptr<int>(F.d_wcnt), ptr<T>(F.d_pbuf), ptr<int64_t>(F.d_poff), st,
-                           p.shared);
+static void sweep_phase(const Factor<T> &F, int mode, const Phase &p, T *v, int nr, int groups, cudaStream_t st) {
+  if (mode != SWEEP_APPLY_W && chunked<T>(p, nr)) {
+    const SweepWork<T> w{ptr<FBox<T>>(F.d_boxes), ptr<int>(F.d_wbox) + p.wfirst, ptr<int>(F.d_wchunk) + p.wfirst,
+                         p.wcount, ptr<int>(F.d_wcnt), (int)F.h_boxes.size(), ptr<T>(F.d_pbuf), F.pbuf_elems,
+                         ptr<int64_t>(F.d_poff)};
+    launch_sweep_chunks<T>(mode, w, p.bmax, v, F.n, nr, groups, st);
     return;
   }
-  launch_sweep<T>(mode, ptr<FBox<T>>(F.d_boxes), p.first, p.count, v, nrhs, p.bmax, p.njmax, st, p.shared);
+  launch_sweep<T>(mode, ptr<FBox<T>>(F.d_boxes), p.first, p.count, v, nr, p.bmax, p.njmax, st, p.shared);
 }
 
 // Every launch of one application of F (Eq. 3.10) or F^{-1} (Eq. 3.11) on
@@ -2273,28 +2302,29 @@ static void enqueue_sweeps(const Factor<T> &F, const double *in, double *out, T 
     if (prof) P.end(pi, st);
   };
   const double sz = sizeof(T);
+  const int nr = group_columns(F, nrhs), groups = (nrhs + nr - 1) / nr;
   int pi = begin(KC_PERMUTE, 0, 0, 0, (double)F.n * nrhs * (8.0 + sz + 8.0));
-  launch_permute<T>(0, ptr<int64_t>(F.d_perm), in, v, nullptr, F.n, nrhs, st);
+  launch_permute<T>(0, ptr<int64_t>(F.d_perm), in, v, nullptr, F.n, nrhs, nr, st);
   end(pi);
   const int fwd = solve ? SWEEP_SOLVE_FWD : SWEEP_APPLY_FWD, bwd = solve ? SWEEP_SOLVE_BWD : SWEEP_APPLY_BWD;
   for (const Phase &p : F.phases) {
     pi = begin(KC_SWEEP, p.first, p.count, nrhs);
-    sweep_phase<T>(F, fwd, p, v, nrhs, st);
+    sweep_phase<T>(F, fwd, p, v, nr, groups, st);
     end(pi);
   }
   double nt = F.ntop;
   pi = begin(KC_TOP, 0, 0, 0, nt * nt * sz + 2.0 * nt * nrhs * sz, 2.0 * nt * nt * nrhs);
   launch_top<T>(solve ? 0 : 1, ptr<T>(F.d_topLU), ptr<int64_t>(F.d_loff), ptr<int>(F.d_toppiv), ptr<int64_t>(F.d_top),
-                ptr<int64_t>(F.d_toff), ptr<int>(F.d_tn), F.nprob, F.ntop, v, nrhs, ptr<T>(F.d_topwork), st,
+                ptr<int64_t>(F.d_toff), ptr<int>(F.d_tn), F.nprob, F.ntop, v, F.n, nr, groups, ptr<T>(F.d_topwork), st,
                 F.d_topinv.p ? ptr<T>(F.d_topinv) : nullptr);
   end(pi);
   for (auto it = F.phases.rbegin(); it != F.phases.rend(); ++it) {
     pi = begin(KC_SWEEP, it->first, it->count, nrhs);
-    sweep_phase<T>(F, bwd, *it, v, nrhs, st);
+    sweep_phase<T>(F, bwd, *it, v, nr, groups, st);
     end(pi);
   }
   pi = begin(KC_PERMUTE, 0, 0, 0, (double)F.n * nrhs * (8.0 + sz + 8.0));
-  launch_permute<T>(1, ptr<int64_t>(F.d_perm), nullptr, v, out, F.n, nrhs, st);
+  launch_permute<T>(1, ptr<int64_t>(F.d_perm), nullptr, v, out, F.n, nrhs, nr, st);
   end(pi);
 }
 
@@ -2337,7 +2367,9 @@ template <typename T> static void capture_solve_graph(const Factor<T> &F, int nr
 template <typename T>
 static void do_sweeps(const Factor<T> &F, const double *in, double *out, int nrhs, bool solve, bool sync = true) {
   cudaStream_t st = F.st;
-  ensure_work(F, nrhs);
+  const int nr = group_columns(F, nrhs), groups = (nrhs + nr - 1) / nr;
+  ensure_work(F, nr * groups);
+  ensure_groups(F, groups);
   T *v = ptr<T>(F.d_work);
   const bool graphed = solve && F.use_graphs && nrhs <= 4 && F.n > 0;
   if (graphed && !(F.sgraph[nrhs].exec && F.sgraph[nrhs].gen == F.work_gen)) {
@@ -2753,7 +2785,7 @@ static void sqrt_apply(const Factor<T> &F, const double *x, double *y, int nrhs,
   T *v = ptr<T>(F.d_work);
   for (int c0 = 0; c0 < nrhs; c0 += c) {
     const int nc = std::min(c, nrhs - c0);
-    launch_permute<T>(0, ptr<int64_t>(F.d_perm), x + (size_t)c0 * F.n, v, nullptr, F.n, nc, st);
+    launch_permute<T>(0, ptr<int64_t>(F.d_perm), x + (size_t)c0 * F.n, v, nullptr, F.n, nc, nc, st);
     auto blocks = [&](int tr) {
       launch_chol_apply<T>(ptr<FBox<T>>(F.d_boxes), nbox, ptr<int64_t>(F.d_top), ptr<int64_t>(F.d_toff),
                            ptr<int>(F.d_tn), np, ptr<T>(F.d_chol), ptr<int64_t>(F.d_coff), v, nc, F.chol_rmax, tr,
@@ -2761,12 +2793,12 @@ static void sqrt_apply(const Factor<T> &F, const double *x, double *y, int nrhs,
     };
     if (!trans) {
       blocks(0);
-      for (auto it = F.phases.rbegin(); it != F.phases.rend(); ++it) sweep_phase<T>(F, SWEEP_APPLY_BWD, *it, v, nc, st);
+      for (auto it = F.phases.rbegin(); it != F.phases.rend(); ++it) sweep_phase<T>(F, SWEEP_APPLY_BWD, *it, v, nc, 1, st);
     } else {
-      for (const Phase &p : F.phases) sweep_phase<T>(F, SWEEP_APPLY_W, p, v, nc, st);
+      for (const Phase &p : F.phases) sweep_phase<T>(F, SWEEP_APPLY_W, p, v, nc, 1, st);
       blocks(1);
     }
-    launch_permute<T>(1, ptr<int64_t>(F.d_perm), nullptr, v, y + (size_t)c0 * F.n, F.n, nc, st);
+    launch_permute<T>(1, ptr<int64_t>(F.d_perm), nullptr, v, y + (size_t)c0 * F.n, F.n, nc, nc, st);
     check_launch("rss_sqrt_apply");
   }
   if (!F.async()) CK(cudaStreamSynchronize(st));
@@ -2826,24 +2858,25 @@ static void solve_noalloc(const Factor<T> &F, const double *b, double *x, int nr
     const int nc = std::min(c, nrhs - c0);
     const double *bc = b + (size_t)c0 * F.n;
     double *xc = x + (size_t)c0 * F.n;
-    launch_permute<T>(0, ptr<int64_t>(F.d_perm), bc, v, nullptr, F.n, nc, st);
-    for (const Phase &p : F.phases) sweep_phase<T>(F, SWEEP_SOLVE_FWD, p, v, nc, st);
+    launch_permute<T>(0, ptr<int64_t>(F.d_perm), bc, v, nullptr, F.n, nc, nc, st);
+    for (const Phase &p : F.phases) sweep_phase<T>(F, SWEEP_SOLVE_FWD, p, v, nc, 1, st);
     launch_top<T>(0, ptr<T>(F.d_topLU), ptr<int64_t>(F.d_loff), ptr<int>(F.d_toppiv), ptr<int64_t>(F.d_top),
-                  ptr<int64_t>(F.d_toff), ptr<int>(F.d_tn), F.nprob, F.ntop, v, nc, topwork, st,
+                  ptr<int64_t>(F.d_toff), ptr<int>(F.d_tn), F.nprob, F.ntop, v, F.n, nc, 1, topwork, st,
                   F.d_topinv.p ? ptr<T>(F.d_topinv) : nullptr);
-    for (auto it = F.phases.rbegin(); it != F.phases.rend(); ++it) sweep_phase<T>(F, SWEEP_SOLVE_BWD, *it, v, nc, st);
-    launch_permute<T>(1, ptr<int64_t>(F.d_perm), nullptr, v, xc, F.n, nc, st);
+    for (auto it = F.phases.rbegin(); it != F.phases.rend(); ++it) sweep_phase<T>(F, SWEEP_SOLVE_BWD, *it, v, nc, 1, st);
+    launch_permute<T>(1, ptr<int64_t>(F.d_perm), nullptr, v, xc, F.n, nc, nc, st);
     check_launch("rss_solve_noalloc");
   }
   if (!F.async()) CK(cudaStreamSynchronize(st));
 }
 
-// Columns in chunks small enough for the sweep kernels' shared-memory
-// vectors (3 b x columns entries of the widest box within 200 KB); calls of
-// up to 4 columns on factors of boxes up to ~2000 wide are one chunk.
+// Columns in passes: groups of four up to 64 columns, or (boxes too wide for
+// those kernels) as many as the one-CTA kernels' shared-memory vectors take
+// (3 b x columns entries of the widest box within 200 KB).
 template <typename T> static void sweeps_chunked(const Factor<T> &F, const double *in, double *out, int nrhs,
                                                  bool solve) {
-  const int cmax = sweep_columns(F, nrhs);
+  // groups of four: 64 columns a pass bound the working vectors
+  const int cmax = nrhs > 4 && group_columns(F, nrhs) == 4 ? 64 : sweep_columns(F, nrhs);
   for (int c0 = 0; c0 < nrhs; c0 += cmax)
     do_sweeps(F, in + (size_t)c0 * F.n, out + (size_t)c0 * F.n, std::min(cmax, nrhs - c0), solve);
 }

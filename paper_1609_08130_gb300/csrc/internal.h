@@ -155,16 +155,27 @@ void launch_logdet(const FBox<T> *boxes, int nbox, const T *topLU, const int64_t
 template <typename T>
 void launch_sweep(int mode, const FBox<T> *boxes, int first, int count, T *v, int nrhs, int bmax,
                   int njmax, cudaStream_t st, int shared = 0);
-// Solve sweeps over work items (box, chunk of SWEEP_CHUNK rows of J) for
-// nrhs <= 4; cnt: per-box counters (zero between launches); pbuf/poff: the
-// backward sweep's per-box partial sums (ceil(nj / SWEEP_CHUNK) x r x 4
-// elements per box).  Shared memory as sweep_chunk_smem.
+// Sweeps over work items (box, chunk of SWEEP_CHUNK rows of J) for groups of
+// nr <= 4 columns (sweep.cu): the group's vector is v + group * n * nr.  cnt:
+// per-box counters of each group (zero between launches); pbuf/poff: per-box
+// partial sums (ceil(nj / SWEEP_CHUNK) x r x 4 entries per box), pstride
+// apart between groups.  Shared memory as sweep_chunk_smem.
 constexpr int SWEEP_CHUNK = 128;
+template <typename T> struct SweepWork {
+  const FBox<T> *boxes;
+  const int *wbox, *wchunk;
+  int nwork;
+  int *cnt;
+  int nbox;
+  T *pbuf;
+  int64_t pstride;
+  const int64_t *poff;
+};
 template <typename T>
-void launch_sweep_chunks(int mode, const FBox<T> *boxes, const int *wbox, const int *wchunk, int nwork, T *v,
-                         int nrhs, int bmax, int *cnt, T *pbuf, const int64_t *poff, cudaStream_t st,
-                         int shared = 0);
-size_t sweep_chunk_smem(int bmax, int nrhs, int elem);
+void launch_sweep_chunks(int mode, const SweepWork<T> &w, int bmax, T *v, int64_t n, int nr, int groups,
+                         cudaStream_t st);
+size_t sweep_chunk_smem(int bmax, int nr, int elem);
+void sweep_chunk_attributes();
 // Set the shared-memory attributes of every sweep kernel on the current device.
 void sweep_kernel_attributes();
 // Top blocks: mode 0 solves with the LU factors (or, for one problem with
@@ -172,8 +183,8 @@ void sweep_kernel_attributes();
 // multiplies by the block.  launch_top_inverse forms Winv (n <= 1024).
 template <typename T>
 void launch_top(int mode, const T *LU, const int64_t *loff, const int *piv, const int64_t *top, const int64_t *toff,
-                const int *tn, int nprob, int ntop_total, T *v, int nrhs, T *work, cudaStream_t st,
-                const T *Winv = nullptr);
+                const int *tn, int nprob, int ntop_total, T *v, int64_t n, int nr, int groups, T *work,
+                cudaStream_t st, const T *Winv = nullptr);
 template <typename T> void launch_top_inverse(const T *LU, int n, T *W, cudaStream_t st);
 template <typename T>
 void launch_lu_batched(T *LU, const int64_t *loff, int *piv, const int64_t *toff, const int *tn, int nprob,
@@ -186,7 +197,7 @@ template <typename T> int64_t id_region_bytes(int b, int PR);
 template <typename T> int64_t elim_ws_elems(int bmax);
 template <typename T>
 void launch_permute(int dir, const int64_t *perm, const double *in, T *out_or_in, double *out,
-                    int64_t n, int nrhs, cudaStream_t st);
+                    int64_t n, int nrhs, int nr, cudaStream_t st);
 // y = A x by direct summation in pairs of FP32 numbers (matvec.cu), FP64 in
 // and out.  split: the points' parts (matvec_split, matvec_split_bytes); xbuf:
 // matvec_x_bytes of scratch.

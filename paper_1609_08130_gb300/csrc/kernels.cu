@@ -32,8 +32,6 @@ void count_launch(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 long long launches_total() { return g_launches.load(std::memory_order_relaxed); }
 
 constexpr int NT = 256;  // threads per CTA for the per-box kernels
-constexpr int SWEEP_TROWS = 4;  // rows of T^T v_S a warp of the forward sweep forms at once
-constexpr int SWEEP_MLP = 8;    // independent loads a sweep thread keeps in flight
 
 // Kernel attributes are set outside stream capture only (a captured launch
 // reuses the attribute set by an earlier uncaptured one).
@@ -3729,297 +3727,6 @@ __global__ void __launch_bounds__(NT) k_sweep(int mode, const FBox<T> *boxes, in
   }
 }
 
-// Solve sweeps (Eq. 3.11) for nrhs = NR <= 4 right-hand sides held in
-// registers, with every box's rows split into chunks of SWEEP_CHUNK so that
-// large boxes are spread over several CTAs.  The CTAs of one box meet at a
-// per-box counter: the last to finish (no waiting) writes the box's own S
-// and R entries, which every CTA of the box reads first, so the result does
-// not depend on which CTA is last.
-template <typename T, int NR>
-__device__ __forceinline__ void sweep_gather(const FBox<T> &fb, const T *v, T *vS, T *vR) {
-  const int k = fb.k, r = fb.r;
-  for (int e = threadIdx.x; e < k * NR; e += NT) vS[e] = v[fb.ids[e / NR] * NR + e % NR];
-  for (int e = threadIdx.x; e < r * NR; e += NT) vR[e] = v[fb.ids[k + e / NR] * NR + e % NR];
-}
-
-// Forward sweep (solve): tmp = v_R - T^T v_S; v_N -= E_N tmp over this CTA's
-// chunk of J; the last CTA of the box: v_S -= E_S tmp, v_R = X_RR^{-1} tmp.
-template <typename T, int NR>
-__global__ void __launch_bounds__(NT) k_sweep_fwd(const FBox<T> *boxes, const int *wbox, const int *wchunk, T *v,
-                                                  int *cnt, int shared) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int s_last;
-  const int bi = wbox[blockIdx.x], ch = wchunk[blockIdx.x];
-  const FBox<T> &fb = boxes[bi];
-  const int k = fb.k, r = fb.r, nj = fb.nj;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  T *vS = reinterpret_cast<T *>(smem_raw);  // k x NR
-  T *vR = vS + (size_t)k * NR;               // r x NR
-  T *tmp = vR + (size_t)r * NR;              // r x NR
-  T *part = tmp + (size_t)r * NR;            // partial sums of X_RR^{-1} tmp
-  sweep_gather<T, NR>(fb, v, vS, vR);
-  __syncthreads();
-  // tmp = v_R - T^T v_S: a warp per SWEEP_TROWS rows at once, so that the
-  // loads of all of them are in flight together
-  for (int ri0 = warp * SWEEP_TROWS; ri0 < r; ri0 += (NT / 32) * SWEEP_TROWS) {
-    T acc[SWEEP_TROWS][NR];
-#pragma unroll
-    for (int u = 0; u < SWEEP_TROWS; u++)
-#pragma unroll
-      for (int c = 0; c < NR; c++) acc[u][c] = (T)0;
-    for (int q = lane; q < k; q += 32) {
-      T tq[SWEEP_TROWS];
-#pragma unroll
-      for (int u = 0; u < SWEEP_TROWS; u++) tq[u] = ri0 + u < r ? __ldg(fb.Tm + q + (int64_t)(ri0 + u) * k) : (T)0;
-#pragma unroll
-      for (int u = 0; u < SWEEP_TROWS; u++)
-#pragma unroll
-        for (int c = 0; c < NR; c++) acc[u][c] += tq[u] * vS[q * NR + c];
-    }
-#pragma unroll
-    for (int u = 0; u < SWEEP_TROWS; u++)
-#pragma unroll
-      for (int c = 0; c < NR; c++) acc[u][c] = warp_sum(acc[u][c]);
-    if (lane == 0)
-#pragma unroll
-      for (int u = 0; u < SWEEP_TROWS; u++)
-        if (ri0 + u < r)
-#pragma unroll
-          for (int c = 0; c < NR; c++) tmp[(ri0 + u) * NR + c] = vR[(ri0 + u) * NR + c] - acc[u][c];
-  }
-  __syncthreads();
-  // rows of E: two threads per row, each over alternate columns, SWEEP_MLP
-  // loads in flight (the last group predicated); every lane of the warp
-  // calls this (valid or not) for the final shuffle
-  auto erow = [&](int a, bool valid, T *acc) {
-    const T *ea = fb.E + a;
-    const int h = tid & 1;
-    for (int ri = valid ? h : r; ri < r; ri += 2 * SWEEP_MLP) {
-      T ev[SWEEP_MLP];
-#pragma unroll
-      for (int u = 0; u < SWEEP_MLP; u++) ev[u] = ri + 2 * u < r ? __ldg(ea + (int64_t)(ri + 2 * u) * nj) : (T)0;
-#pragma unroll
-      for (int u = 0; u < SWEEP_MLP; u++)
-        if (ri + 2 * u < r)
-#pragma unroll
-          for (int c = 0; c < NR; c++) acc[c] += ev[u] * tmp[(ri + 2 * u) * NR + c];
-    }
-#pragma unroll
-    for (int c = 0; c < NR; c++) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], 1);
-  };
-  {
-    const int a = ch * SWEEP_CHUNK + (tid >> 1);
-    T acc[NR];
-#pragma unroll
-    for (int c = 0; c < NR; c++) acc[c] = (T)0;
-    const bool mine = a < nj && a >= k;
-    erow(a, a < nj, acc);
-    if (mine && (tid & 1) == 0) {
-      T *vg = v + fb.J[a] * NR;
-      if (shared) {  // near DOFs other boxes of the phase update too
-#pragma unroll
-        for (int c = 0; c < NR; c++) atomicAdd(vg + c, -acc[c]);
-      } else {
-#pragma unroll
-        for (int c = 0; c < NR; c++) vg[c] -= acc[c];
-      }
-    }
-  }
-  __syncthreads();
-  if (tid == 0) {
-    const int nchunk = max(1, (nj + SWEEP_CHUNK - 1) / SWEEP_CHUNK);
-    s_last = atomicAdd(cnt + bi, 1) == nchunk - 1;
-  }
-  __syncthreads();
-  if (!s_last) return;
-  if (tid == 0) cnt[bi] = 0;
-  // S rows of E (the head of J)
-  for (int a0 = 0; a0 < k; a0 += NT / 2) {
-    const int a = a0 + (tid >> 1);
-    T acc[NR];
-#pragma unroll
-    for (int c = 0; c < NR; c++) acc[c] = (T)0;
-    erow(a, a < k, acc);
-    if (a < k && (tid & 1) == 0) {
-      T *vg = v + fb.ids[a] * NR;
-#pragma unroll
-      for (int c = 0; c < NR; c++) vg[c] = vS[a * NR + c] - acc[c];
-    }
-  }
-  // D^{-1} on R: x_R = X_RR^{-1} tmp (rows split over nch groups of columns)
-  const int nch = r >= NT ? 1 : NT / r;
-  for (int i0 = 0; i0 < r; i0 += NT) {
-    const int i = i0 + tid % (r >= NT ? NT : r), g = r >= NT ? 0 : tid / r;
-    if (i < r && g < nch && tid < (r >= NT ? NT : nch * r)) {
-      T acc[NR];
-#pragma unroll
-      for (int c = 0; c < NR; c++) acc[c] = (T)0;
-      for (int l = g; l < r; l += SWEEP_MLP * nch) {
-        T xv[SWEEP_MLP];
-#pragma unroll
-        for (int u = 0; u < SWEEP_MLP; u++) xv[u] = l + u * nch < r ? __ldg(fb.Xi + i + (int64_t)(l + u * nch) * r) : (T)0;
-#pragma unroll
-        for (int u = 0; u < SWEEP_MLP; u++)
-          if (l + u * nch < r)
-#pragma unroll
-            for (int c = 0; c < NR; c++) acc[c] += xv[u] * tmp[(l + u * nch) * NR + c];
-      }
-#pragma unroll
-      for (int c = 0; c < NR; c++) part[((size_t)g * r + i) * NR + c] = acc[c];
-    }
-  }
-  __syncthreads();
-  for (int i = tid; i < r; i += NT) {
-    T *vg = v + fb.ids[k + i] * NR;
-#pragma unroll
-    for (int c = 0; c < NR; c++) {
-      T sum = (T)0;
-      for (int g = 0; g < nch; g++) sum += part[((size_t)g * r + i) * NR + c];
-      vg[c] = sum;
-    }
-  }
-}
-
-// Backward sweep (solve): partial sums of G v_J over this CTA's chunk of J
-// into pbuf; the last CTA of the box adds them in chunk order,
-// v_R -= G v_J, v_S -= T v_R, and writes v_R and v_S.
-template <typename T, int NR>
-__global__ void __launch_bounds__(NT) k_sweep_bwd(const FBox<T> *boxes, const int *wbox, const int *wchunk, T *v,
-                                                  int *cnt, T *pbuf, const int64_t *poff) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int s_last;
-  const int bi = wbox[blockIdx.x], ch = wchunk[blockIdx.x];
-  const FBox<T> &fb = boxes[bi];
-  const int k = fb.k, r = fb.r, nj = fb.nj;
-  const int tid = threadIdx.x;
-  T *part = reinterpret_cast<T *>(smem_raw);  // nch x r x NR, then vS, vR for the last CTA
-  T *vJc = part + (size_t)NT * NR;             // this chunk's entries of v_J
-  const int a0 = ch * SWEEP_CHUNK, a1 = min(nj, a0 + SWEEP_CHUNK), na = a1 - a0;
-  const int nch = r >= NT ? 1 : NT / r;
-  T *pb = pbuf + poff[bi] + (int64_t)ch * r * NR;
-  // G(i, a) = gq[i * gsi + a * gsa]: the stored G, or E^T under symmetric storage
-  const T *gq = fb.G ? fb.G : fb.E;
-  const int64_t gsi = fb.G ? 1 : nj, gsa = fb.G ? r : 1;
-  // the chunk's v_J gathered once, all loads in flight together
-  for (int e = tid; e < na * NR; e += NT) vJc[e] = v[fb.J[a0 + e / NR] * NR + e % NR];
-  __syncthreads();
-  for (int i0 = 0; i0 < r; i0 += NT) {
-    const int rr = r >= NT ? NT : r;
-    const int i = i0 + tid % rr, g = tid / rr;
-    if (i < r && g < nch) {
-      T acc[NR];
-#pragma unroll
-      for (int c = 0; c < NR; c++) acc[c] = (T)0;
-      const T *gi = gq + i * gsi + a0 * gsa;
-      for (int a = g; a < na; a += SWEEP_MLP * nch) {
-        T gv[SWEEP_MLP];
-#pragma unroll
-        for (int u = 0; u < SWEEP_MLP; u++) gv[u] = a + u * nch < na ? __ldg(gi + (a + u * nch) * gsa) : (T)0;
-#pragma unroll
-        for (int u = 0; u < SWEEP_MLP; u++)
-          if (a + u * nch < na)
-#pragma unroll
-            for (int c = 0; c < NR; c++) acc[c] += gv[u] * vJc[(a + u * nch) * NR + c];
-      }
-#pragma unroll
-      for (int c = 0; c < NR; c++) part[((size_t)g * rr + (i - i0)) * NR + c] = acc[c];
-    }
-    __syncthreads();
-    for (int e = tid; e < (r - i0 < rr ? r - i0 : rr) * NR; e += NT) {
-      const int il = e / NR, c = e % NR;
-      T sum = (T)0;
-      for (int g2 = 0; g2 < nch; g2++) sum += part[((size_t)g2 * rr + il) * NR + c];
-      pb[(int64_t)(i0 + il) * NR + c] = sum;
-    }
-    __syncthreads();
-  }
-  __threadfence();
-  if (tid == 0) {
-    const int nchunk = max(1, (nj + SWEEP_CHUNK - 1) / SWEEP_CHUNK);
-    s_last = atomicAdd(cnt + bi, 1) == nchunk - 1;
-  }
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  if (tid == 0) cnt[bi] = 0;
-  const int nchunk = max(1, (nj + SWEEP_CHUNK - 1) / SWEEP_CHUNK);
-  T *vS = part, *vR = part + (size_t)k * NR;
-  sweep_gather<T, NR>(fb, v, vS, vR);
-  __syncthreads();
-  const T *p0 = pbuf + poff[bi];
-  for (int e = tid; e < r * NR; e += NT) {
-    T sum = (T)0;
-    for (int c2 = 0; c2 < nchunk; c2++) sum += __ldcg(p0 + (int64_t)c2 * r * NR + e);
-    vR[e] -= sum;
-  }
-  __syncthreads();
-  // v_S -= T v_R: the columns of T split over nq groups of threads
-  // (SWEEP_MLP loads in flight each), the groups' partial sums added in group order
-  if (k > 0) {
-    const int kk = k >= NT ? NT : k, nq = k >= NT ? 1 : NT / k;
-    T *tp = part + (size_t)(k + r) * NR;  // nq x kk x NR partial sums
-    for (int q0 = 0; q0 < k; q0 += NT) {
-      const int q = q0 + tid % kk, g = tid / kk;
-      if (q < k && g < nq) {
-        T acc[NR];
-#pragma unroll
-        for (int c = 0; c < NR; c++) acc[c] = (T)0;
-        for (int ri = g; ri < r; ri += SWEEP_MLP * nq) {
-          T tv[SWEEP_MLP];
-#pragma unroll
-          for (int u = 0; u < SWEEP_MLP; u++) tv[u] = ri + u * nq < r ? __ldg(fb.Tm + q + (int64_t)(ri + u * nq) * k) : (T)0;
-#pragma unroll
-          for (int u = 0; u < SWEEP_MLP; u++)
-            if (ri + u * nq < r)
-#pragma unroll
-              for (int c = 0; c < NR; c++) acc[c] += tv[u] * vR[(ri + u * nq) * NR + c];
-        }
-#pragma unroll
-        for (int c = 0; c < NR; c++) tp[((size_t)g * kk + (q - q0)) * NR + c] = acc[c];
-      }
-      __syncthreads();
-      for (int e = tid; e < min(kk, k - q0) * NR; e += NT) {
-        const int ql = e / NR, c = e % NR;
-        T sum = (T)0;
-        for (int g2 = 0; g2 < nq; g2++) sum += tp[((size_t)g2 * kk + ql) * NR + c];
-        v[fb.ids[q0 + ql] * NR + c] = vS[(q0 + ql) * NR + c] - sum;
-      }
-      __syncthreads();
-    }
-  }
-  for (int e = tid; e < r * NR; e += NT) v[fb.ids[k + e / NR] * NR + e % NR] = vR[e];
-}
-
-template <typename T>
-void launch_sweep_chunks(int mode, const FBox<T> *boxes, const int *wbox, const int *wchunk, int nwork, T *v,
-                         int nrhs, int bmax, int *cnt, T *pbuf, const int64_t *poff, cudaStream_t st, int shared) {
-  if (nwork == 0) return;
-  const size_t smem = sweep_chunk_smem(bmax, nrhs, (int)sizeof(T));
-  constexpr int SMAX = (200 << 10) + 64;  // callers keep smem within this
-#define RSS_SWEEP_NR(NRV)                                                                                   \
-  case NRV:                                                                                                \
-    if (mode == SWEEP_SOLVE_FWD) {                                                                         \
-      if (!capturing(st)) cudaFuncSetAttribute(k_sweep_fwd<T, NRV>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMAX); \
-      k_sweep_fwd<T, NRV><<<nwork, NT, smem, st>>>(boxes, wbox, wchunk, v, cnt, shared);                           \
-    } else {                                                                                               \
-      if (!capturing(st)) cudaFuncSetAttribute(k_sweep_bwd<T, NRV>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMAX); \
-      k_sweep_bwd<T, NRV><<<nwork, NT, smem, st>>>(boxes, wbox, wchunk, v, cnt, pbuf, poff);               \
-    }                                                                                                      \
-    break;
-  switch (nrhs) {
-    RSS_SWEEP_NR(1)
-    RSS_SWEEP_NR(2)
-    RSS_SWEEP_NR(3)
-    RSS_SWEEP_NR(4)
-  }
-#undef RSS_SWEEP_NR
-  count_launch();
-}
-
-size_t sweep_chunk_smem(int bmax, int nrhs, int elem) {
-  return ((size_t)4 * bmax + NT + SWEEP_CHUNK) * nrhs * elem + 64;
-}
-
 template <typename T>
 void launch_sweep(int mode, const FBox<T> *boxes, int first, int count, T *v, int nrhs, int bmax, int njmax,
                   cudaStream_t st, int shared) {
@@ -4163,61 +3870,89 @@ void sweep_kernel_attributes() {
   constexpr int SMAX = (200 << 10) + 64;
   cudaFuncSetAttribute(k_sweep<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMAX);
   cudaFuncSetAttribute(k_sweep<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMAX);
-#define RSS_SWEEP_ATTR(TT, NRV)                                                                   \
-  cudaFuncSetAttribute(k_sweep_fwd<TT, NRV>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMAX); \
-  cudaFuncSetAttribute(k_sweep_bwd<TT, NRV>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMAX);
-  RSS_SWEEP_ATTR(float, 1) RSS_SWEEP_ATTR(float, 2) RSS_SWEEP_ATTR(float, 3) RSS_SWEEP_ATTR(float, 4)
-  RSS_SWEEP_ATTR(double, 1) RSS_SWEEP_ATTR(double, 2) RSS_SWEEP_ATTR(double, 3) RSS_SWEEP_ATTR(double, 4)
-#undef RSS_SWEEP_ATTR
+  sweep_chunk_attributes();
 }
 
 // Top blocks of one or more problems (Sec. 3.3.3): problem p has tn[p] DOFs
 // with global ids top[toff[p] ...], its LU (row-major, P A = L U) at
-// LU + loff[p] and pivots at piv + toff[p].  Solve (mode 0) or multiply
-// (mode 1); one CTA per (problem, right-hand side).
+// LU + loff[p] and pivots at piv + toff[p].  Solve: one CTA per (problem,
+// column) of a group (grid.y) of nrhs columns.
 template <typename T>
-__global__ void __launch_bounds__(1024) k_top(int mode, const T *LUall, const int64_t *loff, const int *pivall,
+__global__ void __launch_bounds__(1024) k_top(const T *LUall, const int64_t *loff, const int *pivall,
                                               const int64_t *topall, const int64_t *toff, const int *tn, T *v,
-                                              int nrhs, T *work) {
+                                              int64_t vstride, int nrhs, T *work, int64_t wstride) {
   const int p = blockIdx.x / nrhs, c = blockIdx.x % nrhs;
   const int n = tn[p];
   if (n == 0) return;
+  v += blockIdx.y * vstride;
   const T *LU = LUall + loff[p];
   const int *piv = pivall + toff[p];
   const int64_t *top = topall + toff[p];
-  T *y = work + 2 * (toff[p] * nrhs + (int64_t)c * n);
-  T *u = y + n;
+  T *y = work + blockIdx.y * wstride + 2 * (toff[p] * nrhs + (int64_t)c * n);
   const int tid = threadIdx.x;
-  if (mode == 0) {
-    for (int i = tid; i < n; i += blockDim.x) y[i] = v[top[piv[i]] * nrhs + c];
+  for (int i = tid; i < n; i += blockDim.x) y[i] = v[top[piv[i]] * nrhs + c];
+  __syncthreads();
+  for (int i = 0; i < n; i++) {
+    T yi = y[i];
+    for (int l = i + 1 + tid; l < n; l += blockDim.x) y[l] -= LU[(int64_t)l * n + i] * yi;
     __syncthreads();
-    for (int i = 0; i < n; i++) {
-      T yi = y[i];
-      for (int l = i + 1 + tid; l < n; l += blockDim.x) y[l] -= LU[(int64_t)l * n + i] * yi;
-      __syncthreads();
+  }
+  for (int i = n - 1; i >= 0; i--) {
+    T yi = y[i] / LU[(int64_t)i * n + i];
+    __syncthreads();
+    if (tid == 0) y[i] = yi;
+    for (int l = tid; l < i; l += blockDim.x) y[l] -= LU[(int64_t)l * n + i] * yi;
+    __syncthreads();
+  }
+  for (int i = tid; i < n; i += blockDim.x) v[top[i] * nrhs + c] = y[i];
+}
+
+// Multiply by the top blocks, v_top = P^T L U v_top, in two launches (half 0:
+// u = U v, half 1: v = P^T L u), a warp per row over the row-major factors,
+// all problems' rows in one grid (a CTA per problem and column reading the
+// rows down took 0.3 ms a column at n = 320 in FP64).
+template <typename T, int NR>
+__global__ void __launch_bounds__(256) k_top_mul(int half, const T *LUall, const int64_t *loff, const int *pivall,
+                                                 const int64_t *topall, const int64_t *toff, int nprob, int ntot, T *v,
+                                                 int64_t vstride, T *u, int64_t wstride) {
+  const int lane = threadIdx.x & 31, e = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (e >= ntot) return;
+  int lo = 0, hi = nprob - 1;  // the last problem starting at or before row e
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (toff[mid] <= e) lo = mid;
+    else hi = mid - 1;
+  }
+  const int64_t o = toff[lo];
+  const int n = (int)(toff[lo + 1] - o), i = (int)(e - o);
+  const T *row = LUall + loff[lo] + (int64_t)i * n;
+  const int64_t *top = topall + o;
+  v += blockIdx.y * vstride;
+  u += blockIdx.y * wstride;
+  T acc[NR];
+#pragma unroll
+  for (int c = 0; c < NR; c++) acc[c] = (T)0;
+  if (half == 0) {
+    for (int l = i + lane; l < n; l += 32) {
+      const T a = row[l];
+      const T *x = v + top[l] * NR;
+#pragma unroll
+      for (int c = 0; c < NR; c++) acc[c] += a * x[c];
     }
-    for (int i = n - 1; i >= 0; i--) {
-      T yi = y[i] / LU[(int64_t)i * n + i];
-      __syncthreads();
-      if (tid == 0) y[i] = yi;
-      for (int l = tid; l < i; l += blockDim.x) y[l] -= LU[(int64_t)l * n + i] * yi;
-      __syncthreads();
-    }
-    for (int i = tid; i < n; i += blockDim.x) v[top[i] * nrhs + c] = y[i];
   } else {
-    for (int i = tid; i < n; i += blockDim.x) y[i] = v[top[i] * nrhs + c];
-    __syncthreads();
-    for (int i = tid; i < n; i += blockDim.x) {
-      T s = (T)0;
-      for (int l = i; l < n; l++) s += LU[(int64_t)i * n + l] * y[l];
-      u[i] = s;
+    for (int l = lane; l < i; l += 32) {
+      const T a = row[l];
+      const T *x = u + (o + l) * NR;
+#pragma unroll
+      for (int c = 0; c < NR; c++) acc[c] += a * x[c];
     }
-    __syncthreads();
-    for (int i = tid; i < n; i += blockDim.x) {
-      T s = u[i];
-      for (int l = 0; l < i; l++) s += LU[(int64_t)i * n + l] * u[l];
-      v[top[piv[i]] * nrhs + c] = s;
-    }
+  }
+#pragma unroll
+  for (int c = 0; c < NR; c++) acc[c] = warp_sum(acc[c]);
+  if (lane == 0) {
+    T *out = half == 0 ? u + e * (int64_t)NR : v + top[pivall[e]] * NR;
+#pragma unroll
+    for (int c = 0; c < NR; c++) out[c] = half == 0 ? acc[c] : acc[c] + u[e * (int64_t)NR + c];
   }
 }
 
@@ -4265,19 +4000,53 @@ template <typename T> void launch_top_inverse(const T *LU, int n, T *W, cudaStre
   count_launch();
 }
 
-// y = P v_top (the pivoted gather), then v_top = W y with one warp per row.
+// The same for one group of more than four columns (boxes too wide for the
+// grouped sweeps, or the forced large-box path): one CTA per problem and
+// column, a warp per row.
 template <typename T>
-__global__ void k_top_gather(const int *piv, const int64_t *top, int n, const T *v, int nrhs, T *y) {
+__global__ void __launch_bounds__(256) k_top_mul_wide(const T *LUall, const int64_t *loff, const int *pivall,
+                                                      const int64_t *topall, const int64_t *toff, const int *tn, T *v,
+                                                      int nrhs, T *work) {
+  const int p = blockIdx.x / nrhs, c = blockIdx.x % nrhs, n = tn[p];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const T *LU = LUall + loff[p];
+  const int64_t *top = topall + toff[p];
+  T *y = work + 2 * (toff[p] * nrhs + (int64_t)c * n), *u = y + n;
+  for (int i = threadIdx.x; i < n; i += 256) y[i] = v[top[i] * nrhs + c];
+  __syncthreads();
+  for (int half = 0; half < 2; half++) {
+    const T *x = half == 0 ? y : u;
+    for (int i = warp; i < n; i += 8) {
+      T s = (T)0;
+      for (int l = (half == 0 ? i : 0) + lane; l < (half == 0 ? n : i); l += 32) s += LU[(int64_t)i * n + l] * x[l];
+      s = warp_sum(s);
+      if (lane == 0) {
+        if (half == 0) u[i] = s;
+        else v[top[pivall[toff[p] + i]] * nrhs + c] = u[i] + s;
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// y = P v_top (the pivoted gather), then v_top = W y with one warp per row;
+// grid.y: groups of NR columns.
+template <typename T>
+__global__ void k_top_gather(const int *piv, const int64_t *top, int n, const T *v, int64_t vstride, int nrhs, T *y,
+                             int64_t wstride) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= n * nrhs) return;
   const int kk = e / nrhs, c = e - kk * nrhs;
-  y[e] = v[top[piv[kk]] * nrhs + c];
+  y[blockIdx.y * wstride + e] = v[blockIdx.y * vstride + top[piv[kk]] * nrhs + c];
 }
 template <typename T, int NR>
-__global__ void __launch_bounds__(256) k_top_gemv(const T *W, const int64_t *top, int n, const T *y, T *v) {
+__global__ void __launch_bounds__(256) k_top_gemv(const T *W, const int64_t *top, int n, const T *y, int64_t wstride,
+                                                  T *v, int64_t vstride) {
   const int lane = threadIdx.x & 31;
   const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (i >= n) return;
+  y += blockIdx.y * wstride;
+  v += blockIdx.y * vstride;
   const T *Wi = W + (int64_t)i * n;
   T acc[NR];
 #pragma unroll
@@ -4296,23 +4065,41 @@ __global__ void __launch_bounds__(256) k_top_gemv(const T *W, const int64_t *top
     for (int c = 0; c < NR; c++) v[top[i] * NR + c] = acc[c];
 }
 
+template <typename T, int NR>
+static void launch_top_nr(int mode, const T *LU, const int64_t *loff, const int *piv, const int64_t *top,
+                          const int64_t *toff, int nprob, int ntop, T *v, int64_t vstride, int groups, T *work,
+                          int64_t wstride, const T *Winv, cudaStream_t st) {
+  const dim3 rows((unsigned)((ntop + 7) / 8), groups);
+  if (mode == 0) {
+    k_top_gather<T><<<dim3((unsigned)((ntop * NR + 255) / 256), groups), 256, 0, st>>>(piv, top, ntop, v, vstride, NR,
+                                                                                      work, wstride);
+    k_top_gemv<T, NR><<<rows, 256, 0, st>>>(Winv, top, ntop, work, wstride, v, vstride);
+  } else {
+    for (int half = 0; half < 2; half++)
+      k_top_mul<T, NR><<<rows, 256, 0, st>>>(half, LU, loff, piv, top, toff, nprob, ntop, v, vstride, work, wstride);
+  }
+  count_launch(2);
+}
+
 template <typename T>
 void launch_top(int mode, const T *LU, const int64_t *loff, const int *piv, const int64_t *top, const int64_t *toff,
-                const int *tn, int nprob, int ntop_total, T *v, int nrhs, T *work, cudaStream_t st, const T *Winv) {
+                const int *tn, int nprob, int ntop_total, T *v, int64_t n, int nr, int groups, T *work,
+                cudaStream_t st, const T *Winv) {
   if (ntop_total == 0 || nprob == 0) return;
-  if (mode == 0 && Winv && nprob == 1 && nrhs >= 1 && nrhs <= 4) {
-    const int n = ntop_total;
-    k_top_gather<T><<<(n * nrhs + 255) / 256, 256, 0, st>>>(piv, top, n, v, nrhs, work);
-    count_launch();
-    const unsigned g = (unsigned)((n + 7) / 8);
-    if (nrhs == 1) k_top_gemv<T, 1><<<g, 256, 0, st>>>(Winv, top, n, work, v);
-    else if (nrhs == 2) k_top_gemv<T, 2><<<g, 256, 0, st>>>(Winv, top, n, work, v);
-    else if (nrhs == 3) k_top_gemv<T, 3><<<g, 256, 0, st>>>(Winv, top, n, work, v);
-    else k_top_gemv<T, 4><<<g, 256, 0, st>>>(Winv, top, n, work, v);
+  const int64_t vs = n * nr, ws = (int64_t)2 * ntop_total * nr;
+  if (nr <= 4 && (mode == 1 || (Winv && nprob == 1))) {
+#define RSS_TOP_NR(N) \
+  case N: launch_top_nr<T, N>(mode, LU, loff, piv, top, toff, nprob, ntop_total, v, vs, groups, work, ws, Winv, st); break;
+    switch (nr) { RSS_TOP_NR(1) RSS_TOP_NR(2) RSS_TOP_NR(3) RSS_TOP_NR(4) }
+#undef RSS_TOP_NR
+    return;
+  }
+  if (mode == 1) {
+    k_top_mul_wide<T><<<nprob * nr, 256, 0, st>>>(LU, loff, piv, top, toff, tn, v, nr, work);
     count_launch();
     return;
   }
-  k_top<T><<<nprob * nrhs, 1024, 0, st>>>(mode, LU, loff, piv, top, toff, tn, v, nrhs, work);
+  k_top<T><<<dim3(nprob * nr, groups), 1024, 0, st>>>(LU, loff, piv, top, toff, tn, v, vs, nr, work, ws);
   count_launch();
 }
 
@@ -4401,26 +4188,31 @@ void launch_lu_batched(T *LU, const int64_t *loff, int *piv, const int64_t *toff
   count_launch();
 }
 
-// dir 0: out_t[g*nrhs+c] = in[perm[g] + c*n];  dir 1: out[perm[g] + c*n] = in_t[g*nrhs+c]
+// Caller order (column-major) to tree order (dir 0) or back (dir 1).  Tree-order
+// vectors hold groups of nr columns: column q nr + c of DOF g at
+// [(q n + g) nr + c]; columns past nrhs of the last group are zero.
 template <typename T>
-__global__ void k_permute(int dir, const int64_t *perm, const double *in, T *tv, double *out, int64_t n,
-                          int nrhs) {
-  int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (e >= n * nrhs) return;
-  int64_t g = e / nrhs;
-  int c = (int)(e % nrhs);
+__global__ void k_permute(int dir, const int64_t *perm, const double *in, T *tv, double *out, int64_t n, int nrhs,
+                          int nr) {
+  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (e >= n * nr) return;
+  const int64_t g = e / nr;
+  const int c = (int)(e - g * nr) + blockIdx.y * nr;
+  T *t = tv + (int64_t)blockIdx.y * n * nr + e;
   if (dir == 0)
-    tv[e] = (T)in[perm[g] + (int64_t)c * n];
-  else
-    out[perm[g] + (int64_t)c * n] = (double)tv[e];
+    *t = c < nrhs ? (T)in[perm[g] + (int64_t)c * n] : (T)0;
+  else if (c < nrhs)
+    out[perm[g] + (int64_t)c * n] = (double)*t;
 }
 
 template <typename T>
-void launch_permute(int dir, const int64_t *perm, const double *in, T *tv, double *out, int64_t n, int nrhs,
+void launch_permute(int dir, const int64_t *perm, const double *in, T *tv, double *out, int64_t n, int nrhs, int nr,
                     cudaStream_t st) {
-  int64_t tot = n * nrhs;
+  const int64_t tot = n * nr;
   if (tot == 0) return;
-  k_permute<T><<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(dir, perm, in, tv, out, n, nrhs); count_launch();
+  k_permute<T><<<dim3((unsigned)((tot + 255) / 256), (nrhs + nr - 1) / nr), 256, 0, st>>>(dir, perm, in, tv, out, n,
+                                                                                         nrhs, nr);
+  count_launch();
 }
 
 // ---------------------------------------------------------------------------
@@ -4439,18 +4231,16 @@ void launch_permute(int dir, const int64_t *perm, const double *in, T *tv, doubl
                                 cudaStream_t);                                                                \
   template void launch_dense_lu<T>(T *, int, int *, T *, cudaStream_t, int *);                                     \
   template void launch_sweep<T>(int, const FBox<T> *, int, int, T *, int, int, int, cudaStream_t, int);       \
-  template void launch_sweep_chunks<T>(int, const FBox<T> *, const int *, const int *, int, T *, int, int, int *, \
-                                       T *, const int64_t *, cudaStream_t, int);                             \
   template void launch_chol_from_lu<T>(const FBox<T> *, int, const T *, const int64_t *, const int *,            \
                                        const int64_t *, const int *, int, T *, const int64_t *, int *, cudaStream_t); \
   template void launch_chol_apply<T>(const FBox<T> *, int, const int64_t *, const int64_t *, const int *, int,     \
                                      const T *, const int64_t *, T *, int, int, int, cudaStream_t);              \
   template void launch_top<T>(int, const T *, const int64_t *, const int *, const int64_t *, const int64_t *,     \
-                             const int *, int, int, T *, int, T *, cudaStream_t, const T *);                 \
+                              const int *, int, int, T *, int64_t, int, int, T *, cudaStream_t, const T *);   \
   template void launch_top_inverse<T>(const T *, int, T *, cudaStream_t);                                     \
   template void launch_lu_batched<T>(T *, const int64_t *, int *, const int64_t *, const int *, int, cudaStream_t, \
                                      int *);                                                                  \
-  template void launch_permute<T>(int, const int64_t *, const double *, T *, double *, int64_t, int,          \
+  template void launch_permute<T>(int, const int64_t *, const double *, T *, double *, int64_t, int, int,     \
                                   cudaStream_t);
 RSS_INST(float)
 RSS_INST(double)
