@@ -24,6 +24,7 @@
 #include <type_traits>
 
 #include "internal.h"
+#include "lu_inverse.cuh"
 
 namespace rss {
 
@@ -2291,9 +2292,7 @@ __global__ void __launch_bounds__(NT) k_elim(LevelDev<T> lv, FBox<T> *boxes, con
 
 // ---------------------------------------------------------------------------
 // Elimination, shared-memory form for b small enough: the LU of X_RR is
-// formed by the whole CTA, one rank-1 update per column (warp 0 picks each
-// pivot), X_RR^{-1} = U^{-1} L^{-1} P column by column from the LU factors
-// (a thread per column), and E = X_JR X_RR^{-1},
+// formed in registers by the whole CTA (lu_inverse.cuh), and E = X_JR X_RR^{-1},
 // G = X_RR^{-1} X_RJ are produced in chunks of CH rows / columns of J as
 // shared-memory products, written coalesced.  X_RJ is kept in the scratch
 // for the Schur update.
@@ -2398,18 +2397,19 @@ template <> struct ElimChunk<float> { static constexpr int CH = 32; };
 template <> struct ElimChunk<double> { static constexpr int CH = 32; };
 
 template <typename T>
-__host__ __device__ inline size_t elim2_smem(int b, int k, int r) {
+inline size_t elim2_smem(int b, int k, int r) {
   constexpr int CH = ElimChunk<T>::CH;
   const int ldx = r | 1;
   size_t pers = (size_t)k * r * 3 + (size_t)r * (r + 1);
   size_t u1 = (size_t)b * (b + 1);
   size_t u2 = (size_t)ldx * r + (size_t)(CH + 1) * b + (size_t)(b + 1) * CH;
+  if (sizeof(T) == 4) u2 = std::max(u2, (size_t)ldx * r + (size_t)r * (r + 1));  // a copy of X_RR beside its inverse
   size_t nT = pers + (u1 > u2 ? u1 : u2);
-  return nT * sizeof(T) + (size_t)(b + 2 * r + 8) * sizeof(int) + 64;
+  return nT * sizeof(T) + (size_t)(b + 8) * sizeof(int) + 64;
 }
 
-template <typename T>
-__global__ void __launch_bounds__(NT) k_elim2(LevelDev<T> lv, FBox<T> *boxes, const int *box_list, T *scratch,
+template <typename T, int RB>
+__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (RB == 4 ? 4 : RB == 6 ? 2 : 1) : 1) k_elim2(LevelDev<T> lv, FBox<T> *boxes, const int *box_list, T *scratch,
                                               int64_t sstride, Overflow<T> ovf, int *err, int split, int C) {
   constexpr int CH = ElimChunk<T>::CH;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -2418,6 +2418,7 @@ __global__ void __launch_bounds__(NT) k_elim2(LevelDev<T> lv, FBox<T> *boxes, co
   __shared__ int s_ld_in[27];
   __shared__ int64_t s_rb[ElimChunk<T>::CH], s_cb[ElimChunk<T>::CH];
   __shared__ int s_rl[ElimChunk<T>::CH];
+  __shared__ LuInvShared<T> s_lu;
   // C CTAs per box (split mode only): CTA 0 also does the LU, X_RR^{-1} and
   // the box's records; every CTA forms its share of the chunks of J
   const int q = blockIdx.x / C, cta = blockIdx.x % C;
@@ -2436,35 +2437,47 @@ __global__ void __launch_bounds__(NT) k_elim2(LevelDev<T> lv, FBox<T> *boxes, co
   T *Xi = U0;                                       // X_RR^{-1}, column-major, ld ldx (after the LU)
   T *rawJ = Xi + (size_t)ldx * r;                   // CH rows of J x b  (al + p*(CH+1)) -> X_JR in place
   T *rawC = rawJ + (size_t)(CH + 1) * b;            // b x CH columns of J (p + al*(b+1)) -> X_RJ in place
-  const size_t u1 = (size_t)b * ldb, u2 = (size_t)ldx * r + (size_t)(CH + 1) * b + (size_t)ldb * CH;
+  const size_t u1 = (size_t)b * ldb;
+  size_t u2 = (size_t)ldx * r + (size_t)(CH + 1) * b + (size_t)ldb * CH;
+  if (sizeof(T) == 4) u2 = max(u2, (size_t)ldx * r + (size_t)r * ldl);  // the copy of X_RR
   int *sloc = reinterpret_cast<int *>(U0 + (u1 > u2 ? u1 : u2));
-  int *spiv = sloc + b;
-  int *spinv = spiv + r;
 
-  if (tid == 0) {
-    int nn = 0, acc = k;
-    for (int code = 0; code < ncode3; code++) {
+  if (warp == 0) {  // the 3^d neighbourhood, a lane per cell
+    int nb = -1, cnt = 0, aoff = 0;
+    if (lane < ncode3) {
       int dx, dy, dz;
-      decode3(code, dim, dx, dy, dz);
-      int nb = lv.cell_nbr[(int64_t)c * lv.NB + code5(dx, dy, dz, dim)];
-      s_ncell[code] = nb;
+      decode3(lane, dim, dx, dy, dz);
+      nb = lv.cell_nbr[(int64_t)c * lv.NB + code5(dx, dy, dz, dim)];
+      s_ncell[lane] = nb;
       if (nb >= 0) {
-        s_off_in[code] = lv.pair_off[(int64_t)nb * lv.NB + code5(-dx, -dy, -dz, dim)];
-        s_off_out[code] = lv.pair_off[(int64_t)c * lv.NB + code5(dx, dy, dz, dim)];
-        s_ld_in[code] = lv.cell_b[nb];
+        s_off_in[lane] = lv.pair_off[(int64_t)nb * lv.NB + code5(-dx, -dy, -dz, dim)];
+        s_off_out[lane] = lv.pair_off[(int64_t)c * lv.NB + code5(dx, dy, dz, dim)];
+        s_ld_in[lane] = lv.cell_b[nb];
+        if (lane != center && !lv.weak) {  // weak steps: J = S
+          cnt = max(lv.act_cnt[nb], 0);
+          aoff = (int)lv.cell_dof_off[nb];
+        }
       }
-      if (code == center || nb < 0 || lv.weak) continue;  // weak steps: J = S
-      int cnt = lv.act_cnt[nb];
-      if (cnt <= 0) continue;
-      s_ncode[nn] = code;
-      s_nstart[nn] = acc;
-      s_nact[nn] = (int)lv.cell_dof_off[nb];
-      acc += cnt;
-      nn++;
     }
-    s_nstart[nn] = acc;
-    s_nn = nn;
-    s_ok = (acc <= fb.njmax && cta == 0) ? claim_storage(fb, acc, ovf, err) : 1;  // acc > njmax: reported below
+    const unsigned mask = __ballot_sync(FULL, cnt > 0);
+    int incl = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(FULL, incl, o);
+      if (lane >= o) incl += t;
+    }
+    const int acc = k + __shfl_sync(FULL, incl, 31), nn = __popc(mask);
+    if (cnt > 0) {
+      const int at = __popc(mask & ((1u << lane) - 1));
+      s_ncode[at] = lane;
+      s_nstart[at] = k + incl - cnt;
+      s_nact[at] = aoff;
+    }
+    if (lane == 0) {
+      s_nstart[nn] = acc;
+      s_nn = nn;
+      s_ok = (acc <= fb.njmax && cta == 0) ? claim_storage(fb, acc, ovf, err) : 1;  // acc > njmax: reported below
+    }
   }
   for (int q = tid; q < b; q += NT) sloc[q] = fb.loc[q];
   for (int e = tid; e < k * r; e += NT) Ts[e] = fb.Tm[e];
@@ -2501,10 +2514,21 @@ __global__ void __launch_bounds__(NT) k_elim2(LevelDev<T> lv, FBox<T> *boxes, co
   // stage A_BB in (S|R) order
   const FastDiv fdb(max(b, 1)), fdr(max(r, 1)), fdk(max(k, 1));
   const T *Aii = lv.pool + s_off_in[center];
-  for (int e = tid; e < b * b; e += NT) {
-    int pp, qq;
-    fdb.divmod(e, qq, pp);
-    Ab[pp + qq * ldb] = Aii[sloc[pp] + (int64_t)sloc[qq] * b];
+  for (int e0 = tid; e0 < b * b; e0 += 8 * NT) {  // eight loads in flight a thread
+    T val[8];
+#pragma unroll
+    for (int u = 0; u < 8; u++) {
+      int pp, qq;
+      fdb.divmod(min(e0 + u * NT, b * b - 1), qq, pp);
+      val[u] = Aii[sloc[pp] + (int64_t)sloc[qq] * b];
+    }
+#pragma unroll
+    for (int u = 0; u < 8; u++) {
+      const int e = e0 + u * NT;
+      int pp, qq;
+      fdb.divmod(e, qq, pp);
+      if (e < b * b) Ab[pp + qq * ldb] = val[u];
+    }
   }
   __syncthreads();
   // X_RS = A_RS - T^T A_SS,  X_SR = A_SR - A_SS T,  then
@@ -2540,103 +2564,23 @@ __global__ void __launch_bounds__(NT) k_elim2(LevelDev<T> lv, FBox<T> *boxes, co
   }
   __syncthreads();
   if (cta == 0) {
-  // LU with partial pivoting (largest |entry|, ties to the lowest row): per
-  // column, warp 0 picks the pivot, swaps the rows and scales the column;
-  // then every warp takes rows of the rank-1 update, its lanes 32
-  // consecutive columns
-  for (int i = tid; i < r; i += NT) spiv[i] = i;
-  __syncthreads();
-  for (int j = 0; j < r; j++) {
-    if (warp == 0) {
-      T best = (T)-1;
-      int bi = r;
-      for (int i = j + lane; i < r; i += 32) {
-        T v = fabs(LU[i * ldl + j]);
-        if (v > best) {
-          best = v;
-          bi = i;
-        }
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        T ov = __shfl_xor_sync(FULL, best, o);
-        int oi = __shfl_xor_sync(FULL, bi, o);
-        if (ov > best || (ov == best && oi < bi)) {
-          best = ov;
-          bi = oi;
-        }
-      }
-      if (bi >= r) {  // NaN column: keep the diagonal, report
-        bi = j;
-        if (lane == 0) set_err(err, DERR_NUMERIC);
-      }
-      if (best == (T)0 && lane == 0) set_err(err, DERR_NUMERIC);
-      if (bi != j) {
-        for (int cc = lane; cc < r; cc += 32) {
-          T t0 = LU[j * ldl + cc];
-          LU[j * ldl + cc] = LU[bi * ldl + cc];
-          LU[bi * ldl + cc] = t0;
-        }
-        if (lane == 0) {
-          int tp = spiv[j];
-          spiv[j] = spiv[bi];
-          spiv[bi] = tp;
-        }
-      }
-      __syncwarp();
-      const T d = LU[j * ldl + j];
-      for (int i = j + 1 + lane; i < r; i += 32) LU[i * ldl + j] /= d;
-    }
-    __syncthreads();
-    for (int i = j + 1 + warp; i < r; i += NT / 32) {
-      const T l = LU[i * ldl + j];
-      for (int cc = j + 1 + lane; cc < r; cc += 32) LU[i * ldl + cc] = LU[i * ldl + cc] - l * LU[j * ldl + cc];
-    }
-    __syncthreads();
+  // LU factors and inverse of X_RR; the inverse over A_BB, which is no
+  // longer needed
+  {
+    T *xi = Xi;
+    const int ld = ldx;
+    T *Xc = rawJ;  // a copy of X_RR for the correction
+    if constexpr (sizeof(T) == 4)
+      for (int e = tid; e < r * ldl; e += NT) Xc[e] = LU[e];
+    lu_inverse<T, RB>(r, LU, ldl, s_lu, err, [&](int i, int cc, T v) { xi[i + (size_t)cc * ld] = v; });
+    if constexpr (sizeof(T) == 4) newton_inverse<RB>(r, Xc, ldl, Xi, ldx);
   }
-  for (int i = tid; i < r; i += NT) spinv[spiv[i]] = i;
   for (int e = tid; e < r * r; e += NT) {
     int qi, ri;
     fdr.divmod(e, qi, ri);
-    fb.LU[e] = LU[qi * ldl + ri];
+    fb.LU[e] = LU[s_lu.piv[qi] * ldl + ri];
   }
-  for (int i = tid; i < r; i += NT) fb.piv[i] = spiv[i];
-  __syncthreads();
-  // X_RR^{-1} = U^{-1} L^{-1} P: column cc is U^{-1} L^{-1} e_{pinv[cc]}
-  // (four partial sums per dot product to shorten the dependence chains;
-  // one thread per column measured faster than the whole CTA taking a
-  // rank-1 update per row step)
-  for (int cc = tid; cc < r; cc += NT) {
-    T *x = Xi + (size_t)cc * ldx;
-    const int i0 = spinv[cc];
-    for (int i = 0; i < r; i++) {
-      const T *Li = LU + i * ldl;
-      T s0 = (T)0, s1 = (T)0, s2 = (T)0, s3 = (T)0;
-      int l = i0;  // x[l] = 0 for l < i0
-      for (; l + 3 < i; l += 4) {
-        s0 += Li[l] * x[l];
-        s1 += Li[l + 1] * x[l + 1];
-        s2 += Li[l + 2] * x[l + 2];
-        s3 += Li[l + 3] * x[l + 3];
-      }
-      for (; l < i; l++) s0 += Li[l] * x[l];
-      x[i] = (i == i0 ? (T)1 : (T)0) - ((s0 + s1) + (s2 + s3));
-    }
-    for (int i = r - 1; i >= 0; i--) {
-      const T *Ui = LU + i * ldl;
-      T s0 = (T)0, s1 = (T)0, s2 = (T)0, s3 = (T)0;
-      int l = i + 1;
-      for (; l + 3 < r; l += 4) {
-        s0 += Ui[l] * x[l];
-        s1 += Ui[l + 1] * x[l + 1];
-        s2 += Ui[l + 2] * x[l + 2];
-        s3 += Ui[l + 3] * x[l + 3];
-      }
-      for (; l < r; l++) s0 += Ui[l] * x[l];
-      x[i] = (x[i] - ((s0 + s1) + (s2 + s3))) / Ui[i];
-    }
-  }
-  __syncthreads();
+  for (int i = tid; i < r; i += NT) fb.piv[i] = s_lu.piv[i];
   for (int e = tid; e < r * r; e += NT) {
     int qi, ri;
     fdr.divmod(e, qi, ri);
@@ -2781,16 +2725,17 @@ template int64_t elim_ws_elems<float>(int);
 template int64_t elim_ws_elems<double>(int);
 
 // E = X_JR X_RR^{-1} (nj x r) and G = X_RR^{-1} X_RJ (r x nj) for the boxes
-// of a phase eliminated by k_elim: blockIdx.x = box of the phase,
-// blockIdx.y = a 64 x 64 output tile of E (the first tiles_e) or of G.
-// X_JR (ld nj) and X_RJ (ld r) are in the box's scratch, X_RR^{-1} in the
-// factor (r x r, column-major).  Shared-memory tiles of 16 along the inner
-// dimension; each thread accumulates a 4 x 4 block.
+// of a phase whose X_JR (ld nj) and X_RJ (ld r) are in the scratch:
+// blockIdx.x = box of the phase, blockIdx.y = a 64 x 64 output tile of E (the
+// first tiles_e) or of G; X_RR^{-1} is in the factor (r x r, column-major).
+// The inner dimension is staged 64 (FP32) or 32 (FP64) at a time, one round
+// for the 2D boxes' r of 45-75 but a remainder: small phases pay one load
+// latency instead of one per 16.  Each thread accumulates a 4 x 4 block.
 template <typename T>
 __global__ void __launch_bounds__(NT) k_elim_gemm(const FBox<T> *boxes, const int *box_list, const T *scratch,
                                                   int64_t sstride, int tiles_e, int tcols_e, int tcols_g) {
-  __shared__ T As[16][64 + 1];
-  __shared__ T Bs[16][64 + 1];
+  constexpr int KC = sizeof(T) == 4 ? 64 : 32, LD = 64 + 1;
+  __shared__ T As[KC * LD], Bs[KC * LD];
   const FBox<T> &fb = boxes[box_list[blockIdx.x]];
   const int r = fb.r, nj = fb.nj;
   if (r == 0) return;
@@ -2818,21 +2763,23 @@ __global__ void __launch_bounds__(NT) k_elim_gemm(const FBox<T> *boxes, const in
   for (int x = 0; x < 4; x++)
 #pragma unroll
     for (int y = 0; y < 4; y++) acc[x][y] = (T)0;
-  for (int l0 = 0; l0 < r; l0 += 16) {
-    for (int e = tid; e < 16 * 64; e += NT) {
-      const int ii = e % 64, ll = e / 64;  // A: consecutive rows
-      As[ll][ii] = (i0 + ii < m && l0 + ll < r) ? A[(i0 + ii) + (int64_t)(l0 + ll) * lda] : (T)0;
-      const int l2 = e % 16, jj = e / 16;  // B: consecutive inner index
-      Bs[l2][jj] = (l0 + l2 < r && j0 + jj < n) ? B[(l0 + l2) + (int64_t)(j0 + jj) * ldb] : (T)0;
+  for (int l0 = 0; l0 < r; l0 += KC) {
+    const int kw = min(KC, r - l0);
+#pragma unroll 8
+    for (int e = tid; e < KC * 64; e += NT) {
+      const int ii = e & 63, ll = e >> 6;  // A: consecutive rows
+      As[ll * LD + ii] = (i0 + ii < m && ll < kw) ? A[(i0 + ii) + (int64_t)(l0 + ll) * lda] : (T)0;
+      const int l2 = e % KC, jj = e / KC;  // B: consecutive inner index
+      Bs[l2 * LD + jj] = (l2 < kw && j0 + jj < n) ? B[(l0 + l2) + (int64_t)(j0 + jj) * ldb] : (T)0;
     }
     __syncthreads();
-#pragma unroll
-    for (int u = 0; u < 16; u++) {
+#pragma unroll 4
+    for (int u = 0; u < kw; u++) {
       T av[4], bv[4];
 #pragma unroll
-      for (int x = 0; x < 4; x++) av[x] = As[u][ti + 16 * x];
+      for (int x = 0; x < 4; x++) av[x] = As[u * LD + ti + 16 * x];
 #pragma unroll
-      for (int y = 0; y < 4; y++) bv[y] = Bs[u][tj + 16 * y];
+      for (int y = 0; y < 4; y++) bv[y] = Bs[u * LD + tj + 16 * y];
 #pragma unroll
       for (int x = 0; x < 4; x++)
 #pragma unroll
@@ -2850,6 +2797,13 @@ __global__ void __launch_bounds__(NT) k_elim_gemm(const FBox<T> *boxes, const in
       if (i < m) Cp[i + (int64_t)j * ldc] = acc[x][y];
     }
   }
+}
+
+template <typename T>
+static void launch_elim_gemm(const FBox<T> *boxes, const int *box_list, int nbox, const T *scratch, int64_t sstride,
+                             int tiles, int tr, int tn, cudaStream_t st) {
+  k_elim_gemm<T><<<dim3(nbox, 2 * tiles), NT, 0, st>>>(boxes, box_list, scratch, sstride, tiles, tr, tn);
+  count_launch();
 }
 
 // X_RR = A_RR - T^T A_SR - X_RS T (Sec. 3.1) for the boxes of a phase whose
@@ -3217,21 +3171,22 @@ void launch_elim(const LevelDev<T> &lv, FBox<T> *boxes, const int *box_list, int
     for (int r = 0; r <= bmax; r++) worst = std::max(worst, elim2_smem<T>(bmax, bmax - r, r));
     // boxes of up to 128 DOFs (wider ones take the blocked LU below)
     if (worst <= (size_t)(220 << 10) && bmax <= 128) {
-      cudaFuncSetAttribute(k_elim2<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)worst);
-      k_elim2<T><<<nbox * C, NT, worst, st>>>(lv, boxes, box_list, scratch, scratch_stride, ovf, err, split, C);
+      // registers per thread of the LU: 16, 36 or 64 entries of X_RR (r <= b)
+      auto run = [&](auto kern) {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)worst);
+        kern<<<nbox * C, NT, worst, st>>>(lv, boxes, box_list, scratch, scratch_stride, ovf, err, split, C);
+      };
+      if (bmax <= 64) run(k_elim2<T, 4>);
+      else if (bmax <= 96) run(k_elim2<T, 6>);
+      else run(k_elim2<T, 8>);
       count_launch();
-      if (split) {
-        k_elim_gemm<T><<<dim3(nbox, 2 * tn * tr), NT, 0, st>>>(boxes, box_list, scratch, scratch_stride, tn * tr, tr,
-                                                                 tn);
-        count_launch();
-      }
+      if (split) launch_elim_gemm<T>(boxes, box_list, nbox, scratch, scratch_stride, tn * tr, tr, tn, st);
       return;
     }
   }
   // the global workspace sits after the X_JR / X_RJ scratch of the box
   const int64_t ws_off = scratch_stride - elim_ws_elems<T>(bmax);
-  const int tiles_e = tn * tr;  // E: nj x r
-  const int tiles_g = tr * tn;  // G: r x nj
+  const int tiles_e = tn * tr;  // E: nj x r, and as many of G: r x nj
   if (!force_general) {
     // boxes wider than k_elim2 takes: X_JR and X_RJ over up to 64 CTAs per
     // box, X_RR as tiles, the LU and X_RR^{-1} blocked in one 1024-thread CTA
@@ -3254,9 +3209,8 @@ void launch_elim(const LevelDev<T> &lv, FBox<T> *boxes, const int *box_list, int
         cudaFuncSetAttribute(k_elim_lu<T, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsm);
         k_elim_lu<T, 32><<<nbox, NLU, lsm, st>>>(lv, boxes, box_list, scratch, scratch_stride, ws_off, err);
       }
-      k_elim_gemm<T><<<dim3(nbox, tiles_e + tiles_g), NT, 0, st>>>(boxes, box_list, scratch, scratch_stride,
-                                                                    tiles_e, tr, tn);
-      count_launch(4);
+      count_launch(3);
+      launch_elim_gemm<T>(boxes, box_list, nbox, scratch, scratch_stride, tiles_e, tr, tn, st);
       return;
     }
   }
@@ -3266,9 +3220,8 @@ void launch_elim(const LevelDev<T> &lv, FBox<T> *boxes, const int *box_list, int
   const int Cg = force_general ? 1 : std::min(8, std::max(1, (300 + nbox - 1) / nbox));
   k_elim<T><<<nbox * Cg, NT, 0, st>>>(lv, boxes, box_list, scratch, scratch_stride, ws_off, ovf, err, Cg, 0);
   // E and G: tiles of 64 x 64 over nj x r (E) and r x nj (G), nj <= njmax, r <= bmax
-  k_elim_gemm<T><<<dim3(nbox, tiles_e + tiles_g), NT, 0, st>>>(boxes, box_list, scratch, scratch_stride, tiles_e,
-                                                              tr, tn);
-  count_launch(2);
+  count_launch();
+  launch_elim_gemm<T>(boxes, box_list, nbox, scratch, scratch_stride, tiles_e, tr, tn, st);
 }
 
 // ---------------------------------------------------------------------------
