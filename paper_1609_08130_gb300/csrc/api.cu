@@ -873,7 +873,7 @@ template <typename T> struct Factor : FactorBase {
   std::vector<int> h_tn;
   std::vector<int64_t> h_toff, h_loff;
   DBuf d_top, d_topLU, d_toppiv, d_tn, d_toff, d_loff;
-  DBuf d_topinv;  // one problem's U^{-1} L^{-1} of the top block (ntop <= 1024), else empty
+  DBuf d_topinv;  // U^{-1} L^{-1} of the top blocks (orders up to top_lu_limit), else empty
   mutable DBuf d_work, d_topwork;
   // Cholesky factors of the diagonal blocks for the generalized square root
   // (rss_sqrt_apply), built on its first use
@@ -2191,20 +2191,28 @@ template <typename T> static void run_factor(Factor<T> &F) {
     double fl = 0;
     for (int tn : F.h_tn) fl += 2.0 / 3.0 * (double)tn * tn * tn;
     int pi = F.prof.begin(KC_TOPLU, st, 0, 0, 0, 2.0 * (double)F.h_loff[np] * sizeof(T), fl);
-    DBuf d_panel;  // column-major copy of the current panel
-    if (np == 1) {
+    if (maxt <= top_lu_limit((int)sizeof(T))) {
+      DBuf d_moves, d_diag;
+      d_moves.alloc((size_t)top_lu_scratch_bytes(np), st, 1);
+      launch_top_lu<T>(ptr<T>(F.d_topLU), ptr<int64_t>(F.d_loff), ptr<int>(F.d_toppiv), ptr<int64_t>(F.d_toff),
+                       ptr<int>(F.d_tn), np, maxt, d_moves.p, st, ptr<int>(F.d_err));
+      check_launch("top lu");
+      // the solves multiply by U^{-1} L^{-1} instead of two triangular sweeps
+      F.d_topinv.alloc((size_t)F.h_loff[np] * sizeof(T) + 16, st);
+      d_diag.alloc((size_t)top_inverse_scratch_elems(np, maxt) * sizeof(T), st, 1);
+      F.factor_bytes += F.h_loff[np] * (int64_t)sizeof(T);
+      launch_top_inverse<T>(ptr<T>(F.d_topLU), ptr<int64_t>(F.d_loff), ptr<int>(F.d_tn), np, maxt, ptr<T>(F.d_topinv),
+                            ptr<T>(d_diag), st);
+      check_launch("top inverse");
+    } else if (np == 1) {
+      DBuf d_panel;  // column-major copy of the current panel
       d_panel.alloc((size_t)F.ntop * 32 * sizeof(T) + 32 * sizeof(int), st, 1);  // + the interchanges
       launch_dense_lu<T>(ptr<T>(F.d_topLU), F.ntop, ptr<int>(F.d_toppiv), ptr<T>(d_panel), st, ptr<int>(F.d_err));
-    } else
+      check_launch("top lu");
+    } else {
       launch_lu_batched<T>(ptr<T>(F.d_topLU), ptr<int64_t>(F.d_loff), ptr<int>(F.d_toppiv), ptr<int64_t>(F.d_toff),
                            ptr<int>(F.d_tn), np, st, ptr<int>(F.d_err));
-    check_launch("top lu");
-    if (np == 1 && F.ntop <= 1024) {
-      // the solves multiply by U^{-1} L^{-1} instead of two triangular sweeps
-      F.d_topinv.alloc((size_t)F.ntop * F.ntop * sizeof(T), st);
-      F.factor_bytes += (int64_t)F.ntop * F.ntop * sizeof(T);
-      launch_top_inverse<T>(ptr<T>(F.d_topLU), F.ntop, ptr<T>(F.d_topinv), st);
-      check_launch("top inverse");
+      check_launch("top lu");
     }
     F.prof.end(pi, st);
   }

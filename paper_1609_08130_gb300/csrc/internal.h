@@ -178,14 +178,25 @@ size_t sweep_chunk_smem(int bmax, int nr, int elem);
 void sweep_chunk_attributes();
 // Set the shared-memory attributes of every sweep kernel on the current device.
 void sweep_kernel_attributes();
-// Top blocks: mode 0 solves with the LU factors (or, for one problem with
-// Winv = U^{-1} L^{-1} and at most 4 columns, multiplies by it), mode 1
-// multiplies by the block.  launch_top_inverse forms Winv (n <= 1024).
+// Top blocks: mode 0 solves with the LU factors or, with Winv = U^{-1} L^{-1}
+// and groups of at most 4 columns, multiplies by it; mode 1 multiplies by the
+// block.
 template <typename T>
 void launch_top(int mode, const T *LU, const int64_t *loff, const int *piv, const int64_t *top, const int64_t *toff,
                 const int *tn, int nprob, int ntop_total, T *v, int64_t n, int nr, int groups, T *work,
                 cudaStream_t st, const T *Winv = nullptr);
-template <typename T> void launch_top_inverse(const T *LU, int n, T *W, cudaStream_t st);
+// Top blocks up to top_lu_limit (toplu.cu): the LU of every problem's block
+// (maxn: the largest order; scratch: top_lu_scratch_bytes) and
+// W = U^{-1} L^{-1} at the same offsets (D: top_inverse_scratch_elems of T).
+int top_lu_limit(int elem);
+int64_t top_lu_scratch_bytes(int nprob);
+int64_t top_inverse_scratch_elems(int nprob, int maxn);
+template <typename T>
+void launch_top_lu(T *LU, const int64_t *loff, int *piv, const int64_t *toff, const int *tn, int nprob, int maxn,
+                   void *scratch, cudaStream_t st, int *err);
+template <typename T>
+void launch_top_inverse(const T *LU, const int64_t *loff, const int *tn, int nprob, int maxn, T *W, T *D,
+                        cudaStream_t st);
 template <typename T>
 void launch_lu_batched(T *LU, const int64_t *loff, int *piv, const int64_t *toff, const int *tn, int nprob,
                        cudaStream_t st, int *err);

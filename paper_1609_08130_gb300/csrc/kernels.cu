@@ -3860,6 +3860,17 @@ __global__ void __launch_bounds__(1024) k_top(const T *LUall, const int64_t *lof
   for (int i = tid; i < n; i += blockDim.x) v[top[i] * nrhs + c] = y[i];
 }
 
+// The last problem whose rows start at or before row e.
+__device__ __forceinline__ int problem_of(const int64_t *toff, int nprob, int e) {
+  int lo = 0, hi = nprob - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (toff[mid] <= e) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+
 // Multiply by the top blocks, v_top = P^T L U v_top, in two launches (half 0:
 // u = U v, half 1: v = P^T L u), a warp per row over the row-major factors,
 // all problems' rows in one grid (a CTA per problem and column reading the
@@ -3870,15 +3881,10 @@ __global__ void __launch_bounds__(256) k_top_mul(int half, const T *LUall, const
                                                  int64_t vstride, T *u, int64_t wstride) {
   const int lane = threadIdx.x & 31, e = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (e >= ntot) return;
-  int lo = 0, hi = nprob - 1;  // the last problem starting at or before row e
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (toff[mid] <= e) lo = mid;
-    else hi = mid - 1;
-  }
-  const int64_t o = toff[lo];
-  const int n = (int)(toff[lo + 1] - o), i = (int)(e - o);
-  const T *row = LUall + loff[lo] + (int64_t)i * n;
+  const int p = problem_of(toff, nprob, e);
+  const int64_t o = toff[p];
+  const int n = (int)(toff[p + 1] - o), i = (int)(e - o);
+  const T *row = LUall + loff[p] + (int64_t)i * n;
   const int64_t *top = topall + o;
   v += blockIdx.y * vstride;
   u += blockIdx.y * wstride;
@@ -3907,50 +3913,6 @@ __global__ void __launch_bounds__(256) k_top_mul(int half, const T *LUall, const
 #pragma unroll
     for (int c = 0; c < NR; c++) out[c] = half == 0 ? acc[c] : acc[c] + u[e * (int64_t)NR + c];
   }
-}
-
-// W = U^{-1} L^{-1} for one top block's LU (row-major; unit lower L below
-// the diagonal, U on and above), so that the solve's D^{-1} on the top
-// block is W (P v), a matrix-vector product, instead of two triangular
-// sweeps with a barrier per row.  One warp per column k of W: z = L^{-1}
-// e_k, then U^{-1} z, each row's dot product spread over the lanes; z in
-// shared memory.  Columns are independent, so the warps never wait on one
-// another.
-constexpr int TOPINV_WARPS = 4;
-template <typename T> __global__ void __launch_bounds__(32 * TOPINV_WARPS) k_top_inverse(const T *LU, int n, T *W) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int k = blockIdx.x * TOPINV_WARPS + w;
-  if (k >= n) return;  // the whole warp: no barrier follows
-  T *z = reinterpret_cast<T *>(smem_raw) + (size_t)w * n;
-  for (int i = lane; i < n; i += 32) z[i] = i == k ? (T)1 : (T)0;
-  __syncwarp();
-  for (int i = k + 1; i < n; i++) {
-    const T *Li = LU + (int64_t)i * n;
-    T acc = (T)0;
-    for (int l = k + lane; l < i; l += 32) acc += Li[l] * z[l];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) z[i] = -acc;
-    __syncwarp();
-  }
-  for (int i = n - 1; i >= 0; i--) {
-    const T *Ui = LU + (int64_t)i * n;
-    T acc = (T)0;
-    for (int l = i + 1 + lane; l < n; l += 32) acc += Ui[l] * z[l];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) z[i] = (z[i] - acc) / Ui[i];
-    __syncwarp();
-  }
-  for (int i = lane; i < n; i += 32) W[(int64_t)i * n + k] = z[i];
-}
-
-template <typename T> void launch_top_inverse(const T *LU, int n, T *W, cudaStream_t st) {
-  if (n == 0) return;
-  k_top_inverse<T><<<(n + TOPINV_WARPS - 1) / TOPINV_WARPS, 32 * TOPINV_WARPS,
-                     (size_t)TOPINV_WARPS * n * sizeof(T), st>>>(LU, n, W);
-  count_launch();
 }
 
 // The same for one group of more than four columns (boxes too wide for the
@@ -3982,40 +3944,44 @@ __global__ void __launch_bounds__(256) k_top_mul_wide(const T *LUall, const int6
   }
 }
 
-// y = P v_top (the pivoted gather), then v_top = W y with one warp per row;
-// grid.y: groups of NR columns.
-template <typename T>
-__global__ void k_top_gather(const int *piv, const int64_t *top, int n, const T *v, int64_t vstride, int nrhs, T *y,
-                             int64_t wstride) {
+// y = P v_top (the pivoted gather), then v_top = W y with one warp per row,
+// all problems' rows in one grid; grid.y: groups of NR columns.
+template <typename T, int NR>
+__global__ void __launch_bounds__(256) k_top_gather(const int *piv, const int64_t *top, const int64_t *toff, int nprob,
+                                                    int ntot, const T *v, int64_t vstride, T *y, int64_t wstride) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n * nrhs) return;
-  const int kk = e / nrhs, c = e - kk * nrhs;
-  y[blockIdx.y * wstride + e] = v[blockIdx.y * vstride + top[piv[kk]] * nrhs + c];
+  if (e >= ntot) return;
+  const int64_t o = toff[problem_of(toff, nprob, e)];
+  const T *x = v + blockIdx.y * vstride + top[o + piv[e]] * NR;
+#pragma unroll
+  for (int c = 0; c < NR; c++) y[blockIdx.y * wstride + (int64_t)e * NR + c] = x[c];
 }
 template <typename T, int NR>
-__global__ void __launch_bounds__(256) k_top_gemv(const T *W, const int64_t *top, int n, const T *y, int64_t wstride,
-                                                  T *v, int64_t vstride) {
-  const int lane = threadIdx.x & 31;
-  const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (i >= n) return;
-  y += blockIdx.y * wstride;
+__global__ void __launch_bounds__(256) k_top_gemv(const T *Wall, const int64_t *loff, const int64_t *topall,
+                                                  const int64_t *toff, int nprob, int ntot, const T *y,
+                                                  int64_t wstride, T *v, int64_t vstride) {
+  const int lane = threadIdx.x & 31, e = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (e >= ntot) return;
+  const int p = problem_of(toff, nprob, e);
+  const int64_t o = toff[p];
+  const int n = (int)(toff[p + 1] - o);
+  y += blockIdx.y * wstride + o * NR;
   v += blockIdx.y * vstride;
-  const T *Wi = W + (int64_t)i * n;
+  const T *Wi = Wall + loff[p] + (int64_t)(e - o) * n;
   T acc[NR];
 #pragma unroll
   for (int c = 0; c < NR; c++) acc[c] = (T)0;
+#pragma unroll 4
   for (int kk = lane; kk < n; kk += 32) {
     const T w = Wi[kk];
 #pragma unroll
     for (int c = 0; c < NR; c++) acc[c] += w * y[kk * NR + c];
   }
 #pragma unroll
-  for (int c = 0; c < NR; c++)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
+  for (int c = 0; c < NR; c++) acc[c] = warp_sum(acc[c]);
   if (lane == 0)
 #pragma unroll
-    for (int c = 0; c < NR; c++) v[top[i] * NR + c] = acc[c];
+    for (int c = 0; c < NR; c++) v[topall[e] * NR + c] = acc[c];
 }
 
 template <typename T, int NR>
@@ -4024,9 +3990,9 @@ static void launch_top_nr(int mode, const T *LU, const int64_t *loff, const int 
                           int64_t wstride, const T *Winv, cudaStream_t st) {
   const dim3 rows((unsigned)((ntop + 7) / 8), groups);
   if (mode == 0) {
-    k_top_gather<T><<<dim3((unsigned)((ntop * NR + 255) / 256), groups), 256, 0, st>>>(piv, top, ntop, v, vstride, NR,
-                                                                                      work, wstride);
-    k_top_gemv<T, NR><<<rows, 256, 0, st>>>(Winv, top, ntop, work, wstride, v, vstride);
+    k_top_gather<T, NR><<<dim3((unsigned)((ntop + 255) / 256), groups), 256, 0, st>>>(piv, top, toff, nprob, ntop, v,
+                                                                                     vstride, work, wstride);
+    k_top_gemv<T, NR><<<rows, 256, 0, st>>>(Winv, loff, top, toff, nprob, ntop, work, wstride, v, vstride);
   } else {
     for (int half = 0; half < 2; half++)
       k_top_mul<T, NR><<<rows, 256, 0, st>>>(half, LU, loff, piv, top, toff, nprob, ntop, v, vstride, work, wstride);
@@ -4040,7 +4006,7 @@ void launch_top(int mode, const T *LU, const int64_t *loff, const int *piv, cons
                 cudaStream_t st, const T *Winv) {
   if (ntop_total == 0 || nprob == 0) return;
   const int64_t vs = n * nr, ws = (int64_t)2 * ntop_total * nr;
-  if (nr <= 4 && (mode == 1 || (Winv && nprob == 1))) {
+  if (nr <= 4 && (mode == 1 || Winv)) {
 #define RSS_TOP_NR(N) \
   case N: launch_top_nr<T, N>(mode, LU, loff, piv, top, toff, nprob, ntop_total, v, vs, groups, work, ws, Winv, st); break;
     switch (nr) { RSS_TOP_NR(1) RSS_TOP_NR(2) RSS_TOP_NR(3) RSS_TOP_NR(4) }
@@ -4190,7 +4156,6 @@ void launch_permute(int dir, const int64_t *perm, const double *in, T *tv, doubl
                                      const T *, const int64_t *, T *, int, int, int, cudaStream_t);              \
   template void launch_top<T>(int, const T *, const int64_t *, const int *, const int64_t *, const int64_t *,     \
                               const int *, int, int, T *, int64_t, int, int, T *, cudaStream_t, const T *);   \
-  template void launch_top_inverse<T>(const T *, int, T *, cudaStream_t);                                     \
   template void launch_lu_batched<T>(T *, const int64_t *, int *, const int64_t *, const int *, int, cudaStream_t, \
                                      int *);                                                                  \
   template void launch_permute<T>(int, const int64_t *, const double *, T *, double *, int64_t, int, int,     \
