@@ -907,9 +907,8 @@ template <typename T> struct Factor : FactorBase {
   int grid_side = 0;
   std::vector<int64_t> grid_index;  // caller order
   mutable GridOp G;
-  mutable DBuf g_gidx, g_C, g_X, g_tw;
-  mutable DBuf g_Cf, g_Xf, g_twf;  // FP32 copies for the inner GMRES products
-  mutable bool grid_ready = false, grid_f32_ready = false;
+  mutable DBuf g_gidx, g_spectrum, g_work, g_tables;
+  mutable bool grid_ready = false;
   int mv_ntile = 0;
   DBuf d_mv_ts, d_mv_te, d_mv_sb, d_mv_se;
   DBuf d_mv_split;  // the points in FP32 parts (direct summation only)
@@ -2445,33 +2444,19 @@ template <typename T> static void apply_A_impl(const Factor<T> &F, const double 
       G.kind = F.K.kind;
       G.w = F.K.w;
       G.diag = F.K.diag;
-      int64_t tot = 1;
-      for (int d = 0; d < G.dim; d++) tot *= G.L;
       if (!F.grid_index.empty()) upload(F.g_gidx, F.grid_index, F.st);  // else detected on the device
-      F.g_C.alloc(sizeof(double2) * tot, F.st);
-      F.g_X.alloc(sizeof(double2) * tot, F.st);
-      F.g_tw.alloc(sizeof(double2) * G.L, F.st);
+      size_t bs = 0, bw = 0, bt = 0;
+      grid_op_bytes(G, bs, bw, bt);
+      F.g_spectrum.alloc(bs, F.st);
+      F.g_work.alloc(bw, F.st);
+      F.g_tables.alloc(bt, F.st);
       G.gidx = ptr<int64_t>(F.g_gidx);
-      G.C = ptr<double2>(F.g_C);
-      G.X = ptr<double2>(F.g_X);
-      G.tw = ptr<double2>(F.g_tw);
+      G.spectrum = F.g_spectrum.p;
+      G.work = F.g_work.p;
+      G.tables = F.g_tables.p;
       grid_op_setup(G, F.st);
       check_launch("grid operator setup");
       F.grid_ready = true;
-    }
-    if (f32 && !F.grid_f32_ready) {
-      GridOp &G = F.G;
-      int64_t tot = 1;
-      for (int d = 0; d < G.dim; d++) tot *= G.L;
-      F.g_Cf.alloc(sizeof(float2) * tot, F.st);
-      F.g_Xf.alloc(sizeof(float2) * tot, F.st);
-      F.g_twf.alloc(sizeof(float2) * G.L, F.st);
-      G.Cf = ptr<float2>(F.g_Cf);
-      G.Xf = ptr<float2>(F.g_Xf);
-      G.twf = ptr<float2>(F.g_twf);
-      grid_op_setup_f32(G, F.st);
-      check_launch("grid operator setup (FP32)");
-      F.grid_f32_ready = true;
     }
     grid_op_apply(F.G, x, y, nrhs, F.st, f32);
   } else if (f32) {

@@ -226,23 +226,21 @@ void launch_matvec_f32(int dim, const KernelParams &K, const double *wdof, const
                        double *yout, int64_t n, int nrhs, int ntile, const int64_t *tstart, const int64_t *tend,
                        const int64_t *sbeg, const int64_t *send, const void *split, cudaStream_t st);
 
-// FP64 operator x -> A x for points on an s^d grid of cell centres, by FFT
-// convolution on the circulant of side L = 2s (refine.cu).
+// Operator x -> A x for points on an s^d grid of cell centres, by FFT
+// convolution on the circulant of side L = 2s (refine.cu), in FP64 or (f32) with
+// the transforms in FP32.  The caller allocates the three buffers
+// (grid_op_bytes, which also fixes `pairs`) before grid_op_setup.
 struct GridOp {
   int dim = 0, s = 0, L = 0, logL = 0;
   int64_t n = 0;
   double h = 0, w = 0, diag = 1;
   int kind = 0;
+  int pairs = 1;                  // pairs of columns transformed at once
   const int64_t *gidx = nullptr;  // grid linear index of each point (caller order)
-  double2 *C = nullptr;           // spectrum of the embedded kernel
-  double2 *X = nullptr;           // work
-  double2 *tw = nullptr;          // twiddles
-  float2 *Cf = nullptr, *Xf = nullptr, *twf = nullptr;  // the same in FP32 (inner products of GMRES-IR)
+  void *spectrum = nullptr, *work = nullptr, *tables = nullptr;
 };
+void grid_op_bytes(GridOp &G, size_t &spectrum, size_t &work, size_t &tables);
 void grid_op_setup(GridOp &G, cudaStream_t st);
-// Cf and twf rounded from C and tw (after grid_op_setup; Cf, Xf, twf allocated by the caller)
-void grid_op_setup_f32(GridOp &G, cudaStream_t st);
-// y = A x for nrhs columns; f32: the transforms in FP32 (y still FP64)
 void grid_op_apply(const GridOp &G, const double *x, double *y, int nrhs, cudaStream_t st, bool f32);
 void multidot(const double *V, int64_t vstride, int nv, const double *w, int64_t n, int nrhs, double *part,
               double *out, cudaStream_t st);

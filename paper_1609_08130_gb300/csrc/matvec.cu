@@ -11,11 +11,8 @@
 //     rest), so differences of the first two parts are exact and the distance
 //     keeps 48 bits however near the points are;
 //   - r^2 = sum of squares in pairs (df.cuh);
-//   - log r^2 by Tang's table-driven method (ACM Trans. Math. Softw. 16(4),
-//     1990): r^2 = 2^e m, t = m / c - 1 with 1/c from a 128-entry table,
-//     |t| < 2^-7.9, log = e ln 2 + log c + log(1 + t), the leading terms as
-//     pairs, the cubic and higher ones in FP32 (below 2^-24 of the rest);
-//     1 / r by an FP32 seed and one Newton step in pairs;
+//   - log r^2 table-driven (log_df.cuh), 1 / r by an FP32 seed and one Newton
+//     step in pairs;
 //   - products and sums in pairs, flushed into FP64 every 256 terms.
 // The weight, the kernel's constant and the diagonal term are FP64.  The
 // columns are scaled by powers of two per tile of 256 sources; a tile with
@@ -25,6 +22,7 @@
 
 #include "df.cuh"
 #include "internal.h"
+#include "log_df.cuh"
 
 namespace rss {
 
@@ -54,11 +52,14 @@ __device__ __forceinline__ int extent_exp(unsigned long long mx) {
 }
 
 // part p (of 3) of coordinate d at out[(3 d + p) n + i], scaled by 2^(40 - E):
-// multiples of 2^17, then of 2^-6, then the rest
-__global__ void k_mv_split(const double *xt, int64_t n, int dim, const unsigned long long *mx, float *out) {
+// multiples of 2^17, then of 2^-6, then the rest; the first CTA also fills the
+// logarithm's tables
+__global__ void __launch_bounds__(256) k_mv_split(const double *xt, int64_t n, int dim, const unsigned long long *mx,
+                                                  LogTables *T, float *out) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
   const int sh = MV_SHIFT - extent_exp(*mx);
+  if (blockIdx.x == 0) log_tables_entry(T, threadIdx.x, 2 * sh);
+  if (i >= n) return;
   for (int d = 0; d < dim; d++) {
     const double x = xt[i * dim + d] * pow2(sh / 2) * pow2(sh - sh / 2);
     const double h = rint(x * 0x1p-17) * 0x1p17, l = rint((x - h) * 0x1p6) * 0x1p-6;
@@ -98,32 +99,6 @@ __global__ void __launch_bounds__(MVT) k_mv_x(const int64_t *perm, const double 
   }
 }
 
-// log of r2 > 0 in pairs (see the head of the file); lt: 1/c, log c (pair);
-// et: e ln 2 (pair) by the biased exponent
-__device__ __forceinline__ Df log_df(Df r2, const float4 *lt, const float2 *et) {
-  const unsigned u = __float_as_uint(r2.h);
-  const float4 T = lt[(u >> 16) & 127];
-  const float2 E = et[u >> 23];
-  const float mh = __uint_as_float((u & 0x7fffffu) | 0x3f800000u);
-  const float ml = r2.l * __uint_as_float(0x7f000000u - (u & 0x7f800000u));
-  const float p = __fmul_rn(mh, T.x), pe = __fmaf_rn(mh, T.x, -p);
-  const float th = __fadd_rn(p, -1.f);  // exact
-  const float tl = __fmaf_rn(ml, T.x, pe);
-  const float sq = __fmul_rn(th, th), se = __fmaf_rn(th, th, -sq);
-  float pol = __fmaf_rn(th, -1.f / 6.f, 0.2f);
-  pol = __fmaf_rn(th, pol, -0.25f);
-  pol = __fmaf_rn(th, pol, 1.f / 3.f);
-  float lo = __fmaf_rn(-0.5f, se, __fmul_rn(__fmul_rn(sq, th), pol));
-  // tl's share: tl (1 - th + th^2 - th^3 - tl / 2)
-  const float g = __fmaf_rn(0.5f, tl, __fmaf_rn(sq, th, __fmaf_rn(-th, th, th)));
-  lo = __fadd_rn(lo, __fmaf_rn(-g, tl, tl));
-  const Df ab = quick_two_sum(th, -0.5f * sq);
-  const Df uv = two_sum(E.x, T.y);
-  const Df w = two_sum(uv.h, ab.h);
-  lo = __fadd_rn(__fadd_rn(lo, __fadd_rn(E.y, T.z)), __fadd_rn(__fadd_rn(uv.l, ab.l), w.l));
-  return quick_two_sum(w.h, lo);
-}
-
 // One CTA: 256 / parts targets of one tile, `parts` threads per target, each
 // taking every parts-th source; grid.y: groups of NC columns.  parts = 4 or
 // 16: enough CTAs for every SM down to a few hundred targets (79 CTAs of 256
@@ -151,15 +126,9 @@ __global__ void __launch_bounds__(MVT, NC == 8 ? 2 : 3)
   const int cb = col0 + blockIdx.y * NC;
   const int sh = MV_SHIFT - extent_exp(*mx);
   if (KIND == 0) {
-    if (tid < 128) {
-      const double c = 1.0 + (double)(2 * tid + 1) * (1.0 / 256.0);
-      const double ic12 = rint(4096.0 / c) * (1.0 / 4096.0), lc = -log(ic12);
-      const float h = (float)lc;
-      s_lt[tid] = make_float4((float)ic12, h, (float)(lc - (double)h), 0.f);
-    }
-    const double ev = (double)(tid - 127 - 2 * sh) * 0.69314718055994530942;
-    const float h = (float)ev;
-    s_et[tid] = make_float2(h, (float)(ev - (double)h));
+    const LogTables *T = reinterpret_cast<const LogTables *>(mx + 2);
+    if (tid < 128) s_lt[tid] = T->lt[tid];
+    s_et[tid] = T->et[tid];
   }
   float xi[3 * DIM];
 #pragma unroll
@@ -355,7 +324,9 @@ int mv_parts(int ntile, int groups) { return (int64_t)ntile * groups * 4 >= 1200
 
 }  // namespace
 
-int64_t matvec_split_bytes(int64_t n, int dim) { return 16 + (int64_t)sizeof(float) * 3 * dim * n; }
+// extent (16 bytes), the logarithm's tables, the parts
+constexpr int64_t SPLIT_HEAD = 16 + (int64_t)sizeof(LogTables);
+int64_t matvec_split_bytes(int64_t n, int dim) { return SPLIT_HEAD + (int64_t)sizeof(float) * 3 * dim * n; }
 int64_t matvec_x_bytes(int64_t n, int nrhs, int ntile) {
   return (int64_t)nrhs * (n * (int64_t)sizeof(float2) + ntile * (int64_t)sizeof(int));
 }
@@ -363,11 +334,11 @@ int64_t matvec_x_bytes(int64_t n, int nrhs, int ntile) {
 void matvec_split(const double *x_tree, int64_t n, int dim, void *split, cudaStream_t st) {
   if (n == 0) return;
   unsigned long long *mx = static_cast<unsigned long long *>(split);
-  float *cs = reinterpret_cast<float *>(static_cast<char *>(split) + 16);
+  float *cs = reinterpret_cast<float *>(static_cast<char *>(split) + SPLIT_HEAD);
   cudaMemsetAsync(mx, 0, 16, st);
   const int64_t cnt = n * dim;
   k_mv_extent<<<(unsigned)std::min<int64_t>((cnt + 1023) / 1024, 608), 256, 0, st>>>(x_tree, cnt, mx);
-  k_mv_split<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(x_tree, n, dim, mx, cs);
+  k_mv_split<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(x_tree, n, dim, mx, reinterpret_cast<LogTables *>(mx + 2), cs);
   count_launch(2);
 }
 
@@ -388,7 +359,7 @@ void launch_matvec(const double *x_tree, int dim, const KernelParams &K, const d
                    cudaStream_t st) {
   if (n == 0 || ntile == 0 || nrhs == 0) return;
   const unsigned long long *mx = static_cast<const unsigned long long *>(split);
-  const float *cs = reinterpret_cast<const float *>(static_cast<const char *>(split) + 16);
+  const float *cs = reinterpret_cast<const float *>(static_cast<const char *>(split) + SPLIT_HEAD);
   float2 *xs = static_cast<float2 *>(xbuf);
   int *xk = reinterpret_cast<int *>(xs + (int64_t)nrhs * n);
   k_mv_x<<<dim3((unsigned)ntile, nrhs), MVT, 0, st>>>(perm, xin, n, nrhs, tstart, tend, xs, xk);
@@ -440,7 +411,7 @@ void launch_matvec_f32(int dim, const KernelParams &K, const double *wdof, const
                        const int64_t *sbeg, const int64_t *send, const void *split, cudaStream_t st) {
   if (n == 0 || ntile == 0 || nrhs == 0) return;
   const unsigned long long *mx = static_cast<const unsigned long long *>(split);
-  const float *cs = reinterpret_cast<const float *>(static_cast<const char *>(split) + 16);
+  const float *cs = reinterpret_cast<const float *>(static_cast<const char *>(split) + SPLIT_HEAD);
   for (int c = 0; c < nrhs;) {
     const int left = nrhs - c;
 #define MV(D, N) launch_mv_f32<D, N>(cs, mx, K, wdof, perm, xin, yout, n, c, nrhs, ntile, tstart, tend, sbeg, send, st)
