@@ -25,6 +25,7 @@
 //      counts;
 //   5. within a leaf shallower than 20, the points are put back in original
 //      order (a rank sort of at most leaf_size indices).
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <utility>
@@ -154,6 +155,74 @@ __global__ void __launch_bounds__(1024) k_scan_excl(U *a, int64_t len, U *total)
     __syncthreads();
   }
   if (total && tid == 0) *total = s_carry;
+}
+
+// The same by a cluster of eight blocks: each takes an eighth of 131072
+// consecutive counts at a time (16 per thread), reads the lower blocks' sums
+// from their shared memory and keeps the carry.  One block is a chain of
+// 8192-count rounds (182 us for 262144 counts, 15 us here).
+constexpr int SCAN_CTAS = 8;
+template <typename U>
+__global__ void __cluster_dims__(SCAN_CTAS, 1, 1) __launch_bounds__(1024) k_scan_cluster(U *a, int64_t len, U *total) {
+  constexpr int IT = 16;
+  __shared__ U wsum[32];
+  __shared__ U s_sum[2];
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, rank = (int)cl.block_rank();
+  U carry = 0;
+  int buf = 0;
+  for (int64_t b0 = 0; b0 < len; b0 += (int64_t)SCAN_CTAS * 1024 * IT, buf ^= 1) {
+    const int64_t i0 = b0 + ((int64_t)rank * 1024 + tid) * IT;
+    U v[IT], sum = 0;
+#pragma unroll
+    for (int u = 0; u < IT; u++) {
+      v[u] = i0 + u < len ? a[i0 + u] : (U)0;
+      sum += v[u];
+    }
+    U x = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const U y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) wsum[warp] = x;
+    __syncthreads();
+    if (warp == 0) {
+      U w = wsum[lane];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const U y = __shfl_up_sync(0xffffffffu, w, o);
+        if (lane >= o) w += y;
+      }
+      wsum[lane] = w;  // inclusive over warps
+      if (lane == 31) s_sum[buf] = w;
+    }
+    cl.sync();  // every block's sum of this round (the other buffer is the next round's)
+    U before = 0, all = 0;
+#pragma unroll
+    for (int c = 0; c < SCAN_CTAS; c++) {
+      const U t = *cl.map_shared_rank(&s_sum[buf], c);
+      if (c < rank) before += t;
+      all += t;
+    }
+    U run = carry + before + x - sum + (warp > 0 ? wsum[warp - 1] : (U)0);
+#pragma unroll
+    for (int u = 0; u < IT; u++) {
+      if (i0 + u < len) a[i0 + u] = run;
+      run += v[u];
+    }
+    carry += all;
+    __syncthreads();  // wsum is written again
+  }
+  cl.sync();  // no block leaves while another reads its sums
+  if (total && rank == 0 && tid == 0) *total = carry;
+}
+
+template <typename U> void scan_excl(U *a, int64_t len, U *total, cudaStream_t st) {
+  if (len <= 8192) k_scan_excl<U><<<1, 1024, 0, st>>>(a, len, total);
+  else k_scan_cluster<U><<<SCAN_CTAS, 1024, 0, st>>>(a, len, total);
+  count_launch();
 }
 
 // Radix sort pass, part 2: stable scatter.  Each block walks its tile in
@@ -527,14 +596,14 @@ void tree_gpu_sort(TreeGpu &T, void *scratch, cudaStream_t st) {
   const int bits = dim * MAXD + T.prob_bits;
   for (int sh = 0; sh < bits; sh += 8) {
     k_rs_hist<<<(unsigned)T.nblk, RS_T, 0, st>>>(T.k0, n, sh, T.hist, (int)T.nblk); count_launch();
-    k_scan_excl<uint32_t><<<1, 1024, 0, st>>>(T.hist, 256 * T.nblk, nullptr); count_launch();
+    scan_excl<uint32_t>(T.hist, 256 * T.nblk, nullptr, st);
     k_rs_scatter<<<(unsigned)T.nblk, RS_T, 0, st>>>(T.k0, T.i0, T.k1, T.i1, n, sh, T.hist, (int)T.nblk);
     count_launch();
     std::swap(T.k0, T.k1);
     std::swap(T.i0, T.i1);
   }
   k_tree_depths<<<nb256(n), 256, 0, st>>>(T.k0, n, dim, T.leaf, T.Lp, T.nd); count_launch();
-  k_scan_excl<uint32_t><<<1, 1024, 0, st>>>(T.nd, n, T.total); count_launch();
+  scan_excl<uint32_t>(T.nd, n, T.total, st);
 }
 
 void tree_gpu_nodes(const TreeGpu &T, int *depth, int *parent, int *coord, int64_t *start, int64_t *count,
@@ -612,7 +681,7 @@ void level_gpu_runs(const uint64_t *dk, int64_t na, uint32_t *flag, uint32_t *cp
   if (na == 0) return;
   k_lv_runs<<<nb256(na), 256, 0, st>>>(dk, na, flag); count_launch();
   cudaMemcpyAsync(cpos, flag, sizeof(uint32_t) * (size_t)na, cudaMemcpyDeviceToDevice, st);
-  k_scan_excl<uint32_t><<<1, 1024, 0, st>>>(cpos, na, ncell); count_launch();
+  scan_excl<uint32_t>(cpos, na, ncell, st);
 }
 
 int64_t sort_pairs_hist_bytes(int64_t n) { return 4 * 256 * ((n + RS_TILE - 1) / RS_TILE) + 16; }
@@ -625,7 +694,7 @@ void sort_pairs_u64(uint64_t *k0, int64_t *v0, uint64_t *k1, int64_t *v1, uint32
   int64_t *va = v0, *vb = v1;
   for (int sh = 0; sh < bits; sh += 8) {
     k_rs_hist<<<(unsigned)nblk, RS_T, 0, st>>>(ka, n, sh, hist, nblk); count_launch();
-    k_scan_excl<uint32_t><<<1, 1024, 0, st>>>(hist, 256 * (int64_t)nblk, nullptr); count_launch();
+    scan_excl<uint32_t>(hist, 256 * (int64_t)nblk, nullptr, st);
     k_rs_scatter<<<(unsigned)nblk, RS_T, 0, st>>>(ka, va, kb, vb, n, sh, hist, nblk); count_launch();
     std::swap(ka, kb);
     std::swap(va, vb);
@@ -648,7 +717,7 @@ void level_gpu_tables(const LevelGpu &L, cudaStream_t st) {
   k_lv_nbrs<<<nb256(len), 256, 0, st>>>(L.ncell, L.dim, L.NB, L.side, L.grid, L.cell_key, L.cell_coord, L.cell_b,
                                         L.cell_nbr, L.psz);
   count_launch();
-  k_scan_excl<unsigned long long><<<1, 1024, 0, st>>>(L.psz, len, L.pool_total); count_launch();
+  scan_excl<unsigned long long>(L.psz, len, L.pool_total, st);
   k_lv_pairoff<<<nb256(len), 256, 0, st>>>(len, L.cell_nbr, L.psz, L.pair_off); count_launch();
   if (L.nbox > 0) {
     k_lv_boxes<<<nb256(L.nbox), 256, 0, st>>>(L.nbox, L.node_coord, L.dim, L.side, L.NB, L.grid, L.cell_key, L.ncell,
@@ -661,7 +730,7 @@ void level_gpu_next_active(int ncell, const int64_t *cell_dof_off, const int64_t
                            const int *act_idx, uint32_t *aoff, uint32_t *total, int64_t *next, cudaStream_t st) {
   if (ncell == 0) return;
   cudaMemcpyAsync(aoff, act_cnt, sizeof(uint32_t) * (size_t)ncell, cudaMemcpyDeviceToDevice, st);
-  k_scan_excl<uint32_t><<<1, 1024, 0, st>>>(aoff, ncell, total); count_launch();
+  scan_excl<uint32_t>(aoff, ncell, total, st);
   k_lv_compact<<<(unsigned)(((int64_t)ncell * 32 + 255) / 256), 256, 0, st>>>(ncell, cell_dof_off, cell_dofs, act_cnt,
                                                                             act_idx, aoff, next);
   count_launch();
