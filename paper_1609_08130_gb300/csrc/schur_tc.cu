@@ -7,8 +7,9 @@
 // pair blocks of the level (one dense block per pair of cells at Chebyshev
 // distance <= 2), so the product is scattered into them.
 //
-// One CTA of 256 threads (two warpgroups) per (box, 128 rows of J): the E
-// rows are staged in shared memory, then for every 64 columns of J the X_RJ
+// One CTA of 256 threads (two warpgroups) per (box, 128 rows of J, share of the
+// columns of J): the E rows are staged in shared memory, then for every 64
+// columns of its share the X_RJ
 // columns are staged, the tile E X_RJ is accumulated in tensor memory
 // (M = 128, N = 64, K = 8 per instruction) and every warp reads 32 rows x 32
 // columns of it back (warp w: rows 32 (w mod 4) .., columns 32 (w / 4) ..)
@@ -16,6 +17,8 @@
 // lets four CTAs share an SM, so many scatter loads are in flight.  FP32 accuracy is kept by splitting
 // each operand into a TF32 head and an FP32 remainder: three TF32 products
 // (head x head, head x remainder, remainder x head) per K step.
+#include <algorithm>
+
 #include "internal.h"
 #include "tc.cuh"
 
@@ -45,7 +48,7 @@ __global__ void __launch_bounds__(NTC) k_schur_tc(LevelDev<float> lv, const FBox
   const int a0 = (blockIdx.x % row_tiles) * TM;
   const FBox<float> &fb = boxes[box_list[bi]];
   const int nj = fb.nj, r = fb.r, dim = lv.dim;
-  if (r == 0 || a0 >= nj) return;
+  if (r == 0 || a0 >= nj || (int)blockIdx.y * TN >= nj) return;
   unsigned char *opA_hi = sm, *opA_lo = sm + SchurTcSmem::A_BYTES;
   unsigned char *opB_hi = sm + 2 * SchurTcSmem::A_BYTES, *opB_lo = opB_hi + SchurTcSmem::B_BYTES;
   int64_t *s_po = reinterpret_cast<int64_t *>(sm + SchurTcSmem::OPS);
@@ -93,7 +96,8 @@ __global__ void __launch_bounds__(NTC) k_schur_tc(LevelDev<float> lv, const FBox
   const int nkc = (r + KC - 1) / KC;
   uint32_t phase = 0;
   bool ok = true;
-  for (int c0 = 0; c0 < nj && ok; c0 += TN) {
+  bool first = true;
+  for (int c0 = blockIdx.y * TN; c0 < nj && ok; c0 += TN * gridDim.y) {
     if (tid < TN) {
       const int cc = c0 + tid;
       s_cc[tid] = cc < nj ? fb.Jnb[cc] : 0;
@@ -103,7 +107,7 @@ __global__ void __launch_bounds__(NTC) k_schur_tc(LevelDev<float> lv, const FBox
       const int kw = min(KC, r - kc * KC);       // K of this chunk
       const int kp = (kw + 7) & ~7;              // padded to the MMA's K = 8
       // E rows a0.. (column-major, ld nj): staged when the chunk changes
-      if (c0 == 0 || nkc > 1) {
+      if (first || nkc > 1) {
         const int ra = a0 + (tid & (TM - 1));  // rows over the first 128 threads, again for the next
         const bool ra_ok = ra < nj;
         for (int q = tid / TM; q < kp / 4; q += NTC / TM) {
@@ -119,6 +123,7 @@ __global__ void __launch_bounds__(NTC) k_schur_tc(LevelDev<float> lv, const FBox
           *reinterpret_cast<float4 *>(opA_lo + o) = make_float4(lv4[0], lv4[1], lv4[2], lv4[3]);
         }
       }
+      first = false;
       // X_RJ columns c0.. (column-major, ld r): (column, 4 consecutive k)
       // units, column fastest so the shared-memory stores do not conflict
       const int units = TN * (kp / 4);
@@ -212,7 +217,13 @@ void launch_schur_tc(const LevelDev<float> &lv, const FBox<float> *boxes, const 
   if (cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone)
     cudaFuncSetAttribute(k_schur_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SchurTcSmem::TOTAL);
   const int64_t grid = (int64_t)nbox * rt;
-  k_schur_tc<<<(unsigned)grid, NTC, SchurTcSmem::TOTAL, st>>>(lv, boxes, box_list, rt, scratch, scratch_stride, err);
+  // the columns of J shared by enough CTAs for two rounds of the chip at four
+  // CTAs per SM: a phase of 9 boxes ran 45 CTAs, each through 9 column tiles
+  // one after another (200 us; 30 us over column tiles)
+  const int tiles = (njmax + TN - 1) / TN;
+  const int shares = (int)std::min<int64_t>(tiles, std::max<int64_t>(1, (1216 + grid - 1) / grid));
+  k_schur_tc<<<dim3((unsigned)grid, shares), NTC, SchurTcSmem::TOTAL, st>>>(lv, boxes, box_list, rt, scratch,
+                                                                       scratch_stride, err);
   count_launch();
 }
 
