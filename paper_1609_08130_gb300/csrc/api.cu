@@ -1974,7 +1974,7 @@ template <typename T> static void run_factor(Factor<T> &F) {
       while (kid_ctas > 1 && (double)id_stride * sizeof(T) * mp * kid_ctas > 8e9) kid_ctas /= 2;
     }
     if (!id_smem) grow(gid, (size_t)id_stride * sizeof(T) * std::max(maxphase, 1) * kid_ctas, st, 1);
-    int64_t el_stride = 2 * (int64_t)njmax_lvl * H.bmax + 32 + elim_ws_elems<T>(H.bmax);
+    int64_t el_stride = (int64_t)njmax_lvl * H.bmax + 32 + elim_ws_elems<T>(H.bmax);
     grow(gel, (size_t)el_stride * sizeof(T) * std::max(maxphase, 1), st, 1);
     // the multi-CTA ID's triangle slots (8 CTAs per box of the largest
     // phase, 16 for boxes wider than 256) and tree-node counters

@@ -12,7 +12,7 @@
 //              greedy column-pivoted QR of the triangle;
 //   k_elim   : the operators U_T, L_T (Sec. 3.1) and the elimination of the
 //              redundant DOFs: LU of X_RR, E = X_JR X_RR^{-1},
-//              G = X_RR^{-1} X_RJ (Sec. 2.1, Eq. 3.4);
+//              G = X_RR^{-1} X_RJ = E^T (Sec. 2.1, Eq. 3.4);
 //   k_schur  : X_JJ -= E G scattered into the pair blocks of the level.
 // k_assemble builds the pair blocks of a level (Corollary 3.2: entries not
 // reached by any Schur update are kernel entries) and the top block.
@@ -2060,8 +2060,8 @@ __global__ void __launch_bounds__(NT) k_elim(LevelDev<T> lv, FBox<T> *boxes, con
   __shared__ int s_ld_in[27];
   __shared__ int s_pivrow, s_ok;
 
-  // C CTAs per box: every CTA forms its share of the rows of X_JR and columns
-  // of X_RJ; CTA 0 also forms the S columns of X_RJ (the X_RS its LU needs)
+  // C CTAs per box: every CTA forms its share of the columns of
+  // X_RJ; CTA 0 also forms the S columns of X_RJ (the X_RS its LU needs)
   // and, unless form_only (X_RR, its LU and inverse then follow in
   // k_elim_xrr and k_elim_lu), the LU, X_RR^{-1} and the box's records
   const int q = blockIdx.x / C, cta = blockIdx.x % C;
@@ -2149,34 +2149,12 @@ __global__ void __launch_bounds__(NT) k_elim(LevelDev<T> lv, FBox<T> *boxes, con
     }
   };
 
-  T *Ep = scratch + (int64_t)q * sstride;  // X_JR, nj x r col-major (ld nj)
-  T *Gp = Ep + (int64_t)nj * r;                      // X_RJ, r x nj col-major (ld r)
+  T *Gp = scratch + (int64_t)q * sstride;  // X_RJ, r x nj col-major (ld r)
   const T *pool = lv.pool;
   const T *Aii = pool + s_off_in[center];            // block (c, c), ld b
 
-  // X_JR = A_JR - A_JS T   (L_T applied from the right)
-  for (int a = cta * NT + tid; a < nj; a += C * NT) {
-    int code, la;
-    jinfo(a, code, la);
-    const T *Ab = pool + s_off_in[code];
-    int64_t ld = s_ld_in[code];
-    const T *row = Ab + la;
-    for (int r0 = 0; r0 < r; r0 += 8) {
-      T acc[8];
-#pragma unroll
-      for (int u = 0; u < 8; u++) acc[u] = (r0 + u < r) ? row[(int64_t)sloc[k + r0 + u] * ld] : (T)0;
-      for (int s = 0; s < k; s++) {
-        T as = row[(int64_t)sloc[s] * ld];
-#pragma unroll
-        for (int u = 0; u < 8; u++)
-          if (r0 + u < r) acc[u] -= as * Ts[s + (int64_t)(r0 + u) * k];
-      }
-#pragma unroll
-      for (int u = 0; u < 8; u++)
-        if (r0 + u < r) Ep[a + (int64_t)(r0 + u) * nj] = acc[u];
-    }
-  }
-  // X_RJ = A_RJ - T^T A_SJ  (U_T applied from the left); one warp per column:
+  // X_RJ = A_RJ - T^T A_SJ  (U_T applied from the left; X_JR is its transpose,
+  // see k_elim2); one warp per column:
   // the S columns by CTA 0, the others shared by all CTAs
   auto xrj_col = [&](int a) {
     int code, la;
@@ -2261,8 +2239,8 @@ __global__ void __launch_bounds__(NT) k_elim(LevelDev<T> lv, FBox<T> *boxes, con
     }
     __syncthreads();
   }
-  // E = X_JR X_RR^{-1} and G = X_RR^{-1} X_RJ follow in k_elim_gemm, over
-  // every box of the phase at once, from X_JR, X_RJ (scratch) and X_RR^{-1}
+  // E = X_JR X_RR^{-1} and G = E^T follow in k_elim_gemm, over every box of
+  // the phase at once, from X_RJ (scratch) and X_RR^{-1}
   for (int e = tid; e < r * r; e += NT) fb.LU[e] = LU[(e / r) * ldl + (e % r)];
   for (int i = tid; i < r; i += NT) fb.piv[i] = spiv[i];
   // X_RR^{-1} = U^{-1} L^{-1} P, one column per thread (column piv[i] is
@@ -2400,9 +2378,9 @@ template <typename T>
 inline size_t elim2_smem(int b, int k, int r) {
   constexpr int CH = ElimChunk<T>::CH;
   const int ldx = r | 1;
-  size_t pers = (size_t)k * r * 3 + (size_t)r * (r + 1);
+  size_t pers = (size_t)k * r * 2 + (size_t)r * (r + 1);
   size_t u1 = (size_t)b * (b + 1);
-  size_t u2 = (size_t)ldx * r + (size_t)(CH + 1) * b + (size_t)(b + 1) * CH;
+  size_t u2 = (size_t)ldx * r + (size_t)(CH + 1) * (b + r);
   if (sizeof(T) == 4) u2 = std::max(u2, (size_t)ldx * r + (size_t)r * (r + 1));  // a copy of X_RR beside its inverse
   size_t nT = pers + (u1 > u2 ? u1 : u2);
   return nT * sizeof(T) + (size_t)(b + 8) * sizeof(int) + 64;
@@ -2412,11 +2390,15 @@ template <typename T, int RB>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (RB == 4 ? 4 : RB == 6 ? 2 : 1) : 1) k_elim2(LevelDev<T> lv, FBox<T> *boxes, const int *box_list, T *scratch,
                                               int64_t sstride, Overflow<T> ovf, int *err, int split, int C) {
   constexpr int CH = ElimChunk<T>::CH;
+  // The matrix is symmetric (both kernels are), so X_RJ = X_JR^T and
+  // G = X_RR^{-1} X_RJ = E^T up to rounding: only X_JR and E are formed and
+  // their transposes written, half the loads and products of a chunk (FP32
+  // elimination of the 512^2 grid 4.77 -> 3.76 ms).
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int s_ncode[27], s_ncell[27], s_nstart[28], s_nact[27], s_nn, s_ok;
-  __shared__ int64_t s_off_in[27], s_off_out[27];
+  __shared__ int64_t s_off_in[27];
   __shared__ int s_ld_in[27];
-  __shared__ int64_t s_rb[ElimChunk<T>::CH], s_cb[ElimChunk<T>::CH];
+  __shared__ int64_t s_rb[ElimChunk<T>::CH];
   __shared__ int s_rl[ElimChunk<T>::CH];
   __shared__ LuInvShared<T> s_lu;
   // C CTAs per box (split mode only): CTA 0 also does the LU, X_RR^{-1} and
@@ -2429,16 +2411,15 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (RB == 4 ? 4 : RB == 6 ? 
   const int center = code3(0, 0, 0, dim);
   const int ldx = r | 1, ldl = r + 1, ldb = b + 1;
   T *Ts = reinterpret_cast<T *>(smem_raw);          // k x r  (s + ri*k)
-  T *XRS = Ts + (size_t)k * r;                      // r x k  (ri + s*r)
-  T *XSR = XRS + (size_t)k * r;                     // k x r  (s + ri*k)
+  T *XSR = Ts + (size_t)k * r;                      // k x r  (s + ri*k); X_RS is its transpose
   T *LU = XSR + (size_t)k * r;                      // r x r row-major, ld r+1
   T *U0 = LU + (size_t)r * ldl;                     // union region
   T *Ab = U0;                                       // A_BB in (S|R) order, column-major, ld b+1
   T *Xi = U0;                                       // X_RR^{-1}, column-major, ld ldx (after the LU)
   T *rawJ = Xi + (size_t)ldx * r;                   // CH rows of J x b  (al + p*(CH+1)) -> X_JR in place
-  T *rawC = rawJ + (size_t)(CH + 1) * b;            // b x CH columns of J (p + al*(b+1)) -> X_RJ in place
+  T *ec = rawJ + (size_t)(CH + 1) * b;              // the chunk of E (al + ri*(CH+1))
   const size_t u1 = (size_t)b * ldb;
-  size_t u2 = (size_t)ldx * r + (size_t)(CH + 1) * b + (size_t)ldb * CH;
+  size_t u2 = (size_t)ldx * r + (size_t)(CH + 1) * (b + r);
   if (sizeof(T) == 4) u2 = max(u2, (size_t)ldx * r + (size_t)r * ldl);  // the copy of X_RR
   int *sloc = reinterpret_cast<int *>(U0 + (u1 > u2 ? u1 : u2));
 
@@ -2451,7 +2432,6 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (RB == 4 ? 4 : RB == 6 ? 
       s_ncell[lane] = nb;
       if (nb >= 0) {
         s_off_in[lane] = lv.pair_off[(int64_t)nb * lv.NB + code5(-dx, -dy, -dz, dim)];
-        s_off_out[lane] = lv.pair_off[(int64_t)c * lv.NB + code5(dx, dy, dz, dim)];
         s_ld_in[lane] = lv.cell_b[nb];
         if (lane != center && !lv.weak) {  // weak steps: J = S
           cnt = max(lv.act_cnt[nb], 0);
@@ -2534,11 +2514,6 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (RB == 4 ? 4 : RB == 6 ? 
   // X_RS = A_RS - T^T A_SS,  X_SR = A_SR - A_SS T,  then
   // X_RR = A_RR - T^T A_SR - X_RS T (all as tiled shared-memory products)
   for (int e = tid; e < r * k; e += NT) {
-    int ri, s2;
-    fdr.divmod(e, s2, ri);
-    XRS[ri + s2 * r] = Ab[(k + ri) + s2 * ldb];
-  }
-  for (int e = tid; e < r * k; e += NT) {
     int s2, ri;
     fdk.divmod(e, ri, s2);
     XSR[s2 + ri * k] = Ab[s2 + (k + ri) * ldb];
@@ -2550,9 +2525,8 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (RB == 4 ? 4 : RB == 6 ? 
   }
   __syncthreads();
   {
-    T *xrs = XRS, *xsr = XSR, *lu = LU;
-    const int rr = r, kk = k, ll = ldl;
-    smem_gemm<T, 2>(r, k, k, Ts, k, 1, Ab, ldb, [&](int ri, int s2, T v) { xrs[ri + s2 * rr] -= v; });
+    T *xsr = XSR, *lu = LU;
+    const int kk = k, ll = ldl;
     smem_gemm<T, 1>(k, r, k, Ab, 1, ldb, Ts, k, [&](int s2, int ri, T v) { xsr[s2 + ri * kk] -= v; });
     smem_gemm<T, 2>(r, r, k, Ts, k, 1, Ab + (size_t)k * ldb, ldb, [&](int ri, int rj, T v) { lu[ri * ll + rj] -= v; });
   }
@@ -2560,7 +2534,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (RB == 4 ? 4 : RB == 6 ? 
   {
     T *lu = LU;
     const int ll = ldl;
-    smem_gemm<T, 1>(r, r, k, XRS, 1, r, Ts, k, [&](int ri, int rj, T v) { lu[ri * ll + rj] -= v; });
+    smem_gemm<T, 2>(r, r, k, XSR, k, 1, Ts, k, [&](int ri, int rj, T v) { lu[ri * ll + rj] -= v; });
   }
   __syncthreads();
   if (cta == 0) {
@@ -2587,12 +2561,11 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (RB == 4 ? 4 : RB == 6 ? 
     fb.Xi[e] = Xi[ri + (size_t)qi * ldx];
   }
   }  // cta == 0
-  T *Xrj_out = scratch + (int64_t)q * sstride + (int64_t)nj * r;  // r x nj, for the Schur update
+  T *Xrj_out = scratch + (int64_t)q * sstride;  // r x nj, for the Schur update
   for (int a0 = cta * CH; a0 < nj; a0 += C * CH) {
     const int na = min(CH, nj - a0);
-    // raw rows A(J_a, B) and columns A(B, J_a) of the chunk (S rows come from
-    // X_SR / X_RS); the row / column bases of the chunk are resolved first so
-    // the element loads below are independent of one another
+    // raw rows A(J_a, B) of the chunk (S rows come from X_SR); the rows' bases
+    // are resolved first so the element loads below are independent of one another
     if (tid < na) {
       // (code, local index) of J entry a, as in the J lists above
       const int a = a0 + tid;
@@ -2608,7 +2581,6 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (RB == 4 ? 4 : RB == 6 ? 
       }
       s_rb[tid] = s_off_in[code] + la;
       s_rl[tid] = s_ld_in[code];
-      s_cb[tid] = s_off_out[code] + (int64_t)la * b;
     }
     __syncthreads();
     const FastDiv fdna(max(na, 1));
@@ -2633,69 +2605,42 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (RB == 4 ? 4 : RB == 6 ? 
       for (int u = 0; u < 4; u++)
         if (dst[u] >= 0) rawJ[dst[u]] = val[u];
     }
-    for (int e0 = tid; e0 < na * b; e0 += 4 * NT) {
-      T val[4];
-      int dst[4];
-#pragma unroll
-      for (int u = 0; u < 4; u++) {
-        const int e = e0 + u * NT;
-        val[u] = (T)0;
-        dst[u] = -1;
-        if (e < na * b) {
-          int pp, al;
-          fdb.divmod(e, al, pp);
-          const int a = a0 + al;
-          dst[u] = pp + al * ldb;
-          if (a < k) val[u] = pp >= k ? XRS[(pp - k) + a * r] : (T)0;
-          else val[u] = lv.pool[s_cb[al] + sloc[pp]];
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < 4; u++)
-        if (dst[u] >= 0) rawC[dst[u]] = val[u];
-    }
     __syncthreads();
-    // in place: X_JR = A_JR - A_JS T (rows a >= k);  X_RJ = A_RJ - T^T A_SJ
+    // in place: X_JR = A_JR - A_JS T (rows a >= k)
     {
       const int ldj = CH + 1;
       T *rJ = rawJ;
-      T *rC = rawC;
       const int kk = k, aa0 = a0;
       smem_gemm<T, 1>(na, r, k, rawJ, 1, ldj, Ts, k, [&](int al, int ri, T v) {
         if (aa0 + al >= kk) rJ[al + (kk + ri) * ldj] -= v;
-      });
-      smem_gemm<T, 2>(r, na, k, Ts, k, 1, rawC, ldb, [&](int ri, int al, T v) {
-        if (aa0 + al >= kk) rC[(kk + ri) + al * ldb] -= v;
       });
     }
     __syncthreads();
     for (int e = tid; e < na * r; e += NT) {
       int ri, al;
       fdr.divmod(e, al, ri);
-      Xrj_out[ri + (int64_t)(a0 + al) * r] = rawC[(k + ri) + al * ldb];
+      Xrj_out[ri + (int64_t)(a0 + al) * r] = rawJ[al + (k + ri) * (CH + 1)];
     }
-    if (split) {
-      // X_JR chunk to the scratch (nj x r, ld nj); E and G follow in k_elim_gemm
-      T *Xjr = scratch + (int64_t)q * sstride;
-      for (int e = tid; e < na * r; e += NT) {
-        int al, ri;
-        fdna.divmod(e, ri, al);
-        Xjr[(a0 + al) + (int64_t)ri * nj] = rawJ[al + (k + ri) * (CH + 1)];
-      }
+    if (split) {  // E and G follow in k_elim_gemm from X_RJ
       __syncthreads();
       continue;
     }
-    // E chunk = X_JR chunk * X_RR^{-1};  G chunk = X_RR^{-1} * X_RJ chunk
+    // E chunk = X_JR chunk * X_RR^{-1}, and G's columns
     {
-      T *Eo = fb.E, *Go = fb.G;
-      const int njj = nj, rr = r, aa0 = a0;
-      smem_gemm<T, 1>(na, r, r, rawJ + (size_t)k * (CH + 1), 1, CH + 1, Xi, ldx, [&](int al, int ri, T v) {
-        Eo[(aa0 + al) + (int64_t)ri * njj] = v;
-      });
-      if (Go)  // uniform over the CTA; symmetric storage keeps no G
-        smem_gemm<T, 1>(r, na, r, Xi, 1, ldx, rawC + k, ldb, [&](int ri, int al, T v) {
-          Go[ri + (int64_t)(aa0 + al) * rr] = v;
-        });
+      smem_gemm<T, 1>(na, r, r, rawJ + (size_t)k * (CH + 1), 1, CH + 1, Xi, ldx,
+                      [&](int al, int ri, T v) { ec[al + ri * (CH + 1)] = v; });
+      __syncthreads();
+      for (int e = tid; e < na * r; e += NT) {
+        int al, ri;
+        fdna.divmod(e, ri, al);
+        fb.E[(a0 + al) + (int64_t)ri * nj] = ec[al + ri * (CH + 1)];
+      }
+      if (fb.G)  // uniform over the CTA; symmetric storage keeps no G
+        for (int e = tid; e < na * r; e += NT) {
+          int ri, al;
+          fdr.divmod(e, al, ri);
+          fb.G[ri + (int64_t)(a0 + al) * r] = ec[al + ri * (CH + 1)];
+        }
     }
     __syncthreads();
   }
@@ -2716,7 +2661,7 @@ template <typename T> int64_t elim_smem_bytes(int b, int k, int r) {
 template int64_t elim_smem_bytes<float>(int, int, int);
 template int64_t elim_smem_bytes<double>(int, int, int);
 
-// Elements of T the large-box elimination needs per box beyond X_JR / X_RJ.
+// Elements of T the large-box elimination needs per box beyond X_RJ.
 // k_elim's LU (r x (r+1)) and pivots, or k_elim_lu's X_RR (r x r), r <= bmax
 template <typename T> int64_t elim_ws_elems(int bmax) {
   return (int64_t)bmax * (bmax + 1) + (int64_t)bmax + 64;
@@ -2724,39 +2669,25 @@ template <typename T> int64_t elim_ws_elems(int bmax) {
 template int64_t elim_ws_elems<float>(int);
 template int64_t elim_ws_elems<double>(int);
 
-// E = X_JR X_RR^{-1} (nj x r) and G = X_RR^{-1} X_RJ (r x nj) for the boxes
-// of a phase whose X_JR (ld nj) and X_RJ (ld r) are in the scratch:
-// blockIdx.x = box of the phase, blockIdx.y = a 64 x 64 output tile of E (the
-// first tiles_e) or of G; X_RR^{-1} is in the factor (r x r, column-major).
-// The inner dimension is staged 64 (FP32) or 32 (FP64) at a time, one round
-// for the 2D boxes' r of 45-75 but a remainder: small phases pay one load
-// latency instead of one per 16.  Each thread accumulates a 4 x 4 block.
+// E = X_JR X_RR^{-1} (nj x r) and G = E^T (see k_elim2) for the boxes of a
+// phase whose X_RJ = X_JR^T (r x nj, ld r) is in the scratch: blockIdx.x = box
+// of the phase, blockIdx.y = a 64 x 64 output tile of E; X_RR^{-1} is in the
+// factor (r x r, column-major).  The inner dimension is staged 64 (FP32) or
+// 32 (FP64) at a time, one round for the 2D boxes' r of 45-75 but a remainder:
+// small phases pay one load latency instead of one per 16.  Each thread
+// accumulates a 4 x 4 block.
 template <typename T>
 __global__ void __launch_bounds__(NT) k_elim_gemm(const FBox<T> *boxes, const int *box_list, const T *scratch,
-                                                  int64_t sstride, int tiles_e, int tcols_e, int tcols_g) {
+                                                  int64_t sstride, int tcols) {
   constexpr int KC = sizeof(T) == 4 ? 64 : 32, LD = 64 + 1;
-  __shared__ T As[KC * LD], Bs[KC * LD];
+  __shared__ T sh[2 * KC * LD];  // operands; 64 rows of E for G at the end
+  T *As = sh, *Bs = sh + KC * LD;
   const FBox<T> &fb = boxes[box_list[blockIdx.x]];
   const int r = fb.r, nj = fb.nj;
-  if (r == 0) return;
-  const T *Xjr = scratch + (int64_t)blockIdx.x * sstride;
-  const T *Xrj = Xjr + (int64_t)nj * r;
+  const int i0 = (blockIdx.y / tcols) * 64, j0 = (blockIdx.y % tcols) * 64;
+  if (i0 >= nj || j0 >= r) return;
+  const T *Xrj = scratch + (int64_t)blockIdx.x * sstride;
   const T *Xi = fb.Xi;
-  // C(i, j) = sum_l A(i, l) B(l, j); all operands column-major
-  int m, n, t = blockIdx.y, tcols = tcols_e;
-  const T *A, *B;
-  int64_t lda, ldb, ldc;
-  T *Cp;
-  if (t < tiles_e) {  // E = X_JR Xi: m = nj, n = r
-    m = nj, n = r, A = Xjr, lda = nj, B = Xi, ldb = r, Cp = fb.E, ldc = nj;
-  } else {            // G = Xi X_RJ: m = r, n = nj
-    t -= tiles_e;
-    tcols = tcols_g;
-    m = r, n = nj, A = Xi, lda = r, B = Xrj, ldb = r, Cp = fb.G, ldc = r;
-    if (!Cp) return;  // symmetric storage keeps no G
-  }
-  const int i0 = (t / tcols) * 64, j0 = (t % tcols) * 64;
-  if (i0 >= m || j0 >= n) return;
   const int tid = threadIdx.x, ti = tid & 15, tj = tid >> 4;
   T acc[4][4];
 #pragma unroll
@@ -2767,10 +2698,9 @@ __global__ void __launch_bounds__(NT) k_elim_gemm(const FBox<T> *boxes, const in
     const int kw = min(KC, r - l0);
 #pragma unroll 8
     for (int e = tid; e < KC * 64; e += NT) {
-      const int ii = e & 63, ll = e >> 6;  // A: consecutive rows
-      As[ll * LD + ii] = (i0 + ii < m && ll < kw) ? A[(i0 + ii) + (int64_t)(l0 + ll) * lda] : (T)0;
-      const int l2 = e % KC, jj = e / KC;  // B: consecutive inner index
-      Bs[l2 * LD + jj] = (l2 < kw && j0 + jj < n) ? B[(l0 + l2) + (int64_t)(j0 + jj) * ldb] : (T)0;
+      const int l2 = e % KC, jj = e / KC;  // consecutive inner index
+      As[l2 * LD + jj] = (i0 + jj < nj && l2 < kw) ? Xrj[(l0 + l2) + (int64_t)(i0 + jj) * r] : (T)0;
+      Bs[l2 * LD + jj] = (l2 < kw && j0 + jj < r) ? Xi[(l0 + l2) + (int64_t)(j0 + jj) * r] : (T)0;
     }
     __syncthreads();
 #pragma unroll 4
@@ -2790,19 +2720,27 @@ __global__ void __launch_bounds__(NT) k_elim_gemm(const FBox<T> *boxes, const in
 #pragma unroll
   for (int y = 0; y < 4; y++) {
     const int j = j0 + tj + 16 * y;
-    if (j >= n) continue;
 #pragma unroll
     for (int x = 0; x < 4; x++) {
       const int i = i0 + ti + 16 * x;
-      if (i < m) Cp[i + (int64_t)j * ldc] = acc[x][y];
+      sh[(tj + 16 * y) + (ti + 16 * x) * LD] = acc[x][y];
+      if (i < nj && j < r) fb.E[i + (int64_t)j * nj] = acc[x][y];
+    }
+  }
+  if (fb.G) {  // symmetric storage keeps no G
+    __syncthreads();
+    const int cols = min(64, r - j0), rows = min(64, nj - i0);
+    for (int e = tid; e < 64 * rows; e += NT) {
+      const int j = e & 63, i = e >> 6;
+      if (j < cols) fb.G[(j0 + j) + (int64_t)(i0 + i) * r] = sh[j + i * LD];
     }
   }
 }
 
 template <typename T>
 static void launch_elim_gemm(const FBox<T> *boxes, const int *box_list, int nbox, const T *scratch, int64_t sstride,
-                             int tiles, int tr, int tn, cudaStream_t st) {
-  k_elim_gemm<T><<<dim3(nbox, 2 * tiles), NT, 0, st>>>(boxes, box_list, scratch, sstride, tiles, tr, tn);
+                             int tiles, int tr, cudaStream_t st) {
+  k_elim_gemm<T><<<dim3(nbox, tiles), NT, 0, st>>>(boxes, box_list, scratch, sstride, tr);
   count_launch();
 }
 
@@ -2822,7 +2760,7 @@ __global__ void __launch_bounds__(NT) k_elim_xrr(LevelDev<T> lv, const FBox<T> *
   const int r = fb.r, k = fb.k, b = fb.b, nj = fb.nj;
   const int i0 = (blockIdx.y / tcols) * 64, j0 = (blockIdx.y % tcols) * 64;
   if (r == 0 || i0 >= r || j0 >= r) return;
-  const T *Xrj = scratch + (int64_t)q * sstride + (int64_t)nj * r;
+  const T *Xrj = scratch + (int64_t)q * sstride;
   T *M = scratch + (int64_t)q * sstride + ws_off;
   const int center = code5(0, 0, 0, lv.dim);
   const int self = lv.cell_nbr[(int64_t)fb.cell * lv.NB + center];
@@ -3154,8 +3092,8 @@ void launch_elim(const LevelDev<T> &lv, FBox<T> *boxes, const int *box_list, int
   if (nbox == 0) return;
   const bool force_general = bmax < 0;  // large-box path requested
   if (force_general) bmax = -bmax;
-  // Built in: phases of fewer than 300 boxes (upper levels) leave X_JR and
-  // X_RJ in the scratch and form E and G in k_elim_gemm, spread over the
+  // Built in: phases of fewer than 300 boxes (upper levels) leave X_RJ
+  // in the scratch and form E and G in k_elim_gemm, spread over the
   // whole GPU; large phases form them in the one-CTA-per-box kernel
   // (measured on the 512^2 grid).  The autotuner may choose otherwise.
   int split = nbox < 300 ? 1 : 0;
@@ -3180,16 +3118,15 @@ void launch_elim(const LevelDev<T> &lv, FBox<T> *boxes, const int *box_list, int
       else if (bmax <= 96) run(k_elim2<T, 6>);
       else run(k_elim2<T, 8>);
       count_launch();
-      if (split) launch_elim_gemm<T>(boxes, box_list, nbox, scratch, scratch_stride, tn * tr, tr, tn, st);
+      if (split) launch_elim_gemm<T>(boxes, box_list, nbox, scratch, scratch_stride, tn * tr, tr, st);
       return;
     }
   }
-  // the global workspace sits after the X_JR / X_RJ scratch of the box
+  // the global workspace sits after the X_RJ scratch of the box
   const int64_t ws_off = scratch_stride - elim_ws_elems<T>(bmax);
   const int tiles_e = tn * tr;  // E: nj x r, and as many of G: r x nj
   if (!force_general) {
-    // boxes wider than k_elim2 takes: X_JR and X_RJ over up to 64 CTAs per
-    // box, X_RR as tiles, the LU and X_RR^{-1} blocked in one 1024-thread CTA
+    // boxes wider than k_elim2 takes: X_RJ over up to 64 CTAs per box, X_RR as tiles, the LU and X_RR^{-1} blocked in one 1024-thread CTA
     // per box (3D 32^3 grid: 83 -> 26 ms at eps 1e-3, b ~ 200, and
     // 1063 -> 152 ms at eps 1e-6, b = 448, against k_elim)
     int nbp = sizeof(T) == 4 ? 32 : 16;
@@ -3210,7 +3147,7 @@ void launch_elim(const LevelDev<T> &lv, FBox<T> *boxes, const int *box_list, int
         k_elim_lu<T, 32><<<nbox, NLU, lsm, st>>>(lv, boxes, box_list, scratch, scratch_stride, ws_off, err);
       }
       count_launch(3);
-      launch_elim_gemm<T>(boxes, box_list, nbox, scratch, scratch_stride, tiles_e, tr, tn, st);
+      launch_elim_gemm<T>(boxes, box_list, nbox, scratch, scratch_stride, tiles_e, tr, st);
       return;
     }
   }
@@ -3221,7 +3158,7 @@ void launch_elim(const LevelDev<T> &lv, FBox<T> *boxes, const int *box_list, int
   k_elim<T><<<nbox * Cg, NT, 0, st>>>(lv, boxes, box_list, scratch, scratch_stride, ws_off, ovf, err, Cg, 0);
   // E and G: tiles of 64 x 64 over nj x r (E) and r x nj (G), nj <= njmax, r <= bmax
   count_launch();
-  launch_elim_gemm<T>(boxes, box_list, nbox, scratch, scratch_stride, tiles_e, tr, tn, st);
+  launch_elim_gemm<T>(boxes, box_list, nbox, scratch, scratch_stride, tiles_e, tr, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -3232,7 +3169,7 @@ constexpr int ST = 64;   // output tile
 constexpr int SK = 16;   // inner chunk
 
 // S_JJ = X_JJ - X_JR X_RR^{-1} X_RJ = X_JJ - E X_RJ (Sec. 2.1); X_RJ is still in
-// the elimination scratch of this phase (r x nj column-major after X_JR).
+// the elimination scratch of this phase (r x nj column-major).
 template <typename T>
 __global__ void __launch_bounds__(NT) k_schur(LevelDev<T> lv, const FBox<T> *boxes, const int *box_list,
                                               int tiles1, const T *scratch, int64_t sstride) {
@@ -3250,7 +3187,7 @@ __global__ void __launch_bounds__(NT) k_schur(LevelDev<T> lv, const FBox<T> *box
   const int nj = fb.nj, r = fb.r, dim = lv.dim;
   const int a0 = (tt / tiles1) * ST, c0 = (tt % tiles1) * ST;
   if (a0 >= nj || c0 >= nj || r == 0) return;
-  const T *Xrj = scratch + (int64_t)bi * sstride + (int64_t)nj * r;
+  const T *Xrj = scratch + (int64_t)bi * sstride;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int nc3 = dim == 3 ? 27 : 9;
   if (tid < nc3) {

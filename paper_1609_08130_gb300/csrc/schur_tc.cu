@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(NTC) k_schur_tc(LevelDev<float> lv, const FBox
   uint64_t *s_mbar = reinterpret_cast<uint64_t *>((reinterpret_cast<uintptr_t>(s_misc + 2) + 7) & ~(uintptr_t)7);
 
   const int tid = threadIdx.x, warp = tid >> 5;
-  const float *Xrj = scratch + (int64_t)bi * sstride + (int64_t)nj * r;
+  const float *Xrj = scratch + (int64_t)bi * sstride;
   const int nc3 = dim == 3 ? 27 : 9;
 
   // scatter tables: pair-block offset for every (row cell, column cell) of
