@@ -2662,9 +2662,11 @@ template int64_t elim_smem_bytes<float>(int, int, int);
 template int64_t elim_smem_bytes<double>(int, int, int);
 
 // Elements of T the large-box elimination needs per box beyond X_RJ.
-// k_elim's LU (r x (r+1)) and pivots, or k_elim_lu's X_RR (r x r), r <= bmax
+// k_elim's LU (r x (r+1)) and pivots, or k_elim_lu's X_RR (r x r), r <= bmax;
+// k_elim_gj's X_RR, its inverse and the inverse's residual
 template <typename T> int64_t elim_ws_elems(int bmax) {
-  return (int64_t)bmax * (bmax + 1) + (int64_t)bmax + 64;
+  const int64_t gj = sizeof(T) == 4 && bmax > 128 && bmax <= 224 ? 2 * (int64_t)bmax * bmax : 0;
+  return (int64_t)bmax * (bmax + 1) + (int64_t)bmax + 64 + gj;
 }
 template int64_t elim_ws_elems<float>(int);
 template int64_t elim_ws_elems<double>(int);
@@ -3081,6 +3083,90 @@ __global__ void __launch_bounds__(NLU) k_elim_lu(LevelDev<T> lv, FBox<T> *boxes,
   if (tid == 0) lv.act_cnt[c] = k;
 }
 
+// LU factors of X_RR and its inverse in registers (lu_inverse.cuh, 32 x 32
+// threads) for FP32 boxes of 129..224 DOFs, with the box's skeleton list; the
+// inverse goes to the workspace after X_RR for the Newton step.  Bound: the
+// chain of r steps (32^3 grid, r = 175: 430 us and 75 us for
+// the Newton step, 550 us blocked in shared memory).
+constexpr int GJ_MAX = 224;
+template <int RB>
+__global__ void __launch_bounds__(1024) k_elim_gj(LevelDev<float> lv, FBox<float> *boxes, const int *box_list,
+                                                  float *scratch, int64_t sstride, int64_t ws_off, int *err) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ LuInvShared<float, 32 * RB> s_lu;
+  FBox<float> &fb = boxes[box_list[blockIdx.x]];
+  const int r = fb.r, k = fb.k, tid = threadIdx.x, ldl = r + 1;
+  float *X = reinterpret_cast<float *>(smem_raw);
+  const float *M = scratch + (int64_t)blockIdx.x * sstride + ws_off;  // X_RR, column-major
+  float *V = const_cast<float *>(M) + (int64_t)r * r;                 // its inverse, column-major
+  if (r > 0) {
+    for (int e = tid; e < r * r; e += 1024) X[(e % r) * ldl + e / r] = M[e];
+    __syncthreads();
+    lu_inverse<float, RB, 32, 32 * RB>(r, X, ldl, s_lu, err,
+                                       [&](int i, int c, float v) { V[i + (int64_t)c * r] = v; });
+    for (int e = tid; e < r * r; e += 1024) fb.LU[e] = X[s_lu.piv[e / r] * ldl + e % r];
+    for (int i = tid; i < r; i += 1024) fb.piv[i] = s_lu.piv[i];
+  }
+  // the box's active DOFs are now its skeleton, kept in ascending order
+  const int64_t coff = lv.cell_dof_off[fb.cell];
+  for (int s = tid; s < k; s += 1024) {
+    const int v = fb.loc[s];
+    int rank = 0;
+    for (int s2 = 0; s2 < k; s2++) rank += fb.loc[s2] < v;
+    lv.act_idx[coff + rank] = v;
+  }
+  if (tid == 0) lv.act_cnt[fb.cell] = k;
+}
+
+// The Newton step of those inverses (newton_inverse's, 64 x 64 tiles over the
+// phase): pass 0 R = I - A X after X in the workspace, pass 1 X + X R to the
+// factor.
+template <int PASS>
+__global__ void __launch_bounds__(NT) k_elim_newton(const FBox<float> *boxes, const int *box_list, float *scratch,
+                                                    int64_t sstride, int64_t ws_off, int tr) {
+  constexpr int KC = 64, LD = 64 + 1;
+  __shared__ float As[KC * LD], Bs[KC * LD];
+  const FBox<float> &fb = boxes[box_list[blockIdx.x]];
+  const int r = fb.r, i0 = (blockIdx.y % tr) * 64, j0 = (blockIdx.y / tr) * 64;
+  if (i0 >= r || j0 >= r) return;
+  const int64_t rr = (int64_t)r * r;
+  float *W = scratch + (int64_t)blockIdx.x * sstride + ws_off;
+  const float *A = PASS == 0 ? W : W + rr, *B = PASS == 0 ? W + rr : W + 2 * rr;
+  const int tid = threadIdx.x, ti = tid & 15, tj = tid >> 4;
+  float acc[4][4] = {};
+  for (int l0 = 0; l0 < r; l0 += KC) {
+    const int kw = min(KC, r - l0);
+#pragma unroll 8
+    for (int e = tid; e < KC * 64; e += NT) {
+      const int ii = e & 63, ll = e >> 6;
+      As[ll * LD + ii] = i0 + ii < r && ll < kw ? A[(i0 + ii) + (int64_t)(l0 + ll) * r] : 0.f;
+      Bs[ii * LD + ll] = ii < kw && j0 + ll < r ? B[(l0 + ii) + (int64_t)(j0 + ll) * r] : 0.f;
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int u = 0; u < kw; u++) {
+      float av[4], bv[4];
+#pragma unroll
+      for (int x = 0; x < 4; x++) av[x] = As[u * LD + ti + 16 * x], bv[x] = Bs[u * LD + tj + 16 * x];
+#pragma unroll
+      for (int x = 0; x < 4; x++)
+#pragma unroll
+        for (int y = 0; y < 4; y++) acc[x][y] = fmaf(av[x], bv[y], acc[x][y]);
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int x = 0; x < 4; x++)
+#pragma unroll
+    for (int y = 0; y < 4; y++) {
+      const int i = i0 + ti + 16 * x, j = j0 + tj + 16 * y;
+      if (i >= r || j >= r) continue;
+      const int64_t e = i + (int64_t)j * r;
+      if (PASS == 0) W[2 * rr + e] = (i == j ? 1.f : 0.f) - acc[x][y];
+      else fb.Xi[e] = W[rr + e] + acc[x][y];
+    }
+}
+
 // Shape of the next k_elim2 launch on this thread: (split << 4) | CTAs per
 // box, or 0 for the built-in choice.  Set by the host's autotuner.
 static thread_local int elim_shape_hint = 0;
@@ -3136,6 +3222,23 @@ void launch_elim(const LevelDev<T> &lv, FBox<T> *boxes, const int *box_list, int
       const int Cb = std::min(64, std::max(1, (1216 + nbox - 1) / nbox));
       k_elim<T><<<nbox * Cb, NT, 0, st>>>(lv, boxes, box_list, scratch, scratch_stride, ws_off, ovf, err, Cb, 1);
       k_elim_xrr<T><<<dim3(nbox, tr * tr), NT, 0, st>>>(lv, boxes, box_list, scratch, scratch_stride, ws_off, tr);
+      if constexpr (std::is_same<T, float>::value) {
+        if (bmax <= GJ_MAX) {
+          const size_t xsm = (size_t)bmax * (bmax + 1) * sizeof(float);
+          auto run = [&](auto kern) {
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)xsm);
+            kern<<<nbox, 1024, xsm, st>>>(lv, boxes, box_list, scratch, scratch_stride, ws_off, err);
+          };
+          if (bmax <= 160) run(k_elim_gj<5>);
+          else if (bmax <= 192) run(k_elim_gj<6>);
+          else run(k_elim_gj<7>);
+          k_elim_newton<0><<<dim3(nbox, tr * tr), NT, 0, st>>>(boxes, box_list, scratch, scratch_stride, ws_off, tr);
+          k_elim_newton<1><<<dim3(nbox, tr * tr), NT, 0, st>>>(boxes, box_list, scratch, scratch_stride, ws_off, tr);
+          count_launch(5);
+          launch_elim_gemm<T>(boxes, box_list, nbox, scratch, scratch_stride, tiles_e, tr, st);
+          return;
+        }
+      }
       if (nbp == 8) {
         cudaFuncSetAttribute(k_elim_lu<T, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsm);
         k_elim_lu<T, 8><<<nbox, NLU, lsm, st>>>(lv, boxes, box_list, scratch, scratch_stride, ws_off, err);

@@ -7,10 +7,10 @@
 // replaced by the multipliers.  The rows not yet used go through exactly the
 // steps of an LU factorization, so their multipliers and the pivot rows are L
 // and U; after r steps the registers hold the inverse (of P X, rows and columns
-// in pivot order).  256 threads as 16 x 16, each with RB x RB entries (row
-// ti + 16 x, column tj + 16 y).  A step is two barriers: the half-warp that
-// holds column j picks the pivot and publishes the column, the threads of row
-// p publish the row, all update.
+// in pivot order).  TG x TG threads (16 or 32), each with RB x RB entries (row
+// ti + TG x, column tj + TG y).  A step is two barriers: the TG threads (a half
+// or a whole warp) that hold column j pick the pivot and publish the column,
+// the threads of row p publish the row, all update.
 //
 // Bound: the chain of r steps.  Separate stages (LU in shared memory, 39-56 us
 // at r = 46-66, and a triangular solve per column for the inverse, 41-58 us)
@@ -20,38 +20,38 @@
 
 namespace rss {
 
-template <typename T> struct LuInvShared {
-  T col[2][128], row[2][128], rd[2];
+template <typename T, int NMAX = 128> struct LuInvShared {
+  T col[2][NMAX], row[2][NMAX], rd[2];
   int p[2];
-  int piv[128], pos[128];
+  int piv[NMAX], pos[NMAX];
 };
 
 // X: r x r row-major in shared memory, leading dimension ldl; overwritten by
 // L\U with physical row piv[j] holding row j of P X's factors.  store(i, c, v):
-// entry (i, c) of X^{-1}.  r <= 16 RB.  A zero or NaN pivot records
+// entry (i, c) of X^{-1}.  r <= TG RB <= NMAX.  A zero or NaN pivot records
 // DERR_NUMERIC.  s.piv, s.pos (its inverse) are complete on return.
-template <typename T, int RB, typename Store>
-__device__ __forceinline__ void lu_inverse(int r, T *X, int ldl, LuInvShared<T> &s, int *err, Store store) {
-  const int tid = threadIdx.x, ti = tid & 15, tj = tid >> 4;
+template <typename T, int RB, int TG = 16, int NMAX = 128, typename Store>
+__device__ __forceinline__ void lu_inverse(int r, T *X, int ldl, LuInvShared<T, NMAX> &s, int *err, Store store) {
+  const int tid = threadIdx.x, ti = tid % TG, tj = tid / TG;
   T a[RB][RB];
 #pragma unroll
   for (int x = 0; x < RB; x++)
 #pragma unroll
     for (int y = 0; y < RB; y++) {
-      const int i = ti + 16 * x, c = tj + 16 * y;
+      const int i = ti + TG * x, c = tj + TG * y;
       a[x][y] = i < r && c < r ? X[i * ldl + c] : (T)0;
     }
   unsigned used = 0;  // bit x: row ti + 16 x has been a pivot (or does not exist)
 #pragma unroll
   for (int x = 0; x < RB; x++)
-    if (ti + 16 * x >= r) used |= 1u << x;
+    if (ti + TG * x >= r) used |= 1u << x;
 #pragma unroll
   for (int yj = 0; yj < RB; yj++) {
-    for (int jj = 0; jj < 16; jj++) {
-      const int j = 16 * yj + jj, buf = j & 1;
+    for (int jj = 0; jj < TG; jj++) {
+      const int j = TG * yj + jj, buf = j & 1;
       if (j >= r) break;
       if (tj == jj) {
-        const unsigned half = 0xffffu << (threadIdx.x & 16);
+        const unsigned half = TG == 32 ? 0xffffffffu : 0xffffu << (threadIdx.x & 16);
         // magnitudes compared in FP32 (NaN above infinity), ties to the lowest row
         unsigned key = 0;
         int row = 0x7fffffff;
@@ -59,7 +59,7 @@ __device__ __forceinline__ void lu_inverse(int r, T *X, int ldl, LuInvShared<T> 
         for (int x = 0; x < RB; x++)
           if (!(used >> x & 1)) {
             const unsigned kx = __float_as_uint((float)a[x][yj]) & 0x7fffffffu;
-            if (row == 0x7fffffff || kx > key) key = kx, row = ti + 16 * x;
+            if (row == 0x7fffffff || kx > key) key = kx, row = ti + TG * x;
           }
         const unsigned best = __reduce_max_sync(half, key);
         const int p = __reduce_min_sync(half, key == best ? row : 0x7fffffff);
@@ -69,9 +69,9 @@ __device__ __forceinline__ void lu_inverse(int r, T *X, int ldl, LuInvShared<T> 
           s.pos[p] = j;
         }
 #pragma unroll
-        for (int x = 0; x < RB; x++) s.col[buf][ti + 16 * x] = a[x][yj];
-        if (ti == (p & 15)) {  // the pivot's reciprocal
-          const int xp = p >> 4;
+        for (int x = 0; x < RB; x++) s.col[buf][ti + TG * x] = a[x][yj];
+        if (ti == (p % TG)) {  // the pivot's reciprocal
+          const int xp = p / TG;
           T d = a[0][yj];
 #pragma unroll
           for (int x = 1; x < RB; x++) d = xp == x ? a[x][yj] : d;
@@ -81,12 +81,12 @@ __device__ __forceinline__ void lu_inverse(int r, T *X, int ldl, LuInvShared<T> 
       }
       __syncthreads();
       const int p = s.p[buf];
-      if (ti == (p & 15)) {
-        const int xp = p >> 4;
+      if (ti == (p % TG)) {
+        const int xp = p / TG;
         used |= 1u << xp;
 #pragma unroll
         for (int y = 0; y < RB; y++) {
-          const int c = tj + 16 * y;
+          const int c = tj + TG * y;
           T v = a[0][y];
 #pragma unroll
           for (int x = 1; x < RB; x++) v = xp == x ? a[x][y] : v;
@@ -98,10 +98,10 @@ __device__ __forceinline__ void lu_inverse(int r, T *X, int ldl, LuInvShared<T> 
       const T rd = s.rd[buf];
       T rs[RB];  // the scaled pivot row, 1 / pivot in column j
 #pragma unroll
-      for (int y = 0; y < RB; y++) rs[y] = (y == yj && tj == jj) ? rd : s.row[buf][tj + 16 * y] * rd;
+      for (int y = 0; y < RB; y++) rs[y] = (y == yj && tj == jj) ? rd : s.row[buf][tj + TG * y] * rd;
 #pragma unroll
       for (int x = 0; x < RB; x++) {
-        const int i = ti + 16 * x;
+        const int i = ti + TG * x;
         const T f = s.col[buf][i];
         if (tj == jj) {
           if (!(used >> x & 1)) X[i * ldl + j] = f * rd;
@@ -122,7 +122,7 @@ __device__ __forceinline__ void lu_inverse(int r, T *X, int ldl, LuInvShared<T> 
   for (int x = 0; x < RB; x++)
 #pragma unroll
     for (int y = 0; y < RB; y++) {
-      const int i = ti + 16 * x, c = tj + 16 * y;
+      const int i = ti + TG * x, c = tj + TG * y;
       if (i < r && c < r) store(s.pos[i], s.piv[c], a[x][y]);
     }
   __syncthreads();
