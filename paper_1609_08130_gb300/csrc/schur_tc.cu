@@ -8,15 +8,22 @@
 // distance <= 2), so the product is scattered into them.
 //
 // One CTA of 256 threads (two warpgroups) per (box, 128 rows of J, share of the
-// columns of J): the E rows are staged in shared memory, then for every 64
-// columns of its share the X_RJ
-// columns are staged, the tile E X_RJ is accumulated in tensor memory
-// (M = 128, N = 64, K = 8 per instruction) and every warp reads 32 rows x 32
-// columns of it back (warp w: rows 32 (w mod 4) .., columns 32 (w / 4) ..)
-// and subtracts them from the pair blocks.  54 KB of shared memory per CTA
-// lets four CTAs share an SM, so many scatter loads are in flight.  FP32 accuracy is kept by splitting
-// each operand into a TF32 head and an FP32 remainder: three TF32 products
-// (head x head, head x remainder, remainder x head) per K step.
+// columns of J): for every 64 columns of its share the E rows and X_RJ columns
+// are staged in shared memory 32 of r at a time (the E rows once if r <= 32),
+// the tile E X_RJ is accumulated in tensor memory (M = 128, N = 64, K = 8 per
+// instruction) and every warp reads 32 rows x 32 columns of it back (warp w:
+// rows 32 (w mod 4) .., columns 32 (w / 4) ..) and subtracts them from the pair
+// blocks.  FP32 accuracy is kept by splitting each operand into a TF32 head and
+// an FP32 remainder: three TF32 products (head x head, head x remainder,
+// remainder x head) per K step.
+//
+// Bound: the pair blocks' read-modify-write (the 512^2 grid's first phase: 2.7 GB).
+// What kept it from that was latency, one dependent load after another: the next
+// chunk's operands are now in flight in registers during the MMAs and the
+// scatter, and the scatter is additions that read nothing back; 54 KB of shared
+// memory lets four CTAs share an SM.  Whole class: 64^2 grid 0.45 -> 0.24 ms,
+// 512^2 2.71 -> 2.42, 32^3 4.25 -> 3.57 (a batch of eight loads before its stores
+// instead of the additions: 0.26, 2.68, 3.60).
 #include <algorithm>
 
 #include "internal.h"
@@ -41,7 +48,7 @@ struct SchurTcSmem {
 
 }  // namespace
 
-__global__ void __launch_bounds__(NTC) k_schur_tc(LevelDev<float> lv, const FBox<float> *boxes, const int *box_list,
+__global__ void __launch_bounds__(NTC, 4) k_schur_tc(LevelDev<float> lv, const FBox<float> *boxes, const int *box_list,
                                                   int row_tiles, const float *scratch, int64_t sstride, int *err) {
   extern __shared__ __align__(1024) unsigned char sm[];
   const int bi = blockIdx.x / row_tiles;
@@ -94,9 +101,34 @@ __global__ void __launch_bounds__(NTC) k_schur_tc(LevelDev<float> lv, const FBox
   const uint32_t idesc = tc::idesc_tf32(TM, TN);
   const uint32_t mbar = tc::smem_u32(s_mbar);
   const int nkc = (r + KC - 1) / KC;
+  const float *E = fb.E;
+  // a chunk's operands on their way through registers.  E (column-major, ld
+  // nj): thread = row, two groups of 128 threads over the quads of k.  X_RJ
+  // (column-major, ld r): a warp reads 4 k of 8 columns at a time, whose
+  // shared-memory words are in 32 different banks
+  float pa[KC / 2], pb[TN * KC / NTC];
+  const int arow = tid & (TM - 1), aq = tid / TM, bn = warp * 8 + ((tid & 31) >> 2), bk = tid & 3;
+  auto load_a = [&](int kc) {
+#pragma unroll
+    for (int i = 0; i < KC / 2; i++) {
+      const int k = kc * KC + 4 * (aq + 2 * (i / 4)) + (i & 3);
+      pa[i] = a0 + arow < nj && k < r ? E[a0 + arow + (int64_t)k * nj] : 0.f;
+    }
+  };
+  auto load_b = [&](int kc, int c0) {
+#pragma unroll
+    for (int i = 0; i < KC / 4; i++) {
+      const int k = kc * KC + 4 * i + bk;
+      pb[i] = c0 + bn < nj && k < r ? Xrj[k + (int64_t)(c0 + bn) * r] : 0.f;
+    }
+  };
   uint32_t phase = 0;
   bool ok = true;
   bool first = true;
+  if ((int)blockIdx.y * TN < nj) {
+    load_a(0);
+    load_b(0, blockIdx.y * TN);
+  }
   for (int c0 = blockIdx.y * TN; c0 < nj && ok; c0 += TN * gridDim.y) {
     if (tid < TN) {
       const int cc = c0 + tid;
@@ -106,40 +138,28 @@ __global__ void __launch_bounds__(NTC) k_schur_tc(LevelDev<float> lv, const FBox
     for (int kc = 0; kc < nkc && ok; kc++) {
       const int kw = min(KC, r - kc * KC);       // K of this chunk
       const int kp = (kw + 7) & ~7;              // padded to the MMA's K = 8
-      // E rows a0.. (column-major, ld nj): staged when the chunk changes
-      if (first || nkc > 1) {
-        const int ra = a0 + (tid & (TM - 1));  // rows over the first 128 threads, again for the next
-        const bool ra_ok = ra < nj;
-        for (int q = tid / TM; q < kp / 4; q += NTC / TM) {
+      if (first || nkc > 1) {  // one chunk: E stays staged
+#pragma unroll
+        for (int i = 0; i < KC / 8; i++) {
+          const int q = aq + 2 * i;
+          if (4 * q >= kp) break;
           float hv[4], lv4[4];
 #pragma unroll
-          for (int u = 0; u < 4; u++) {
-            const int k = 4 * q + u;
-            const float x = (ra_ok && k < kw) ? fb.E[ra + (int64_t)(kc * KC + k) * nj] : 0.f;
-            tc::split_tf32(x, hv[u], lv4[u]);
-          }
-          const uint32_t o = tc::kmajor_off(tid & (TM - 1), 4 * q, TM);
+          for (int u = 0; u < 4; u++) tc::split_tf32(pa[4 * i + u], hv[u], lv4[u]);
+          const uint32_t o = tc::kmajor_off(arow, 4 * q, TM);
           *reinterpret_cast<float4 *>(opA_hi + o) = make_float4(hv[0], hv[1], hv[2], hv[3]);
           *reinterpret_cast<float4 *>(opA_lo + o) = make_float4(lv4[0], lv4[1], lv4[2], lv4[3]);
         }
       }
       first = false;
-      // X_RJ columns c0.. (column-major, ld r): (column, 4 consecutive k)
-      // units, column fastest so the shared-memory stores do not conflict
-      const int units = TN * (kp / 4);
-      for (int u0 = tid; u0 < units; u0 += NTC) {
-        const int n = u0 % TN, q = u0 / TN;
-        const int cc = c0 + n;
-        float hv[4], lv4[4];
 #pragma unroll
-        for (int u = 0; u < 4; u++) {
-          const int k = 4 * q + u;
-          const float x = (cc < nj && k < kw) ? Xrj[(kc * KC + k) + (int64_t)cc * r] : 0.f;
-          tc::split_tf32(x, hv[u], lv4[u]);
-        }
-        const uint32_t o = tc::kmajor_off(n, 4 * q, TN);
-        *reinterpret_cast<float4 *>(opB_hi + o) = make_float4(hv[0], hv[1], hv[2], hv[3]);
-        *reinterpret_cast<float4 *>(opB_lo + o) = make_float4(lv4[0], lv4[1], lv4[2], lv4[3]);
+      for (int i = 0; i < KC / 4; i++) {
+        if (4 * i >= kp) break;
+        float h, l;
+        tc::split_tf32(pb[i], h, l);
+        const uint32_t o = tc::kmajor_off(bn, 4 * i + bk, TN);
+        *reinterpret_cast<float *>(opB_hi + o) = h;
+        *reinterpret_cast<float *>(opB_lo + o) = l;
       }
       tc::fence_async_smem();
       tc::fence_before_sync();
@@ -156,6 +176,16 @@ __global__ void __launch_bounds__(NTC) k_schur_tc(LevelDev<float> lv, const FBox
           tc::mma_tf32(tmem, tc::smem_desc(al + oa, 128, 256), tc::smem_desc(bh + ob, 128, 256), idesc, 1u);
         }
         tc::mma_commit(mbar);
+      }
+      // the next chunk's operands fly while the MMAs run (and, at a tile's
+      // end, while the tile is scattered)
+      {
+        const bool more = kc + 1 < nkc;
+        const int nk = more ? kc + 1 : 0, nc = more ? c0 : c0 + TN * (int)gridDim.y;
+        if (nc < nj) {
+          if (nkc > 1) load_a(nk);
+          load_b(nk, nc);
+        }
       }
       // the MMAs have read the operands (and written the accumulator) once
       // the mbarrier's phase completes; a wait that gives up ends the CTA's
@@ -182,12 +212,9 @@ __global__ void __launch_bounds__(NTC) k_schur_tc(LevelDev<float> lv, const FBox
       tc::tmem_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)j0, v);
       if (row_ok) {
 #pragma unroll
-        for (int j = 0; j < 16; j++) {
-          if (c0 + j0 + j >= nj) break;
-          float *dst = pool + po_row[s_cc[j0 + j]] + (int64_t)s_cl[j0 + j] * ld;
-          if (lv.shared) atomicAdd(dst, -v[j]);  // pair blocks other boxes of the phase update too
-          else *dst -= v[j];
-        }
+        for (int j = 0; j < 16; j++)  // other boxes of a 2^d phase may update the same pair blocks
+          if (c0 + j0 + j < nj)
+            atomicAdd(pool + po_row[s_cc[j0 + j]] + (int64_t)s_cl[j0 + j] * ld, -v[j]);
       }
     }
     tc::fence_before_sync();
