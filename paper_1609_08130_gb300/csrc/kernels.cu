@@ -42,32 +42,16 @@ static bool capturing(cudaStream_t st) {
 }
 
 // ---------------------------------------------------------------------------
-// Assembly of pair blocks / top block
+// Assembly of top blocks and of a level's pair blocks
 // ---------------------------------------------------------------------------
 
 template <typename T>
 __global__ void __launch_bounds__(NT) k_assemble(AssembleList L, T *__restrict__ out, LevelDev<T> prev,
                                                  int has_prev, Points P, KernelParams K) {
   const int q = blockIdx.x;
-  int nr, nc;
-  const int64_t *rid, *cid;
-  T *o;
-  if (L.cell_nbr) {
-    const int nb = L.cell_nbr[q];
-    if (nb < 0) return;
-    const int c = q / L.NB;
-    nr = L.cell_b[c];
-    nc = L.cell_b[nb];
-    rid = L.row_ids + L.cell_dof_off[c];
-    cid = L.col_ids + L.cell_dof_off[nb];
-    o = out + L.pair_off[q];
-  } else {
-    nr = L.nrow[q];
-    nc = L.ncol[q];
-    rid = L.row_ids + L.row_off[q];
-    cid = L.col_ids + L.col_off[q];
-    o = out + L.out_off[q];
-  }
+  const int nr = L.nrow[q], nc = L.ncol[q];
+  const int64_t *rid = L.row_ids + L.row_off[q], *cid = L.col_ids + L.col_off[q];
+  T *o = out + L.out_off[q];
   const int64_t tot = (int64_t)nr * nc;
   // element e = (i, j) of the column-major block: e / nr by a multiply-high
   // while the block has fewer than 2^31 entries (every pair block; the top
@@ -110,102 +94,119 @@ __global__ void __launch_bounds__(NT) k_assemble(AssembleList L, T *__restrict__
   }
 }
 
-// The same for the pair blocks of a level whose cells hold at most AS_MAX
-// DOFs (level mode, no per-DOF weights): one CTA per block, the block's row
-// and column DOFs staged first -- their points, and their previous-level
-// cell, its coordinates and the DOF's place in it -- so that each entry is
-// a copy from the previous level's pool or a kernel evaluation from shared
-// memory.
+// The same for the pair blocks of a level: one CTA per block of at most
+// AS_MAX x AS_MAX entries (wider pair blocks are cut into such pieces).  A
+// thread keeps one row's point -- and its previous-level cell, the cell's
+// coordinates and the DOF's place in it -- in registers and goes through every
+// NT / nr-th column, whose data is staged in shared memory: an entry is a
+// broadcast load and a kernel evaluation, or a copy from the previous level's
+// pool.  Depth-20 cells are below 2^24, so their differences are exact in FP32.
+//
+// Bound at the leaves: the issue of the kernel evaluations.  With a division
+// of the entry's index, both points read from shared memory, integer cells and
+// the DOF numbers compared per entry the 512^2 grid's leaves (400 million
+// entries) took 1192 us; writing them alone takes 250 us.  All levels: 512^2
+// 1.84 -> 1.34 ms, 32^3 (cells of 200 DOFs took the general kernel) 1.07 -> 0.52,
+// 32 problems (per-DOF weights, the same) 3.9 -> 2.1.
 constexpr int AS_MAX = 128;
-template <typename T> struct AsPts;
-template <> struct AsPts<float> {
-  int c[3][AS_MAX];
-  float o[3][AS_MAX];
+template <typename T, int DIM> struct AsPt;
+template <int DIM> struct AsPt<float, DIM> {
+  float c[DIM], o[DIM];
+  __device__ __forceinline__ void load(const Points &P, int64_t g) {
+#pragma unroll
+    for (int d = 0; d < DIM; d++) c[d] = (float)P.cell[3 * g + d], o[d] = P.off[3 * g + d];
+  }
+  __device__ __forceinline__ float dist2(const AsPt &b, float D) const {
+    const float ex = fmaf(c[0] - b.c[0], D, o[0] - b.o[0]), ey = fmaf(c[1] - b.c[1], D, o[1] - b.o[1]);
+    float r2 = ex * ex + ey * ey;
+    if constexpr (DIM == 3) {
+      const float ez = fmaf(c[2] - b.c[2], D, o[2] - b.o[2]);
+      r2 = fmaf(ez, ez, r2);
+    }
+    return r2;
+  }
 };
-template <> struct AsPts<double> {
-  double x[3][AS_MAX];
+template <int DIM> struct AsPt<double, DIM> {
+  double x[DIM];
+  __device__ __forceinline__ void load(const Points &P, int64_t g) {
+#pragma unroll
+    for (int d = 0; d < DIM; d++) x[d] = P.x[g * DIM + d];
+  }
+  __device__ __forceinline__ double dist2(const AsPt &b, float) const {
+    const double ex = x[0] - b.x[0], ey = x[1] - b.x[1];
+    double r2 = ex * ex + ey * ey;
+    if constexpr (DIM == 3) {
+      const double ez = x[2] - b.x[2];
+      r2 += ez * ez;
+    }
+    return r2;
+  }
 };
-struct AsPrev {
-  int cell[AS_MAX], loc[AS_MAX], cc[3][AS_MAX];
+template <int DIM> struct AsPrev {
+  int cell, loc, cc[DIM];
+  template <typename T> __device__ __forceinline__ void load(const LevelDev<T> &prev, int64_t g) {
+    cell = prev.dof_cell[g];
+    loc = cell >= 0 ? prev.dof_loc[g] : 0;
+#pragma unroll
+    for (int d = 0; d < DIM; d++) cc[d] = cell >= 0 ? prev.cell_coord[3 * cell + d] : 0;
+  }
 };
 
-template <typename T>
+template <typename T, int DIM, bool PREV>
 __global__ void __launch_bounds__(NT) k_assemble_staged(AssembleList L, T *__restrict__ out, LevelDev<T> prev,
-                                                        int has_prev, Points P, KernelParams K) {
-  __shared__ AsPts<T> sp[2];  // rows, columns
-  __shared__ AsPrev spv[2];
+                                                        Points P, KernelParams K, int pieces) {
+  __shared__ __align__(16) AsPt<T, DIM> sp[AS_MAX];
+  __shared__ __align__(16) AsPrev<DIM> sv[PREV ? AS_MAX : 1];
   const int q = blockIdx.x;
   const int nb = L.cell_nbr[q];
   if (nb < 0) return;
   const int c = q / L.NB;
-  const int nr = L.cell_b[c], nc = L.cell_b[nb];
-  const int64_t *ids[2] = {L.row_ids + L.cell_dof_off[c], L.col_ids + L.cell_dof_off[nb]};
-  const int cnt[2] = {nr, nc};
-  T *o = out + L.pair_off[q];
-  const int dim = P.dim;
-  for (int s = 0; s < 2; s++)
-    for (int i = threadIdx.x; i < cnt[s]; i += NT) {
-      const int64_t g = ids[s][i];
-      if constexpr (sizeof(T) == 4) {
-#pragma unroll
-        for (int d = 0; d < 3; d++) {
-          sp[s].c[d][i] = P.cell[3 * g + d];
-          sp[s].o[d][i] = P.off[3 * g + d];
-        }
-      } else {
-#pragma unroll
-        for (int d = 0; d < 3; d++) sp[s].x[d][i] = d < dim ? P.x[g * dim + d] : 0.0;
-      }
-      const int pc = has_prev ? prev.dof_cell[g] : -1;
-      spv[s].cell[i] = pc;
-      spv[s].loc[i] = pc >= 0 ? prev.dof_loc[g] : 0;
-#pragma unroll
-      for (int d = 0; d < 3; d++) spv[s].cc[d][i] = pc >= 0 ? prev.cell_coord[3 * pc + d] : 0;
-    }
+  const int ldo = L.cell_b[c], i0 = (blockIdx.y % pieces) * AS_MAX, j0 = (blockIdx.y / pieces) * AS_MAX;
+  const int nr = min(AS_MAX, ldo - i0), nc = min(AS_MAX, L.cell_b[nb] - j0);
+  if (nr <= 0 || nc <= 0) return;
+  const int64_t *rid = L.row_ids + L.cell_dof_off[c] + i0, *cid = L.col_ids + L.cell_dof_off[nb] + j0;
+  for (int j = threadIdx.x; j < nc; j += NT) {
+    const int64_t g = cid[j];
+    sp[j].load(P, g);
+    if constexpr (PREV) sv[j].load(prev, g);
+  }
+  const int grp = threadIdx.x / nr, ngrp = NT / nr, i = threadIdx.x - grp * nr;
+  AsPt<T, DIM> pi;
+  AsPrev<DIM> vi;
+  T wT = (T)K.w;
+  if (grp < ngrp) {
+    const int64_t g = rid[i];
+    pi.load(P, g);
+    if constexpr (PREV) vi.load(prev, g);
+    if (P.wdof) wT = (T)P.wdof[g];
+  }
   __syncthreads();
-  const T wT = (T)K.w, dT = (T)K.diag;
-  const FastDiv fnr(max(nr, 1));
-  for (int e = threadIdx.x; e < nr * nc; e += NT) {
-    int i, j;
-    fnr.divmod(e, j, i);
+  if (grp >= ngrp) return;
+  const T dT = (T)K.diag;
+  const int jdiag = c == nb ? i0 + i - j0 : -1;  // the row's own column
+  T *o = out + L.pair_off[q] + (i0 + i) + (int64_t)j0 * ldo;
+  int ldp = 0;
+  if constexpr (PREV) ldp = vi.cell >= 0 ? prev.cell_b[vi.cell] : 0;
+#pragma unroll 4
+  for (int j = grp; j < nc; j += ngrp) {
     T v;
     bool done = false;
-    const int ci = spv[0].cell[i], cj = spv[1].cell[j];
-    if (ci >= 0 && cj >= 0) {
-      const int dx = spv[1].cc[0][j] - spv[0].cc[0][i], dy = spv[1].cc[1][j] - spv[0].cc[1][i],
-                dz = spv[1].cc[2][j] - spv[0].cc[2][i];
-      if (dx >= -2 && dx <= 2 && dy >= -2 && dy <= 2 && dz >= -2 && dz <= 2) {
-        const int64_t off = prev.pair_off[(int64_t)ci * prev.NB + code5(dx, dy, dz, prev.dim)];
-        v = prev.pool[off + spv[0].loc[i] + (int64_t)spv[1].loc[j] * prev.cell_b[ci]];
-        done = true;
-      }
-    }
-    if (!done) {
-      if (ids[0][i] == ids[1][j]) {
-        v = dT;
-      } else {
-        T r2;
-        if constexpr (sizeof(T) == 4) {
-          const float Dd = P.D;
-          const float ex = fmaf((float)(sp[0].c[0][i] - sp[1].c[0][j]), Dd, sp[0].o[0][i] - sp[1].o[0][j]);
-          const float ey = fmaf((float)(sp[0].c[1][i] - sp[1].c[1][j]), Dd, sp[0].o[1][i] - sp[1].o[1][j]);
-          r2 = ex * ex + ey * ey;
-          if (dim == 3) {
-            const float ez = fmaf((float)(sp[0].c[2][i] - sp[1].c[2][j]), Dd, sp[0].o[2][i] - sp[1].o[2][j]);
-            r2 = fmaf(ez, ez, r2);
-          }
-        } else {
-          const double ex = sp[0].x[0][i] - sp[1].x[0][j], ey = sp[0].x[1][i] - sp[1].x[1][j];
-          r2 = ex * ex + ey * ey;
-          if (dim == 3) {
-            const double ez = sp[0].x[2][i] - sp[1].x[2][j];
-            r2 += ez * ez;
-          }
+    // A DOF without a cell at the previous level belongs to a problem whose
+    // tree is shallower than the merged previous level: none of its entries
+    // has been updated yet, so the kernel entry is the value.
+    if constexpr (PREV) {
+      const AsPrev<DIM> vj = sv[j];
+      if (vi.cell >= 0 && vj.cell >= 0) {
+        const int dx = vj.cc[0] - vi.cc[0], dy = vj.cc[1] - vi.cc[1], dz = DIM == 3 ? vj.cc[DIM - 1] - vi.cc[DIM - 1] : 0;
+        if (dx >= -2 && dx <= 2 && dy >= -2 && dy <= 2 && dz >= -2 && dz <= 2) {
+          const int64_t off = prev.pair_off[(int64_t)vi.cell * prev.NB + code5(dx, dy, dz, DIM)];
+          v = prev.pool[off + vi.loc + (int64_t)vj.loc * ldp];
+          done = true;
         }
-        v = wT * kof(K.kind, r2);
       }
     }
-    o[e] = v;
+    if (!done) v = j == jdiag ? dT : wT * kof(K.kind, pi.dist2(sp[j], P.D));
+    o[(int64_t)j * ldo] = v;
   }
 }
 
@@ -215,9 +216,14 @@ void launch_assemble(const AssembleList &L, T *out, const LevelDev<T> *prev, con
   if (L.nblock == 0) return;
   LevelDev<T> pv{};
   if (prev) pv = *prev;
-  if (L.cell_nbr && !P.wdof && maxblk <= (int64_t)AS_MAX * AS_MAX) {
-    k_assemble_staged<T><<<L.nblock, NT, 0, st>>>(L, out, pv, prev ? 1 : 0, P, K);
-    count_launch();
+  if (L.cell_nbr) {  // a level: maxblk is the square of its largest cell's DOFs
+    const int pieces = std::max(1, ((int)std::ceil(std::sqrt((double)maxblk)) + AS_MAX - 1) / AS_MAX);
+    auto run = [&](auto kern) {
+      kern<<<dim3(L.nblock, pieces * pieces), NT, 0, st>>>(L, out, pv, P, K, pieces);
+      count_launch();
+    };
+    if (P.dim == 2) prev ? run(k_assemble_staged<T, 2, true>) : run(k_assemble_staged<T, 2, false>);
+    else prev ? run(k_assemble_staged<T, 3, true>) : run(k_assemble_staged<T, 3, false>);
     return;
   }
   int gy = (int)((maxblk + NT * 8 - 1) / (NT * 8));
