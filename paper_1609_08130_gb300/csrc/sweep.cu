@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(NT) k_apply_fwd(const FBox<T> *boxes, const in
   __shared__ int64_t s_j[SWEEP_CHUNK];
   __shared__ int s_last;
   pdl_launch_next();
-  const int bi = wbox[blockIdx.x], ch = wchunk[blockIdx.x], tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int bi = wbox[blockIdx.x], ch = wchunk[blockIdx.x], tid = threadIdx.x;
   T *v = vall + blockIdx.y * vstride, *p0 = pball + blockIdx.y * pstride + poff[bi];
   Box<T, NR> x = open_box<T, NR>(boxes, bi, ch, sm);
   const int k = x.k, r = x.r, a0 = ch * SWEEP_CHUNK;
@@ -308,36 +308,14 @@ __global__ void __launch_bounds__(NT) k_apply_fwd(const FBox<T> *boxes, const in
   if (!last_of_box(cntall + (int64_t)blockIdx.y * nbox + bi, x.nchunk, &s_last)) return;
   __threadfence();
   sum_chunks(x, p0, vR, (T)1);
-  // U v_R, then L of it: a warp per row of the row-major LU
+  // U v_R, then L of it (row-major LU), as full products with zeros: a warp per
+  // row spent 20 FP64 additions of its lanes' sums on 4 results, 14 us of the
+  // FP64 unit per triangle at r = 60
   const T *LU = x.fb.LU;
-  T *y = x.w;
-  for (int half = 0; half < 2; half++) {
-    const T *in = half == 0 ? vR : y;
-    for (int i = warp; i < r; i += NT / 32) {
-      T acc[NR];
-#pragma unroll
-      for (int c = 0; c < NR; c++) acc[c] = (T)0;
-      const int l0 = half == 0 ? i : 0, l1 = half == 0 ? r : i;
-      for (int l = l0 + lane; l < l1; l += 32) {
-        const T a = __ldg(LU + (int64_t)i * r + l);
-#pragma unroll
-        for (int c = 0; c < NR; c++) acc[c] += a * in[l * NR + c];
-      }
-#pragma unroll
-      for (int c = 0; c < NR; c++) acc[c] = warp_sum(acc[c]);
-      if (lane == 0) {
-        if (half == 0) {
-#pragma unroll
-          for (int c = 0; c < NR; c++) y[i * NR + c] = acc[c];
-        } else {
-          T *vg = v + x.ids[k + x.fb.piv[i]] * NR;
-#pragma unroll
-          for (int c = 0; c < NR; c++) vg[c] = y[i * NR + c] + acc[c];
-        }
-      }
-    }
-    __syncthreads();
-  }
+  T *y = x.w, *z = x.w + (size_t)(k + r) * NR;
+  mat_vec<T, NR>(r, r, [&](int i, int l) { return l >= i ? __ldg(LU + (int64_t)i * r + l) : (T)0; }, vR, x.part, y);
+  mat_vec<T, NR>(r, r, [&](int i, int l) { return l < i ? __ldg(LU + (int64_t)i * r + l) : (T)0; }, y, x.part, z);
+  for (int e = tid; e < r * NR; e += NT) v[x.ids[k + x.fb.piv[e / NR]] * NR + e % NR] = y[e] + z[e];
   for (int e = tid; e < k * NR; e += NT) v[x.ids[e / NR] * NR + e % NR] = x.vB[e];
 }
 
