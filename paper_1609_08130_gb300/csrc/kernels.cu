@@ -3092,16 +3092,19 @@ __global__ void __launch_bounds__(NLU) k_elim_lu(LevelDev<T> lv, FBox<T> *boxes,
 // LU factors of X_RR and its inverse in registers (lu_inverse.cuh, 32 x 32
 // threads) for FP32 boxes of 129..224 DOFs, with the box's skeleton list; the
 // inverse goes to the workspace after X_RR for the Newton step.  Bound: the
-// chain of r steps (32^3 grid, r = 175: 430 us and 75 us for
-// the Newton step, 550 us blocked in shared memory).
+// chain of r steps.  32^3 grid, r = 175: 430 us with 7 x 7 entries a thread (which
+// spill), about 280 us with the 6 x 6 of boxes with r <= 192, and 75 us for the
+// Newton step; 550 us blocked in shared memory (elimination class 7.0 -> 5.3 ms).
 constexpr int GJ_MAX = 224;
 template <int RB>
 __global__ void __launch_bounds__(1024) k_elim_gj(LevelDev<float> lv, FBox<float> *boxes, const int *box_list,
-                                                  float *scratch, int64_t sstride, int64_t ws_off, int *err) {
+                                                  float *scratch, int64_t sstride, int64_t ws_off, int *err,
+                                                  int rmin, int rmax) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ LuInvShared<float, 32 * RB> s_lu;
   FBox<float> &fb = boxes[box_list[blockIdx.x]];
   const int r = fb.r, k = fb.k, tid = threadIdx.x, ldl = r + 1;
+  if (r < rmin || r > rmax) return;
   float *X = reinterpret_cast<float *>(smem_raw);
   const float *M = scratch + (int64_t)blockIdx.x * sstride + ws_off;  // X_RR, column-major
   float *V = const_cast<float *>(M) + (int64_t)r * r;                 // its inverse, column-major
@@ -3231,16 +3234,18 @@ void launch_elim(const LevelDev<T> &lv, FBox<T> *boxes, const int *box_list, int
       if constexpr (std::is_same<T, float>::value) {
         if (bmax <= GJ_MAX) {
           const size_t xsm = (size_t)bmax * (bmax + 1) * sizeof(float);
-          auto run = [&](auto kern) {
+          // boxes by their own r: 7 x 7 entries do not quite fit the registers
+          // of 1024 threads
+          auto run = [&](auto kern, int rmin, int rmax) {
             cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)xsm);
-            kern<<<nbox, 1024, xsm, st>>>(lv, boxes, box_list, scratch, scratch_stride, ws_off, err);
+            kern<<<nbox, 1024, xsm, st>>>(lv, boxes, box_list, scratch, scratch_stride, ws_off, err, rmin, rmax);
+            count_launch();
           };
-          if (bmax <= 160) run(k_elim_gj<5>);
-          else if (bmax <= 192) run(k_elim_gj<6>);
-          else run(k_elim_gj<7>);
+          run(k_elim_gj<6>, 0, 192);
+          if (bmax > 192) run(k_elim_gj<7>, 193, GJ_MAX);
           k_elim_newton<0><<<dim3(nbox, tr * tr), NT, 0, st>>>(boxes, box_list, scratch, scratch_stride, ws_off, tr);
           k_elim_newton<1><<<dim3(nbox, tr * tr), NT, 0, st>>>(boxes, box_list, scratch, scratch_stride, ws_off, tr);
-          count_launch(5);
+          count_launch(4);
           launch_elim_gemm<T>(boxes, box_list, nbox, scratch, scratch_stride, tiles_e, tr, st);
           return;
         }
