@@ -5,15 +5,17 @@
 // dimension), a panel per step:
 //   k_lu_panel  one CTA per problem: a thread holds its rows of the panel in
 //               registers; a column step is one barrier (every warp publishes
-//               its best row, all threads pick the winner); rows are moved once
-//               at the end;
+//               its best row, every warp picks the winner by a reduction over
+//               the warps' keys); rows are moved once at the end;
 //   k_lu_trsm   the panel's row moves on the other columns, U12;
 //   k_lu_gemm   A22 -= L21 U12.
 // Each launch is a programmatic dependent of the one before.  Bound: the chain
-// of n column steps.  Measured, LU and inverse: FP32 n = 305 1.29 -> 0.55 ms (a
+// of n column steps.  Measured, LU and inverse: FP32 n = 305 1.29 -> 0.46 ms (a
 // panel in shared memory with three barriers a column before), n = 1600
-// 9.5 -> 6.1 ms (the LU alone before), FP64 n = 313 2.78 -> 1.56 ms, 32 problems of
-// n = 310 10.4 -> 1.5 ms (one CTA each, unblocked, before).
+// 9.5 -> 5.7 ms (the LU alone before), FP64 n = 313 2.78 -> 1.49 ms, 32 problems of
+// n = 310 10.4 -> 1.4 ms (one CTA each, unblocked, before).  A column's
+// pivot row in 16-byte pieces and the winner by a warp reduction instead of 16
+// reads and compares a thread are 0.08, 0.5 and 0.06 ms of it.
 //
 // k_top_inverse forms W = U^{-1} L^{-1}: the diagonal blocks' inverses first,
 // then a CTA per group of columns goes through the row blocks of L and of U
@@ -37,6 +39,12 @@ __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// 16 bytes of a pivot row
+template <typename T> struct alignas(16) Pack {
+  static constexpr int N = 16 / sizeof(T);
+  T x[N];
+};
+
 // a panel's row moves: position dst[e] (from the panel's first row) takes the
 // row that was at src[e]
 struct Moves {
@@ -51,7 +59,7 @@ struct Moves {
 template <typename T, int NB, int RPT>
 __global__ void __launch_bounds__(PT) k_lu_panel(T *LUall, const int64_t *loff, const int *tn, int *pivall,
                                                  const int64_t *toff, int kb, Moves *moves, int *err) {
-  constexpr int NW = PT / 32;
+  constexpr int NW = PT / 32, VW = Pack<T>::N;
   __shared__ unsigned s_key[2][NW];
   __shared__ int s_idx[2][NW], s_prow[NB], s_at[PT * RPT], s_where[PT * RPT];
   __shared__ __align__(16) T s_row[2][NW][NB];
@@ -98,20 +106,23 @@ __global__ void __launch_bounds__(PT) k_lu_panel(T *LUall, const int64_t *loff, 
         s_key[buf][warp] = kw;
         s_idx[buf][warp] = tid + PT * qb;
 #pragma unroll
-        for (int c = j; c < NB; c++) {
-          T v = a[0][c];
+        for (int c0 = j / VW * VW; c0 < NB; c0 += VW) {
+          Pack<T> v;
 #pragma unroll
-          for (int q = 1; q < RPT; q++) v = qb == q ? a[q][c] : v;
-          s_row[buf][warp][c] = v;
+          for (int c = 0; c < VW; c++) {
+            v.x[c] = a[0][c0 + c];
+#pragma unroll
+            for (int q = 1; q < RPT; q++) v.x[c] = qb == q ? a[q][c0 + c] : v.x[c];
+          }
+          *reinterpret_cast<Pack<T> *>(&s_row[buf][warp][c0]) = v;
         }
       }
       __syncthreads();
-      int bw = -1;
-      unsigned bk = 0;
-#pragma unroll
-      for (int x = 0; x < NW; x++)
-        if (s_idx[buf][x] >= 0 && (bw < 0 || s_key[buf][x] > bk)) bk = s_key[buf][x], bw = x;
-      const int pr = s_idx[buf][bw];
+      // the first of the warps' largest keys (0: a warp with no row left)
+      const int wi = s_idx[buf][lane % NW];
+      const unsigned wk = wi >= 0 ? s_key[buf][lane % NW] + 1u : 0u;
+      const int bw = (__ffs(__ballot_sync(0xffffffffu, wk == __reduce_max_sync(0xffffffffu, wk))) - 1) % NW;
+      const int pr = __shfl_sync(0xffffffffu, wi, bw);
       const T *row = s_row[buf][bw];
       T rd;
       if (sizeof(T) == 8) {  // one reciprocal on the FP64 pipe instead of one a warp
@@ -125,15 +136,33 @@ __global__ void __launch_bounds__(PT) k_lu_panel(T *LUall, const int64_t *loff, 
         s_prow[j] = pr;
         if (!(row[j] > (T)0 || row[j] < (T)0)) set_err(err, DERR_NUMERIC);
       }
+      T l[RPT];
 #pragma unroll
       for (int q = 0; q < RPT; q++) {
         if (tid + PT * q == pr) used |= 1u << q;
-        else if (!(used >> q & 1)) {
-          const T l = a[q][j] * rd;
-          a[q][j] = l;
+        l[q] = (T)0;
+        if (!(used >> q & 1)) a[q][j] = l[q] = a[q][j] * rd;
+      }
+      auto update = [&](int q, int c0) {
+        const Pack<T> v = *reinterpret_cast<const Pack<T> *>(row + c0);
 #pragma unroll
-          for (int c = j + 1; c < NB; c++) a[q][c] -= l * row[c];
-        }
+        for (int c = 0; c < VW; c++)
+          if (c0 + c > j) a[q][c0 + c] -= l[q] * v.x[c];
+      };
+      // FP64 row by row, so that a warp without rows left issues nothing
+      if constexpr (sizeof(T) == 8) {
+#pragma unroll
+        for (int q = 0; q < RPT; q++)
+          if (!(used >> q & 1)) {
+#pragma unroll
+            for (int c0 = (j + 1) / VW * VW; c0 < NB; c0 += VW) update(q, c0);
+          }
+      } else {
+#pragma unroll
+        for (int c0 = (j + 1) / VW * VW; c0 < NB; c0 += VW)
+#pragma unroll
+          for (int q = 0; q < RPT; q++)
+            if (!(used >> q & 1)) update(q, c0);
       }
     }
   }
