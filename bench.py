@@ -307,12 +307,9 @@ def run_reference(args, rank, world):
 
 # DRAM bytes (read + write) per launch of a kernel class from an ncu capture,
 # valid only for the kernel source it was taken on (sha-256 of kernels.cu).
-NCU_TRAFFIC = {
-    # the ID's DRAM bytes per launch of the 512^2 step: an ncu capture of
-    # every ID launch of the 256^2 step, scaled by box count per depth
-    "id": {"bytes_per_launch": 56.5e6,
-           "kernels_sha256": "99f814ed756e6b283225728feb3d05a00f1215091221cac1355706e1481e9379"},
-}
+# Entry: class -> {"bytes_per_launch": ..., "kernels_sha256": ...}; none is held
+# for the current source.
+NCU_TRAFFIC = {}
 
 
 def ncu_traffic(cls):

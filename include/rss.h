@@ -268,8 +268,8 @@ rss_status rss_sqrt_apply(const rss_factorization *f, const double *x, double *y
 /* rss_matvec -- y = A x in FP64 with the exact operator being factored:
  * an FFT convolution when the points are the cell centres of an s^dim grid
  * (s a power of two; exact up to FP64 rounding), direct summation over all
- * pairs otherwise (the 2D kernel's logarithm table-driven, to a few units
- * of FP64 rounding).  Device buffers, n x nrhs column-major. */
+ * pairs otherwise (in pairs of FP32 numbers, 48 bits a term, the terms added
+ * up in FP64: an error no larger than that of a plain FP64 sum).  Device buffers, n x nrhs column-major. */
 rss_status rss_matvec(const rss_factorization *f, const double *x, double *y, int nrhs);
 
 /* rss_sync -- wait for the factor's stream, then report an error the device
@@ -406,7 +406,14 @@ rss_status rss_box_features(const rss_factorization *f, float *feat, int32_t *ra
  * every candidate on its own boxes (the ID launch is idempotent), keeps the
  * fastest for the rest of the process and re-runs it, so factorizations
  * with the same key compute the same result.  Disabled per factorization by
- * RSS_FLAG_NO_AUTOTUNE.  *nbytes in/out as in rss_tree_query. */
+ * RSS_FLAG_NO_AUTOTUNE.  *nbytes in/out as in rss_tree_query.
+ * An FP32 factor with eps >= 5e-7 and boxes of at most 512 DOFs has one more
+ * form of the ID, from the rows' exact Gram matrix on the tensor cores (the
+ * same truncation, ranks equal up to ties): it is timed once per key beside
+ * these shapes and taken where it is faster than all of them.  It is not in
+ * the table; a shape fixed by rss_autotune_set is always used as set.  With
+ * RSS_FLAG_NO_AUTOTUNE, and for boxes wider than 256, such a factor takes it
+ * without timing. */
 rss_status rss_autotune_table(int32_t *buf, size_t *nbytes);
 
 /* rss_autotune_set -- fix the shape used for one key (e.g. a table saved
@@ -423,7 +430,7 @@ rss_status rss_autotune_set(int elem_bytes, int width, int phase_class, int tpc,
  * (64 or 128), phase-size class, chosen split flag and CTAs per box, then the
  * measured time in microseconds of the 5 candidates (split, CTAs per box) =
  * (0,1) (1,1) (1,2) (1,4) (1,8)}.  Split 0 forms E and G in the same kernel
- * as the LU of X_RR, one CTA per box; split 1 leaves X_JR and X_RJ in scratch
+ * as the LU of X_RR, one CTA per box; split 1 leaves X_RJ in scratch
  * for a phase-wide product kernel, the box's rows of J shared by that many
  * CTAs.  The first phase of a key times every candidate (the elimination of
  * a phase writes the same values however often it runs), keeps the fastest

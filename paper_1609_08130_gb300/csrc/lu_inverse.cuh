@@ -14,7 +14,8 @@
 //
 // Bound: the chain of r steps.  Separate stages (LU in shared memory, 39-56 us
 // at r = 46-66, and a triangular solve per column for the inverse, 41-58 us)
-// were most of an upper level's elimination launch.
+// were most of an upper level's elimination launch (elimination of the 64^2 grid
+// 2.24 -> 1.48 ms with this form, of the 100^2 grid in FP64 12.9 -> 10.1).
 #pragma once
 #include "common.cuh"
 
