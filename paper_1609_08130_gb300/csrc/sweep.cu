@@ -31,6 +31,7 @@ namespace {
 constexpr int NT = 256;
 constexpr int MLP = 8;            // independent loads a thread keeps in flight
 constexpr int T_STAGE = 2048;     // entries of T staged in shared memory (every 2D box; wider boxes read it from L2)
+constexpr int WIDE_ENTRIES = 64 * NT;  // X_RR^{-1} and E_S of a box shared by its CTAs above this
 constexpr int SWEEP_SMEM = (200 << 10) + 64;
 
 __device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -181,10 +182,16 @@ template <typename T, int NR> __device__ __forceinline__ int64_t near_id(const B
 }  // namespace
 
 // Solve, forward: y = v_R - T^T v_S; v_N -= E_N y; the last CTA: v_S -= E_S y,
-// v_R = X_RR^{-1} y.
+// v_R = X_RR^{-1} y.  Where that last product is more than 64 entries a thread
+// (the 32^3 grid's upper boxes: 137, a chain of 22 rounds of loads) every CTA
+// forms its share of the rows and the last one only adds them in (32^3 case
+// 22.9 -> 21.6 ms); below, the round trip through memory costs more than it
+// saves.  For one or two columns: with more the registers it takes slowed the
+// large phases (16 columns on the 256^2 grid by 1 %).
 template <typename T, int NR>
 __global__ void __launch_bounds__(NT) k_sweep_fwd(const FBox<T> *boxes, const int *wbox, const int *wchunk, T *vall,
-                                                  int64_t vstride, int *cntall, int nbox) {
+                                                  int64_t vstride, int *cntall, int nbox, T *pball, int64_t pstride,
+                                                  const int64_t *poff) {
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ int s_last;
   pdl_launch_next();
@@ -203,13 +210,32 @@ __global__ void __launch_bounds__(NT) k_sweep_fwd(const FBox<T> *boxes, const in
   for (int e = tid; e < r * NR; e += NT) y[e] = x.vB[k * NR + e] - y[e];
   __syncthreads();
   add_near(x, jid, y, (T)-1, v);
-  if (!last_of_box(cntall + (int64_t)blockIdx.y * nbox + bi, x.nchunk, &s_last)) return;
   // the k rows of E at the head of J and the r rows of X_RR^{-1} as one
-  // product of b rows
+  // product of b rows, i0 .. i0 + ni - 1 of them
   const T *E = x.fb.E, *Xi = x.fb.Xi;
-  mat_vec<T, NR>(k + r, r,
-                 [&](int i, int l) { return i < k ? __ldg(E + i + (int64_t)l * nj) : __ldg(Xi + (i - k) + (int64_t)l * r); },
-                 y, x.part, z);
+  auto product = [&](int i0, int ni, T *out) {
+    mat_vec<T, NR>(ni, r,
+                   [&](int i, int l) {
+                     return i0 + i < k ? __ldg(E + i0 + i + (int64_t)l * nj) : __ldg(Xi + (i0 + i - k) + (int64_t)l * r);
+                   },
+                   y, x.part, out);
+  };
+  // the partial sums' space of the backward sweep holds r rows a chunk
+  const bool shared_rows = NR <= 2 && (k + r) * r > WIDE_ENTRIES && x.nchunk > 1 && k + r <= x.nchunk * r;
+  T *p0 = pball + blockIdx.y * pstride + poff[bi];
+  if (shared_rows) {
+    const int per = (k + r + x.nchunk - 1) / x.nchunk, i0 = min(k + r, ch * per);
+    product(i0, min(per, k + r - i0), p0 + (int64_t)i0 * NR);
+    __threadfence();
+  }
+  if (!last_of_box(cntall + (int64_t)blockIdx.y * nbox + bi, x.nchunk, &s_last)) return;
+  if (shared_rows) {
+    __threadfence();
+    for (int e = tid; e < (k + r) * NR; e += NT) z[e] = __ldcg(p0 + e);
+    __syncthreads();
+  } else {
+    product(0, k + r, z);
+  }
   for (int e = tid; e < (k + r) * NR; e += NT) v[x.ids[e / NR] * NR + e % NR] = e < k * NR ? x.vB[e] - z[e] : z[e];
 }
 
@@ -387,7 +413,8 @@ static void launch_chunks(int mode, const SweepWork<T> &w, int bmax, T *v, int64
   }
   const int64_t vs = n * NR;
   if (mode == SWEEP_SOLVE_FWD)
-    launch_dependent(k_sweep_fwd<T, NR>, grid, smem, st, w.boxes, w.wbox, w.wchunk, v, vs, w.cnt, w.nbox);
+    launch_dependent(k_sweep_fwd<T, NR>, grid, smem, st, w.boxes, w.wbox, w.wchunk, v, vs, w.cnt, w.nbox, w.pbuf,
+                     w.pstride, w.poff);
   else if (mode == SWEEP_SOLVE_BWD)
     launch_dependent(k_sweep_bwd<T, NR>, grid, smem, st, w.boxes, w.wbox, w.wchunk, v, vs, w.cnt, w.nbox, w.pbuf,
                      w.pstride, w.poff);

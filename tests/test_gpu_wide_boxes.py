@@ -44,3 +44,6 @@ def test_wide_boxes(pkg, case):
     assert float(torch.linalg.norm(y - ax) / torch.linalg.norm(ax)) <= 10 * eps
     z = f.solve(y)
     assert float(torch.linalg.norm(z - x) / torch.linalg.norm(x)) <= 10 * eps
+    for m in (1, 2):  # narrow groups: the box's CTAs share the last product
+        z = f.solve(y[:m].contiguous())
+        assert float(torch.linalg.norm(z - x[:m]) / torch.linalg.norm(x[:m])) <= 10 * eps
