@@ -58,7 +58,8 @@ typedef enum { RSS_FP64 = 0, RSS_MIXED = 1 } rss_precision;
 typedef struct rss_mlp rss_mlp; /* rank-proposal network (rss_mlp_create) */
 
 typedef struct {
-  int prec;            /* rss_precision: FP64 everywhere, or an FP32 factor */
+  int prec;            /* rss_precision: FP64 everywhere (direct sums: to
+                          FP64's accuracy), or an FP32 factor */
   int n_proxy;         /* proxy points; 0: 64 (2D) / 512 (3D) (Sec. 4) */
   double proxy_radius; /* in box sides; 0: 2.5 (Sec. 3.2) */
   int use_graphs;      /* 1: each solve with nrhs <= 4 replays a CUDA graph
@@ -268,8 +269,9 @@ rss_status rss_sqrt_apply(const rss_factorization *f, const double *x, double *y
 /* rss_matvec -- y = A x in FP64 with the exact operator being factored:
  * an FFT convolution when the points are the cell centres of an s^dim grid
  * (s a power of two; exact up to FP64 rounding), direct summation over all
- * pairs otherwise (in pairs of FP32 numbers, 48 bits a term, the terms added
- * up in FP64: an error no larger than that of a plain FP64 sum).  Device buffers, n x nrhs column-major. */
+ * pairs otherwise (in sums of three FP32 numbers, about 56 bits a term,
+ * flushed into FP64 sums: an error no larger than that of a plain FP64 sum).
+ * Device buffers, n x nrhs column-major. */
 rss_status rss_matvec(const rss_factorization *f, const double *x, double *y, int nrhs);
 
 /* rss_sync -- wait for the factor's stream, then report an error the device

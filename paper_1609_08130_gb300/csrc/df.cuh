@@ -7,7 +7,9 @@
 // FMA.  The _rn intrinsics keep the compiler from contracting or reassociating
 // them.
 #pragma once
+#ifdef __CUDACC__
 #include <cuda_runtime.h>
+#endif
 
 namespace rss {
 

@@ -209,8 +209,8 @@ template <typename T> int64_t elim_ws_elems(int bmax);
 template <typename T>
 void launch_permute(int dir, const int64_t *perm, const double *in, T *out_or_in, double *out,
                     int64_t n, int nrhs, int nr, cudaStream_t st);
-// y = A x by direct summation in pairs of FP32 numbers (matvec.cu), FP64 in
-// and out.  split: the points' parts (matvec_split, matvec_split_bytes); xbuf:
+// y = A x by direct summation in sums of three FP32 numbers (matvec.cu), FP64
+// in and out.  split: the points' parts (matvec_split, matvec_split_bytes); xbuf:
 // matvec_x_bytes of scratch.
 int64_t matvec_split_bytes(int64_t n, int dim);
 int64_t matvec_x_bytes(int64_t n, int nrhs, int ntile);

@@ -1,28 +1,32 @@
 // matvec.cu -- the exact operator y = A x by direct summation (scattered
-// points), FP64 in and out, evaluated in pairs of FP32 numbers.
+// points), FP64 in and out, evaluated in sums of three FP32 numbers.
 //
 // FP64 arithmetic runs at 2.15 operations per clock and SM here, FP32 at 128:
-// a plain FP64 sum (about 17 FP64 operations a pair of points and column) took
-// 37 ms for a product of 20011 points x 3 columns, 34 ms for 20000 3D points x
-// 2 columns; in this form 4 ms and 2.1 ms, with an error no larger (measured
-// 0.03-1 of the FP64 sum's on 4000-20011 points, against extended precision).
-// A pair of points is about 90 FP32 instructions and 14 per column:
-//   - coordinates are three FP32 parts on fixed grids (24 + 23 bits and the
+// a plain FP64 sum does about 17 FP64 operations a pair of points and column.
+// FP32 numbers in threes (tf.cuh) carry the distance, the kernel and the sums to
+// about 2^-56, so the result's error is that of its last FP64 roundings:
+//   - coordinates are three FP32 parts on fixed grids (24 + 24 bits and the
 //     rest), so differences of the first two parts are exact and the distance
-//     keeps 48 bits however near the points are;
-//   - r^2 = sum of squares in pairs (df.cuh);
-//   - log r^2 table-driven (log_df.cuh), 1 / r by an FP32 seed and one Newton
-//     step in pairs;
-//   - products and sums in pairs, flushed into FP64 every 256 terms.
+//     keeps its bits however near the points are (exceptions below);
+//   - r^2 = sum of squares; log r^2 table-driven (log_tf.cuh), 1 / r by an FP32
+//     seed and a Newton step of second order;
+//   - products and sums, flushed into FP64 every 256 terms.
 // The weight, the kernel's constant and the diagonal term are FP64.  The
 // columns are scaled by powers of two per tile of 256 sources; a tile with
 // a value that is not finite takes plain FP64 arithmetic, and so do points
 // that (nearly) coincide.
+//
+// About 130 FP32 instructions a pair of points and 45 a column.  Two columns of
+// 20000 3D points: plain FP64 34 ms, here 3.6 ms.  Relative error of the
+// kernel's part (diag 0, 64 to 20000 points, right-hand sides of both signs):
+// 1.4e-16 to 2.3e-16, of the FP64 sum 2.8e-16 to 6.3e-15.  Pairs of FP32
+// numbers took 2.1 ms, but left 2.1e-15 to 2.4e-14.
 #include <algorithm>
+#include <vector>
 
-#include "df.cuh"
 #include "internal.h"
-#include "log_df.cuh"
+#include "log_table.h"
+#include "log_tf.cuh"
 
 namespace rss {
 
@@ -30,7 +34,12 @@ namespace {
 
 constexpr int MVT = 256;    // sources per tile, threads per CTA
 constexpr int MV_SHIFT = 40;  // scaled coordinates stay below 2^40
-constexpr float R2_MIN = 0x1p-60f;  // scaled r^2 whose pair would lose its low part
+// Pairs of points with a scaled r^2 below this take FP64 arithmetic: R2_MIN,
+// where the third part would underflow; R2_AXIS for a target with a coordinate
+// below NEAR_AXIS, where a coordinate's last bits may be finer than the 2^-32
+// that its third part holds (2^-72 of the largest coordinate) and matter
+// against a distance below 2^22.
+constexpr float R2_MIN = 0x1p-60f, R2_AXIS = 0x1p44f, NEAR_AXIS = 0x1p23f;
 constexpr int KBAD = 1 << 30;  // column scale of a tile with values that are not finite
 
 __device__ __forceinline__ double pow2(int k) { return __longlong_as_double((long long)(1023 + k) << 52); }
@@ -52,27 +61,27 @@ __device__ __forceinline__ int extent_exp(unsigned long long mx) {
 }
 
 // part p (of 3) of coordinate d at out[(3 d + p) n + i], scaled by 2^(40 - E):
-// multiples of 2^17, then of 2^-6, then the rest; the first CTA also fills the
-// logarithm's tables
+// multiples of 2^17, then of 2^-7 (differences of either are below 2^24 of
+// them), then the rest; the first CTA also fills the logarithm's exponent table
 __global__ void __launch_bounds__(256) k_mv_split(const double *xt, int64_t n, int dim, const unsigned long long *mx,
                                                   LogTables *T, float *out) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int sh = MV_SHIFT - extent_exp(*mx);
-  if (blockIdx.x == 0) log_tables_entry(T, threadIdx.x, 2 * sh);
+  if (blockIdx.x == 0) T->et[threadIdx.x] = log_tables_exponent((int)threadIdx.x - 127 - 2 * sh);
   if (i >= n) return;
   for (int d = 0; d < dim; d++) {
     const double x = xt[i * dim + d] * pow2(sh / 2) * pow2(sh - sh / 2);
-    const double h = rint(x * 0x1p-17) * 0x1p17, l = rint((x - h) * 0x1p6) * 0x1p-6;
+    const double h = rint(x * 0x1p-17) * 0x1p17, l = rint((x - h) * 0x1p7) * 0x1p-7;
     out[(3 * d) * n + i] = (float)h;
     out[(3 * d + 1) * n + i] = (float)l;
     out[(3 * d + 2) * n + i] = (float)((x - h) - l);
   }
 }
 
-// The columns in tree order as pairs, scaled by 2^-k: k a multiple of 64 near
-// the tile's largest exponent (0 for ordinary data).
+// The columns in tree order in three parts (planes of n), scaled by 2^-k: k a
+// multiple of 64 near the tile's largest exponent (0 for ordinary data).
 __global__ void __launch_bounds__(MVT) k_mv_x(const int64_t *perm, const double *xin, int64_t n, int ncol,
-                                              const int64_t *tstart, const int64_t *tend, float2 *xs, int *xk) {
+                                              const int64_t *tstart, const int64_t *tend, float *xs, int *xk) {
   __shared__ unsigned s_e;
   const int q = blockIdx.x, c = blockIdx.y;
   const int64_t i = tstart[q] + threadIdx.x;
@@ -89,13 +98,18 @@ __global__ void __launch_bounds__(MVT) k_mv_x(const int64_t *perm, const double 
   const int k = em == 0x7ff ? KBAD : em == 0 ? 0 : ((em - 1023 + 32 + 1024) >> 6) * 64 - 1024;
   if (threadIdx.x == 0) xk[(int64_t)c * gridDim.x + q] = k;
   if (live) {
-    float2 v = make_float2(0.f, 0.f);
+    Tf v{0.f, 0.f, 0.f};
     if (k != KBAD) {
       const double s = x * pow2(-(k / 2)) * pow2(-(k - k / 2));
-      v.x = (float)s;
-      v.y = (float)(s - (double)v.x);
+      v.h = (float)s;
+      const double r = s - (double)v.h;
+      v.m = (float)r;
+      v.l = (float)(r - (double)v.m);
     }
-    xs[(int64_t)c * n + i] = v;
+    float *o = xs + (int64_t)3 * c * n + i;
+    o[0] = v.h;
+    o[n] = v.m;
+    o[2 * n] = v.l;
   }
 }
 
@@ -106,13 +120,12 @@ __global__ void __launch_bounds__(MVT) k_mv_x(const int64_t *perm, const double 
 template <int DIM, int KIND, int NC>
 __global__ void __launch_bounds__(MVT, NC == 8 ? 2 : 3)
     k_mv(const float *cs, const double *xt, const unsigned long long *mx, KernelParams K, const double *wdof,
-         const int64_t *perm, const double *xin, const float2 *xs, const int *xk, double *yout, int64_t n, int col0,
+         const int64_t *perm, const double *xin, const float *xs, const int *xk, double *yout, int64_t n, int col0,
          int ncol, int ntile, int parts, const int64_t *tstart, const int64_t *tend, const int64_t *sbeg,
          const int64_t *send) {
   __shared__ float sc[3 * DIM][MVT];
-  __shared__ float2 sx[NC][MVT];
-  __shared__ float4 s_lt[KIND == 0 ? 128 : 1];
-  __shared__ float2 s_et[KIND == 0 ? 256 : 1];
+  __shared__ float sx[NC][3][MVT];
+  __shared__ float4 s_lt[KIND == 0 ? LOG_CELLS : 1], s_et[KIND == 0 ? 256 : 1];
   __shared__ double s_red[MVT];
   const int tid = threadIdx.x;
   const int q = blockIdx.x / parts, sub = blockIdx.x % parts;
@@ -127,23 +140,27 @@ __global__ void __launch_bounds__(MVT, NC == 8 ? 2 : 3)
   const int sh = MV_SHIFT - extent_exp(*mx);
   if (KIND == 0) {
     const LogTables *T = reinterpret_cast<const LogTables *>(mx + 2);
-    if (tid < 128) s_lt[tid] = T->lt[tid];
+    for (int e = tid; e < LOG_CELLS; e += MVT) s_lt[e] = T->lt[e];
     s_et[tid] = T->et[tid];
   }
   float xi[3 * DIM];
 #pragma unroll
   for (int d = 0; d < 3 * DIM; d++) xi[d] = cs[(int64_t)d * n + ic];
-  Df acc[NC];
+  float r2min = R2_MIN;
+#pragma unroll
+  for (int d = 0; d < DIM; d++)
+    if (fabsf(xi[3 * d] + xi[3 * d + 1]) < NEAR_AXIS) r2min = R2_AXIS;
+  Tf acc[NC];
   double sum[NC];
   int kc[NC];
 #pragma unroll
-  for (int c = 0; c < NC; c++) acc[c] = Df{0.f, 0.f}, sum[c] = 0.0, kc[c] = 0;
-  // scaled pairs so far into the FP64 sums
+  for (int c = 0; c < NC; c++) acc[c] = Tf{0.f, 0.f, 0.f}, sum[c] = 0.0, kc[c] = 0;
+  // the scaled sums so far into the FP64 ones
   auto flush = [&]() {
 #pragma unroll
     for (int c = 0; c < NC; c++) {
-      sum[c] += ((double)acc[c].h + (double)acc[c].l) * pow2(kc[c] / 2) * pow2(kc[c] - kc[c] / 2);
-      acc[c] = Df{0.f, 0.f};
+      sum[c] += ((double)acc[c].h + ((double)acc[c].m + (double)acc[c].l)) * pow2(kc[c] / 2) * pow2(kc[c] - kc[c] / 2);
+      acc[c] = Tf{0.f, 0.f, 0.f};
     }
   };
   int terms = 0;
@@ -164,12 +181,14 @@ __global__ void __launch_bounds__(MVT, NC == 8 ? 2 : 3)
       for (int d = 0; d < 3 * DIM; d++) sc[d][tid] = cs[(int64_t)d * n + j0 + tid];
 #pragma unroll
       for (int c = 0; c < NC; c++)
-        sx[c][tid] = cb + c < ncol ? xs[(int64_t)(cb + c) * n + j0 + tid] : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int p = 0; p < 3; p++)
+          sx[c][p][tid] = cb + c < ncol ? xs[(int64_t)(3 * (cb + c) + p) * n + j0 + tid] : 0.f;
     }
     __syncthreads();
     const int64_t self64 = i - j0;
     const int self = self64 >= 0 && self64 < lim ? (int)self64 : -1;
-    // source s in plain FP64, in units of the scaled distances as the pairs
+    // source s in plain FP64, in units of the scaled distances as the sums
     auto plain = [&](int s) {
       double r2 = 0.0;
       for (int d = 0; d < DIM; d++) {
@@ -192,37 +211,19 @@ __global__ void __launch_bounds__(MVT, NC == 8 ? 2 : 3)
       for (int c = 0; c < NC; c++) kc[c] = kn[c];
     }
     terms += (lim + parts - 1) / parts;
-    for (int s0 = part; s0 < lim; s0 += 8 * parts) {
 #pragma unroll 2
-      for (int u = 0; u < 8; u++) {
-        const int s = s0 + u * parts;
-        if (s >= lim) break;
-        Df r2;
+    for (int s = part; s < lim; s += parts) {
+      float dx[3 * DIM];
 #pragma unroll
-        for (int d = 0; d < DIM; d++) {
-          // exact differences of the two leading parts
-          const Df t = quick_two_sum(__fadd_rn(xi[3 * d], -sc[3 * d][s]), __fadd_rn(xi[3 * d + 1], -sc[3 * d + 1][s]));
-          const Df z = quick_two_sum(t.h, __fadd_rn(t.l, __fadd_rn(xi[3 * d + 2], -sc[3 * d + 2][s])));
-          const float p = __fmul_rn(z.h, z.h);
-          const float e = __fmaf_rn(2.f * z.h, z.l, __fmaf_rn(z.l, z.l, __fmaf_rn(z.h, z.h, -p)));
-          if (d == 0) {
-            r2 = Df{p, e};
-          } else {
-            const Df w = two_sum(r2.h, p);
-            r2 = Df{w.h, __fadd_rn(w.l, __fadd_rn(r2.l, e))};
-          }
-        }
-        r2 = quick_two_sum(r2.h, r2.l);
-        Df a = KIND == 0 ? log_df(r2, s_lt, s_et) : rsqrt_df(r2);
-        if (r2.h < R2_MIN) {  // the target itself, or a point (nearly) on it
-          a = Df{0.f, 0.f};
-          if (s != self) plain(s);
-        }
-#pragma unroll
-        for (int c = 0; c < NC; c++) acc[c] = add_mul(acc[c], a, Df{sx[c][s].x, sx[c][s].y});
+      for (int d = 0; d < 3 * DIM; d++) dx[d] = __fadd_rn(xi[d], -sc[d][s]);
+      const Tf r2 = dist2_tf<DIM>(dx);
+      Tf a = KIND == 0 ? log_tf(r2, s_lt, s_et) : rsqrt_tf(r2);
+      if (!(r2.h >= r2min)) {  // the target itself, or a point (nearly) on it
+        a = Tf{0.f, 0.f, 0.f};
+        if (s != self) plain(s);
       }
 #pragma unroll
-      for (int c = 0; c < NC; c++) acc[c] = quick_two_sum(acc[c].h, acc[c].l);
+      for (int c = 0; c < NC; c++) add_mul_tf(acc[c], a, Tf{sx[c][0][s], sx[c][1][s], sx[c][2][s]});
     }
   }
   flush();
@@ -328,12 +329,19 @@ int mv_parts(int ntile, int groups) { return (int64_t)ntile * groups * 4 >= 1200
 constexpr int64_t SPLIT_HEAD = 16 + (int64_t)sizeof(LogTables);
 int64_t matvec_split_bytes(int64_t n, int dim) { return SPLIT_HEAD + (int64_t)sizeof(float) * 3 * dim * n; }
 int64_t matvec_x_bytes(int64_t n, int nrhs, int ntile) {
-  return (int64_t)nrhs * (n * (int64_t)sizeof(float2) + ntile * (int64_t)sizeof(int));
+  return (int64_t)nrhs * (n * 3 * (int64_t)sizeof(float) + ntile * (int64_t)sizeof(int));
 }
 
 void matvec_split(const double *x_tree, int64_t n, int dim, void *split, cudaStream_t st) {
   if (n == 0) return;
+  static const std::vector<float> lt = [] {  // made once, never written again
+    std::vector<float> t(4 * LOG_CELLS);
+    for (int i = 0; i < LOG_CELLS; i++) log_table_entry(i, LOG_CELLS, LOG_M, &t[4 * i]);
+    return t;
+  }();
   unsigned long long *mx = static_cast<unsigned long long *>(split);
+  cudaMemcpyAsync(reinterpret_cast<LogTables *>(mx + 2)->lt, lt.data(), sizeof(float4) * LOG_CELLS,
+                  cudaMemcpyHostToDevice, st);
   float *cs = reinterpret_cast<float *>(static_cast<char *>(split) + SPLIT_HEAD);
   cudaMemsetAsync(mx, 0, 16, st);
   const int64_t cnt = n * dim;
@@ -344,7 +352,7 @@ void matvec_split(const double *x_tree, int64_t n, int dim, void *split, cudaStr
 
 template <int DIM, int KIND, int NC>
 static void launch_mv(const float *cs, const double *xt, const unsigned long long *mx, const KernelParams &K,
-                      const double *wdof, const int64_t *perm, const double *xin, const float2 *xs, const int *xk,
+                      const double *wdof, const int64_t *perm, const double *xin, const float *xs, const int *xk,
                       double *yout, int64_t n, int col0, int ncol, int ntile, const int64_t *tstart,
                       const int64_t *tend, const int64_t *sbeg, const int64_t *send, cudaStream_t st) {
   const int groups = std::max(1, (ncol - col0) / NC), parts = mv_parts(ntile, groups);
@@ -360,12 +368,12 @@ void launch_matvec(const double *x_tree, int dim, const KernelParams &K, const d
   if (n == 0 || ntile == 0 || nrhs == 0) return;
   const unsigned long long *mx = static_cast<const unsigned long long *>(split);
   const float *cs = reinterpret_cast<const float *>(static_cast<const char *>(split) + SPLIT_HEAD);
-  float2 *xs = static_cast<float2 *>(xbuf);
-  int *xk = reinterpret_cast<int *>(xs + (int64_t)nrhs * n);
+  float *xs = static_cast<float *>(xbuf);
+  int *xk = reinterpret_cast<int *>(xs + (int64_t)3 * nrhs * n);
   k_mv_x<<<dim3((unsigned)ntile, nrhs), MVT, 0, st>>>(perm, xin, n, nrhs, tstart, tend, xs, xk);
   count_launch();
-  // columns in groups of eight, then four, two or one: the distance and the
-  // kernel cost as much as seven columns' products
+  // columns in groups of eight, then four to one: the distance and the kernel
+  // cost as much as three columns' products
 #define MV(D, KD, N) \
   launch_mv<D, KD, N>(cs, x_tree, mx, K, wdof, perm, xin, xs, xk, yout, n, c, nrhs, ntile, tstart, tend, sbeg, send, st)
 #define MVN(N)                           \
@@ -380,9 +388,12 @@ void launch_matvec(const double *x_tree, int dim, const KernelParams &K, const d
     if (left >= 8) {
       MVN(8);
       c += left / 8 * 8;
-    } else if (left >= 3) {
+    } else if (left >= 4) {
       MVN(4);
       c += 4;
+    } else if (left == 3) {
+      MVN(3);
+      c += 3;
     } else if (left == 2) {
       MVN(2);
       c += 2;
