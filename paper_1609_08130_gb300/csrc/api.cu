@@ -914,11 +914,13 @@ template <typename T> struct Factor : FactorBase {
   DBuf d_mv_split;  // the points in FP32 parts (direct summation only)
   // rank proposal: the network (borrowed during rss_factor only), the
   // features of every box (MLP_NFEAT each, box order) and storage accounting
-  // solve sweeps: work items (box, chunk) of every phase, per-box counters,
-  // partial sums of the backward sweep
-  DBuf d_wbox, d_wchunk, d_poff;
-  mutable DBuf d_wcnt, d_pbuf;
-  mutable int work_groups = 1;  // column groups d_wcnt and d_pbuf hold
+  // sweeps: work items (box, chunk) of every phase, per-box counters and
+  // partial sums.  d_wcnt and d_pbuf serve one group of columns and stay where
+  // they are until rss_free, since a caller may have captured an
+  // rss_solve_noalloc that uses them; calls with several groups have their own.
+  DBuf d_wbox, d_wchunk, d_poff, d_wcnt, d_pbuf;
+  mutable DBuf d_wcnt_wide, d_pbuf_wide;
+  mutable int wide_groups = 0;  // column groups the wide ones hold
   int64_t pbuf_elems = 0;       // partial sums of one group
   const struct MlpModel *mlp = nullptr;
   std::vector<float> feats;
@@ -2142,7 +2144,6 @@ template <typename T> static void run_factor(Factor<T> &F) {
     F.d_wcnt.alloc(sizeof(int) * std::max<size_t>(F.h_boxes.size(), 1), st);
     CK(cudaMemsetAsync(F.d_wcnt.p, 0, sizeof(int) * std::max<size_t>(F.h_boxes.size(), 1), st));
     F.pbuf_elems = std::max<int64_t>(poff.back(), 1);
-    F.work_groups = 1;
     F.d_pbuf.alloc(sizeof(T) * F.pbuf_elems, st);
   }
 
@@ -2256,15 +2257,15 @@ template <typename F> static rss_status guard(F &&fn) {
   }
 }
 
-// Counters and partial sums for `groups` groups of columns.
+// Counters and partial sums for calls with `groups` > 1 groups of columns.  No
+// captured graph of the library holds them (those are of one group).
 template <typename T> static void ensure_groups(const Factor<T> &F, int groups) {
-  if (F.work_groups >= groups) return;
+  if (groups <= 1 || F.wide_groups >= groups) return;
   const size_t nb = sizeof(int) * std::max<size_t>(F.h_boxes.size(), 1) * groups;
-  F.d_wcnt.alloc(nb, F.st);
-  CK(cudaMemsetAsync(F.d_wcnt.p, 0, nb, F.st));
-  F.d_pbuf.alloc(sizeof(T) * (size_t)F.pbuf_elems * groups, F.st);
-  F.work_groups = groups;
-  F.work_gen++;  // captured sweeps hold the old buffers
+  F.d_wcnt_wide.alloc(nb, F.st);
+  CK(cudaMemsetAsync(F.d_wcnt_wide.p, 0, nb, F.st));
+  F.d_pbuf_wide.alloc(sizeof(T) * (size_t)F.pbuf_elems * groups, F.st);
+  F.wide_groups = groups;
 }
 
 // Whether the chunked kernels take groups of nr <= 4 columns of this phase
@@ -2286,9 +2287,10 @@ template <typename T> static int group_columns(const Factor<T> &F, int nrhs) {
 template <typename T>
 static void sweep_phase(const Factor<T> &F, int mode, const Phase &p, T *v, int nr, int groups, cudaStream_t st) {
   if (mode != SWEEP_APPLY_W && chunked<T>(p, nr)) {
+    const bool wide = groups > 1;
     const SweepWork<T> w{ptr<FBox<T>>(F.d_boxes), ptr<int>(F.d_wbox) + p.wfirst, ptr<int>(F.d_wchunk) + p.wfirst,
-                         p.wcount, ptr<int>(F.d_wcnt), (int)F.h_boxes.size(), ptr<T>(F.d_pbuf), F.pbuf_elems,
-                         ptr<int64_t>(F.d_poff)};
+                         p.wcount, ptr<int>(wide ? F.d_wcnt_wide : F.d_wcnt), (int)F.h_boxes.size(),
+                         ptr<T>(wide ? F.d_pbuf_wide : F.d_pbuf), F.pbuf_elems, ptr<int64_t>(F.d_poff)};
     launch_sweep_chunks<T>(mode, w, p.bmax, v, F.n, nr, groups, st);
     return;
   }
