@@ -24,6 +24,7 @@
 
 #include "../../include/rss.h"
 #include "internal.h"
+#include "workspace.h"
 
 namespace rss {
 
@@ -937,11 +938,11 @@ template <typename T> struct Factor : FactorBase {
 };
 
 template <typename T> static void ensure_work(const Factor<T> &F, int nrhs) {
-  if (F.work_nrhs >= nrhs) return;
-  F.d_work.alloc((size_t)std::max<int64_t>(F.n, 1) * nrhs * sizeof(T), F.st);
-  F.d_topwork.alloc((size_t)std::max(F.ntop, 1) * 2 * nrhs * sizeof(T), F.st);
-  F.work_nrhs = nrhs;
-  F.work_gen++;  // captured sweeps hold the old buffers
+  regrow(F.work_nrhs, nrhs, [&] {
+    F.work_gen++;  // captured sweeps hold the old buffers
+    F.d_work.alloc((size_t)std::max<int64_t>(F.n, 1) * nrhs * sizeof(T), F.st);
+    F.d_topwork.alloc((size_t)std::max(F.ntop, 1) * 2 * nrhs * sizeof(T), F.st);
+  });
 }
 
 // Algorithmic work of one launch over boxes [first, first+count):
@@ -2260,12 +2261,13 @@ template <typename F> static rss_status guard(F &&fn) {
 // Counters and partial sums for calls with `groups` > 1 groups of columns.  No
 // captured graph of the library holds them (those are of one group).
 template <typename T> static void ensure_groups(const Factor<T> &F, int groups) {
-  if (groups <= 1 || F.wide_groups >= groups) return;
-  const size_t nb = sizeof(int) * std::max<size_t>(F.h_boxes.size(), 1) * groups;
-  F.d_wcnt_wide.alloc(nb, F.st);
-  CK(cudaMemsetAsync(F.d_wcnt_wide.p, 0, nb, F.st));
-  F.d_pbuf_wide.alloc(sizeof(T) * (size_t)F.pbuf_elems * groups, F.st);
-  F.wide_groups = groups;
+  if (groups <= 1) return;
+  regrow(F.wide_groups, groups, [&] {
+    const size_t nb = sizeof(int) * std::max<size_t>(F.h_boxes.size(), 1) * groups;
+    F.d_wcnt_wide.alloc(nb, F.st);
+    CK(cudaMemsetAsync(F.d_wcnt_wide.p, 0, nb, F.st));
+    F.d_pbuf_wide.alloc(sizeof(T) * (size_t)F.pbuf_elems * groups, F.st);
+  });
 }
 
 // Whether the chunked kernels take groups of nr <= 4 columns of this phase

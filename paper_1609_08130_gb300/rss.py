@@ -43,7 +43,8 @@ def _nvcc():
 def build(force: bool = False) -> str:
     """Compile librss.so in-tree for sm_103a (translation units in parallel)."""
     srcs = [os.path.join(_CSRC, s) for s in SOURCES]
-    deps = srcs + [os.path.join(_CSRC, h) for h in ("common.cuh", "internal.h", "tc.cuh", "df.cuh", "tf.cuh", "lu_inverse.cuh", "log_tf.cuh", "log_table.h")] + \
+    deps = srcs + [os.path.join(_CSRC, h) for h in ("common.cuh", "internal.h", "tc.cuh", "df.cuh", "tf.cuh", "lu_inverse.cuh", "log_tf.cuh",
+                                                     "log_table.h", "workspace.h")] + \
         [os.path.join(_INC, "rss.h")]
     if not force and os.path.exists(LIB_PATH) and \
             os.path.getmtime(LIB_PATH) >= max(os.path.getmtime(d) for d in deps):
