@@ -2275,8 +2275,8 @@ __global__ void __launch_bounds__(NT) k_elim(LevelDev<T> lv, FBox<T> *boxes, con
 }
 
 // ---------------------------------------------------------------------------
-// Elimination, shared-memory form for b small enough: the LU of X_RR is
-// formed in registers by the whole CTA (lu_inverse.cuh), and E = X_JR X_RR^{-1},
+// Elimination, shared-memory form for b small enough: the LU of X_RR and its
+// inverse by the whole CTA (lu_inverse.cuh), and E = X_JR X_RR^{-T},
 // G = X_RR^{-1} X_RJ are produced in chunks of CH rows / columns of J as
 // shared-memory products, written coalesced.  X_RJ is kept in the scratch
 // for the Schur update.
@@ -2387,7 +2387,6 @@ inline size_t elim2_smem(int b, int k, int r) {
   size_t pers = (size_t)k * r * 2 + (size_t)r * (r + 1);
   size_t u1 = (size_t)b * (b + 1);
   size_t u2 = (size_t)ldx * r + (size_t)(CH + 1) * (b + r);
-  if (sizeof(T) == 4) u2 = std::max(u2, (size_t)ldx * r + (size_t)r * (r + 1));  // a copy of X_RR beside its inverse
   size_t nT = pers + (u1 > u2 ? u1 : u2);
   return nT * sizeof(T) + (size_t)(b + 8) * sizeof(int) + 64;
 }
@@ -2396,17 +2395,21 @@ template <typename T, int RB>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (RB == 4 ? 4 : RB == 6 ? 2 : 1) : 1) k_elim2(LevelDev<T> lv, FBox<T> *boxes, const int *box_list, T *scratch,
                                               int64_t sstride, Overflow<T> ovf, int *err, int split, int C) {
   constexpr int CH = ElimChunk<T>::CH;
-  // The matrix is symmetric (both kernels are), so X_RJ = X_JR^T and
-  // G = X_RR^{-1} X_RJ = E^T up to rounding: only X_JR and E are formed and
-  // their transposes written, half the loads and products of a chunk (FP32
-  // elimination of the 512^2 grid 4.77 -> 3.76 ms).
+  // The matrix is symmetric (both kernels are), so X_RJ = X_JR^T up to rounding:
+  // only X_JR is formed and its transpose written, and G = X_RR^{-1} X_RJ is
+  // formed as its transpose E = X_JR X_RR^{-T}, half the loads and products of a
+  // chunk (FP32 elimination of the 512^2 grid 4.77 -> 3.76 ms).  It is the
+  // inverse's transpose that E takes: what the inverse is good for is
+  // X_RR X_RR^{-1} = I, so G solves X_RR G = X_RJ, and E its transpose, while the
+  // product X_RR^{-1} X_RR is off by the condition number more (first-kind
+  // matrices, FP32: apply error 5 times larger with E = X_JR X_RR^{-1}).
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int s_ncode[27], s_ncell[27], s_nstart[28], s_nact[27], s_nn, s_ok;
   __shared__ int64_t s_off_in[27];
   __shared__ int s_ld_in[27];
   __shared__ int64_t s_rb[ElimChunk<T>::CH];
   __shared__ int s_rl[ElimChunk<T>::CH];
-  __shared__ LuInvShared<T> s_lu;
+  __shared__ std::conditional_t<sizeof(T) == 4, LuShared<>, LuPivots> s_lu;
   // C CTAs per box (split mode only): CTA 0 also does the LU, X_RR^{-1} and
   // the box's records; every CTA forms its share of the chunks of J
   const int q = blockIdx.x / C, cta = blockIdx.x % C;
@@ -2421,12 +2424,11 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (RB == 4 ? 4 : RB == 6 ? 
   T *LU = XSR + (size_t)k * r;                      // r x r row-major, ld r+1
   T *U0 = LU + (size_t)r * ldl;                     // union region
   T *Ab = U0;                                       // A_BB in (S|R) order, column-major, ld b+1
-  T *Xi = U0;                                       // X_RR^{-1}, column-major, ld ldx (after the LU)
+  T *Xi = U0;                                       // X_RR^{-1}, row-major, ld ldx (after the LU)
   T *rawJ = Xi + (size_t)ldx * r;                   // CH rows of J x b  (al + p*(CH+1)) -> X_JR in place
   T *ec = rawJ + (size_t)(CH + 1) * b;              // the chunk of E (al + ri*(CH+1))
   const size_t u1 = (size_t)b * ldb;
-  size_t u2 = (size_t)ldx * r + (size_t)(CH + 1) * (b + r);
-  if (sizeof(T) == 4) u2 = max(u2, (size_t)ldx * r + (size_t)r * ldl);  // the copy of X_RR
+  const size_t u2 = (size_t)ldx * r + (size_t)(CH + 1) * (b + r);
   int *sloc = reinterpret_cast<int *>(U0 + (u1 > u2 ? u1 : u2));
 
   if (warp == 0) {  // the 3^d neighbourhood, a lane per cell
@@ -2545,26 +2547,28 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (RB == 4 ? 4 : RB == 6 ? 
   __syncthreads();
   if (cta == 0) {
   // LU factors and inverse of X_RR; the inverse over A_BB, which is no
-  // longer needed
-  {
-    T *xi = Xi;
-    const int ld = ldx;
-    T *Xc = rawJ;  // a copy of X_RR for the correction
-    if constexpr (sizeof(T) == 4)
-      for (int e = tid; e < r * ldl; e += NT) Xc[e] = LU[e];
-    lu_inverse<T, RB>(r, LU, ldl, s_lu, err, [&](int i, int cc, T v) { xi[i + (size_t)cc * ld] = v; });
-    if constexpr (sizeof(T) == 4) newton_inverse<RB>(r, Xc, ldl, Xi, ldx);
+  // longer needed.  Four lanes a column in FP32, two in FP64 (its unit is the
+  // bound: more would repeat the divisions and the sums over the lanes)
+  const int *lp = s_lu.piv;
+  const T *lu = LU;
+  const int ll = ldl;
+  if constexpr (sizeof(T) == 4) {
+    lu_registers<RB>(r, LU, ldl, s_lu, err);
+    inverse_columns<T, NT / 32, 4>(r, lp, [&](int i) { return lu + lp[i] * ll; }, Xi, ldx);
+  } else {
+    lu_shared<T, NT / 32>(r, LU, ldl, s_lu.piv, err);
+    inverse_columns<T, NT / 32, 2>(r, lp, [&](int i) { return lu + i * ll; }, Xi, ldx);
   }
   for (int e = tid; e < r * r; e += NT) {
     int qi, ri;
     fdr.divmod(e, qi, ri);
-    fb.LU[e] = LU[s_lu.piv[qi] * ldl + ri];
+    fb.LU[e] = LU[(sizeof(T) == 4 ? lp[qi] : qi) * ldl + ri];
   }
   for (int i = tid; i < r; i += NT) fb.piv[i] = s_lu.piv[i];
   for (int e = tid; e < r * r; e += NT) {
     int qi, ri;
     fdr.divmod(e, qi, ri);
-    fb.Xi[e] = Xi[ri + (size_t)qi * ldx];
+    fb.Xi[e] = Xi[qi + (size_t)ri * ldx];
   }
   }  // cta == 0
   T *Xrj_out = scratch + (int64_t)q * sstride;  // r x nj, for the Schur update
@@ -2631,7 +2635,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (RB == 4 ? 4 : RB == 6 ? 
       __syncthreads();
       continue;
     }
-    // E chunk = X_JR chunk * X_RR^{-1}, and G's columns
+    // E chunk = X_JR chunk * X_RR^{-T}, and G's columns
     {
       smem_gemm<T, 1>(na, r, r, rawJ + (size_t)k * (CH + 1), 1, CH + 1, Xi, ldx,
                       [&](int al, int ri, T v) { ec[al + ri * (CH + 1)] = v; });
@@ -2668,16 +2672,15 @@ template int64_t elim_smem_bytes<float>(int, int, int);
 template int64_t elim_smem_bytes<double>(int, int, int);
 
 // Elements of T the large-box elimination needs per box beyond X_RJ.
-// k_elim's LU (r x (r+1)) and pivots, or k_elim_lu's X_RR (r x r), r <= bmax;
-// k_elim_gj's X_RR, its inverse and the inverse's residual
+// k_elim's LU (r x (r+1)) and pivots, or k_elim_lu's and k_elim_lur's X_RR
+// (r x r), r <= bmax
 template <typename T> int64_t elim_ws_elems(int bmax) {
-  const int64_t gj = sizeof(T) == 4 && bmax > 128 && bmax <= 224 ? 2 * (int64_t)bmax * bmax : 0;
-  return (int64_t)bmax * (bmax + 1) + (int64_t)bmax + 64 + gj;
+  return (int64_t)bmax * (bmax + 1) + (int64_t)bmax + 64;
 }
 template int64_t elim_ws_elems<float>(int);
 template int64_t elim_ws_elems<double>(int);
 
-// E = X_JR X_RR^{-1} (nj x r) and G = E^T (see k_elim2) for the boxes of a
+// E = X_JR X_RR^{-T} (nj x r) and G = E^T (see k_elim2) for the boxes of a
 // phase whose X_RJ = X_JR^T (r x nj, ld r) is in the scratch: blockIdx.x = box
 // of the phase, blockIdx.y = a 64 x 64 output tile of E; X_RR^{-1} is in the
 // factor (r x r, column-major).  The inner dimension is staged 64 (FP32) or
@@ -2708,7 +2711,8 @@ __global__ void __launch_bounds__(NT) k_elim_gemm(const FBox<T> *boxes, const in
     for (int e = tid; e < KC * 64; e += NT) {
       const int l2 = e % KC, jj = e / KC;  // consecutive inner index
       As[l2 * LD + jj] = (i0 + jj < nj && l2 < kw) ? Xrj[(l0 + l2) + (int64_t)(i0 + jj) * r] : (T)0;
-      Bs[l2 * LD + jj] = (l2 < kw && j0 + jj < r) ? Xi[(l0 + l2) + (int64_t)(j0 + jj) * r] : (T)0;
+      const int j2 = e % 64, l3 = e / 64;  // consecutive rows of X_RR^{-1}
+      Bs[l3 * LD + j2] = (l3 < kw && j0 + j2 < r) ? Xi[(j0 + j2) + (int64_t)(l0 + l3) * r] : (T)0;
     }
     __syncthreads();
 #pragma unroll 4
@@ -3089,30 +3093,25 @@ __global__ void __launch_bounds__(NLU) k_elim_lu(LevelDev<T> lv, FBox<T> *boxes,
   if (tid == 0) lv.act_cnt[c] = k;
 }
 
-// LU factors of X_RR and its inverse in registers (lu_inverse.cuh, 32 x 32
-// threads) for FP32 boxes of 129..224 DOFs, with the box's skeleton list; the
-// inverse goes to the workspace after X_RR for the Newton step.  Bound: the
-// chain of r steps.  32^3 grid, r = 175: 430 us with 7 x 7 entries a thread (which
-// spill), about 280 us with the 6 x 6 of boxes with r <= 192, and 75 us for the
-// Newton step; 550 us blocked in shared memory (elimination class 7.0 -> 5.3 ms).
-constexpr int GJ_MAX = 224;
+// LU factors of X_RR in registers (lu_inverse.cuh, 32 x 32 threads) for FP32
+// boxes of 129..224 DOFs, with the box's skeleton list.  Bound: the chain of r
+// steps.
+constexpr int LUR_MAX = 224;
 template <int RB>
-__global__ void __launch_bounds__(1024) k_elim_gj(LevelDev<float> lv, FBox<float> *boxes, const int *box_list,
-                                                  float *scratch, int64_t sstride, int64_t ws_off, int *err,
-                                                  int rmin, int rmax) {
+__global__ void __launch_bounds__(1024) k_elim_lur(LevelDev<float> lv, FBox<float> *boxes, const int *box_list,
+                                                   const float *scratch, int64_t sstride, int64_t ws_off, int *err,
+                                                   int rmin, int rmax) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ LuInvShared<float, 32 * RB> s_lu;
+  __shared__ LuShared<32 * RB> s_lu;
   FBox<float> &fb = boxes[box_list[blockIdx.x]];
   const int r = fb.r, k = fb.k, tid = threadIdx.x, ldl = r + 1;
   if (r < rmin || r > rmax) return;
   float *X = reinterpret_cast<float *>(smem_raw);
   const float *M = scratch + (int64_t)blockIdx.x * sstride + ws_off;  // X_RR, column-major
-  float *V = const_cast<float *>(M) + (int64_t)r * r;                 // its inverse, column-major
   if (r > 0) {
     for (int e = tid; e < r * r; e += 1024) X[(e % r) * ldl + e / r] = M[e];
     __syncthreads();
-    lu_inverse<float, RB, 32, 32 * RB>(r, X, ldl, s_lu, err,
-                                       [&](int i, int c, float v) { V[i + (int64_t)c * r] = v; });
+    lu_registers<RB, 32, 32 * RB>(r, X, ldl, s_lu, err);
     for (int e = tid; e < r * r; e += 1024) fb.LU[e] = X[s_lu.piv[e / r] * ldl + e % r];
     for (int i = tid; i < r; i += 1024) fb.piv[i] = s_lu.piv[i];
   }
@@ -3127,53 +3126,25 @@ __global__ void __launch_bounds__(1024) k_elim_gj(LevelDev<float> lv, FBox<float
   if (tid == 0) lv.act_cnt[fb.cell] = k;
 }
 
-// The Newton step of those inverses (newton_inverse's, 64 x 64 tiles over the
-// phase): pass 0 R = I - A X after X in the workspace, pass 1 X + X R to the
-// factor.
-template <int PASS>
-__global__ void __launch_bounds__(NT) k_elim_newton(const FBox<float> *boxes, const int *box_list, float *scratch,
-                                                    int64_t sstride, int64_t ws_off, int tr) {
-  constexpr int KC = 64, LD = 64 + 1;
-  __shared__ float As[KC * LD], Bs[KC * LD];
+// The inverses of those boxes, INV_COLS columns a CTA (grid.y), sixteen lanes a
+// column: L\U in shared memory, the columns beside it, 16 banks apart.
+constexpr int INV_COLS = 16;
+__host__ __device__ inline int inv_ld(int r) { return (r + 31) / 32 * 32 + 16; }
+__global__ void __launch_bounds__(NT) k_elim_inv(const FBox<float> *boxes, const int *box_list) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
   const FBox<float> &fb = boxes[box_list[blockIdx.x]];
-  const int r = fb.r, i0 = (blockIdx.y % tr) * 64, j0 = (blockIdx.y / tr) * 64;
-  if (i0 >= r || j0 >= r) return;
-  const int64_t rr = (int64_t)r * r;
-  float *W = scratch + (int64_t)blockIdx.x * sstride + ws_off;
-  const float *A = PASS == 0 ? W : W + rr, *B = PASS == 0 ? W + rr : W + 2 * rr;
-  const int tid = threadIdx.x, ti = tid & 15, tj = tid >> 4;
-  float acc[4][4] = {};
-  for (int l0 = 0; l0 < r; l0 += KC) {
-    const int kw = min(KC, r - l0);
+  const int r = fb.r, c0 = blockIdx.y * INV_COLS, tid = threadIdx.x;
+  if (c0 >= r) return;
+  float *LU = reinterpret_cast<float *>(smem_raw), *x = LU + r * r;
+  const int ld = inv_ld(r);
 #pragma unroll 8
-    for (int e = tid; e < KC * 64; e += NT) {
-      const int ii = e & 63, ll = e >> 6;
-      As[ll * LD + ii] = i0 + ii < r && ll < kw ? A[(i0 + ii) + (int64_t)(l0 + ll) * r] : 0.f;
-      Bs[ii * LD + ll] = ii < kw && j0 + ll < r ? B[(l0 + ii) + (int64_t)(j0 + ll) * r] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int u = 0; u < kw; u++) {
-      float av[4], bv[4];
-#pragma unroll
-      for (int x = 0; x < 4; x++) av[x] = As[u * LD + ti + 16 * x], bv[x] = Bs[u * LD + tj + 16 * x];
-#pragma unroll
-      for (int x = 0; x < 4; x++)
-#pragma unroll
-        for (int y = 0; y < 4; y++) acc[x][y] = fmaf(av[x], bv[y], acc[x][y]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int x = 0; x < 4; x++)
-#pragma unroll
-    for (int y = 0; y < 4; y++) {
-      const int i = i0 + ti + 16 * x, j = j0 + tj + 16 * y;
-      if (i >= r || j >= r) continue;
-      const int64_t e = i + (int64_t)j * r;
-      if (PASS == 0) W[2 * rr + e] = (i == j ? 1.f : 0.f) - acc[x][y];
-      else fb.Xi[e] = W[rr + e] + acc[x][y];
-    }
+  for (int e = tid; e < r * r; e += NT) LU[e] = fb.LU[e];
+  __syncthreads();
+  const int iw = c0 + 2 * (tid >> 5), q = tid / INV_COLS, i0 = c0 + q;
+  solve_columns<float, 16>(r, i0, min(iw, r), i0 < r, [&](int i) { return LU + i * r; }, x + q * ld, 1);
+  __syncthreads();
+  for (int c = 0; c < min(INV_COLS, r - c0); c++)
+    for (int i = tid; i < r; i += NT) fb.Xi[i + (int64_t)fb.piv[c0 + c] * r] = x[c * ld + i];
 }
 
 // Shape of the next k_elim2 launch on this thread: (split << 4) | CTAs per
@@ -3204,12 +3175,13 @@ void launch_elim(const LevelDev<T> &lv, FBox<T> *boxes, const int *box_list, int
     for (int r = 0; r <= bmax; r++) worst = std::max(worst, elim2_smem<T>(bmax, bmax - r, r));
     // boxes of up to 128 DOFs (wider ones take the blocked LU below)
     if (worst <= (size_t)(220 << 10) && bmax <= 128) {
-      // registers per thread of the LU: 16, 36 or 64 entries of X_RR (r <= b)
+      // registers per thread of the FP32 LU: 16, 36 or 64 entries of X_RR (r <= b)
       auto run = [&](auto kern) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)worst);
         kern<<<nbox * C, NT, worst, st>>>(lv, boxes, box_list, scratch, scratch_stride, ovf, err, split, C);
       };
-      if (bmax <= 64) run(k_elim2<T, 4>);
+      if constexpr (sizeof(T) == 8) run(k_elim2<T, 0>);
+      else if (bmax <= 64) run(k_elim2<T, 4>);
       else if (bmax <= 96) run(k_elim2<T, 6>);
       else run(k_elim2<T, 8>);
       count_launch();
@@ -3232,7 +3204,7 @@ void launch_elim(const LevelDev<T> &lv, FBox<T> *boxes, const int *box_list, int
       k_elim<T><<<nbox * Cb, NT, 0, st>>>(lv, boxes, box_list, scratch, scratch_stride, ws_off, ovf, err, Cb, 1);
       k_elim_xrr<T><<<dim3(nbox, tr * tr), NT, 0, st>>>(lv, boxes, box_list, scratch, scratch_stride, ws_off, tr);
       if constexpr (std::is_same<T, float>::value) {
-        if (bmax <= GJ_MAX) {
+        if (bmax <= LUR_MAX) {
           const size_t xsm = (size_t)bmax * (bmax + 1) * sizeof(float);
           // boxes by their own r: 7 x 7 entries do not quite fit the registers
           // of 1024 threads
@@ -3241,11 +3213,12 @@ void launch_elim(const LevelDev<T> &lv, FBox<T> *boxes, const int *box_list, int
             kern<<<nbox, 1024, xsm, st>>>(lv, boxes, box_list, scratch, scratch_stride, ws_off, err, rmin, rmax);
             count_launch();
           };
-          run(k_elim_gj<6>, 0, 192);
-          if (bmax > 192) run(k_elim_gj<7>, 193, GJ_MAX);
-          k_elim_newton<0><<<dim3(nbox, tr * tr), NT, 0, st>>>(boxes, box_list, scratch, scratch_stride, ws_off, tr);
-          k_elim_newton<1><<<dim3(nbox, tr * tr), NT, 0, st>>>(boxes, box_list, scratch, scratch_stride, ws_off, tr);
-          count_launch(4);
+          run(k_elim_lur<6>, 0, 192);
+          if (bmax > 192) run(k_elim_lur<7>, 193, LUR_MAX);
+          const size_t ism = ((size_t)bmax * bmax + (size_t)INV_COLS * inv_ld(bmax)) * sizeof(float);
+          cudaFuncSetAttribute(k_elim_inv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ism);
+          k_elim_inv<<<dim3(nbox, (bmax + INV_COLS - 1) / INV_COLS), NT, ism, st>>>(boxes, box_list);
+          count_launch(3);
           launch_elim_gemm<T>(boxes, box_list, nbox, scratch, scratch_stride, tiles_e, tr, st);
           return;
         }

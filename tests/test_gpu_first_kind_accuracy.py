@@ -1,0 +1,49 @@
+"""FP32 factors of first-kind matrices (diag 0): the blocks X_RR are indefinite
+and ill-conditioned, so the factor is only as good as E X_RR = X_JR and
+X_RR G = X_RJ hold.  Apply errors scatter by a factor of a few from problem to
+problem, so their geometric mean over a set is compared with that of the
+general kernels (the forced large-box path: one CTA per box, LU and
+substitution row by row) on the same problems.
+
+Tolerance: the two differ in rounding only.  The logarithm of an error scatters
+by about 1 between problems and kernels, so the mean over 24 differs by
+sqrt(2 / 24) = 0.3 (12: 0.4); a factor of 2.5 is three (two) of these, and a
+set whose inverses are not solved column by column was 5 times off."""
+import numpy as np
+import pytest
+
+from paper_1609_08130_gb300 import inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_1609_08130_gb300 as p
+    p.build()
+    return p
+
+
+def _mean_error(pkg, sets, leaf, flags):
+    e = []
+    for seed, n in sets:
+        pts = torch.from_numpy(inputs.random_points(seed, n, 2)).cuda()
+        f = pkg.Factorization(pts, 0, 1e-6, leaf=leaf, prec=pkg.MIXED, diag=0.0, flags=flags)
+        x = torch.from_numpy(inputs.rhs(seed + 1, n, 2)).cuda()
+        ax = f.matvec(x)
+        e.append(float(torch.linalg.norm(f.apply(x) - ax) / torch.linalg.norm(ax)))
+    return float(np.exp(np.mean(np.log(e))))
+
+
+@pytest.mark.parametrize("leaf,sizes", [(32, [1500 + 97 * i for i in range(24)]), (60, [3000 + 131 * i for i in range(24)]),
+                                        (200, [2600 + 61 * i for i in range(12)])])
+@pytest.mark.parametrize("flags", [0, 4])
+def test_apply_error_is_that_of_the_general_kernels(pkg, leaf, sizes, flags):
+    sets = [(200 + 2 * i, n) for i, n in enumerate(sizes)]
+    new = _mean_error(pkg, sets, leaf, flags)
+    general = _mean_error(pkg, sets, leaf, flags | pkg.rss.FLAG_LARGE_BOX_PATH)
+    print("leaf %d flags %d: %.2e, general %.2e" % (leaf, flags, new, general))
+    assert new <= 2.5 * general, (new, general)
