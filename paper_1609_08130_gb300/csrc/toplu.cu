@@ -45,6 +45,15 @@ template <typename T> struct alignas(16) Pack {
   T x[N];
 };
 
+// A magnitude's order as 32 bits, NaN above infinity: FP32 entries as they are,
+// FP64 ones by their upper word (20 bits of the mantissa, the whole range of the
+// exponent; a conversion to FP32 would make zeros of what is below 1e-45 and
+// infinities of what is above 3e38), a zero below every other number.
+__device__ __forceinline__ unsigned pivot_key(float v) { return __float_as_uint(v) & 0x7fffffffu; }
+__device__ __forceinline__ unsigned pivot_key(double v) {
+  return ((unsigned)__double2hiint(v) & 0x7fffffffu) | (__double2loint(v) != 0);
+}
+
 // a panel's row moves: position dst[e] (from the panel's first row) takes the
 // row that was at src[e]
 struct Moves {
@@ -54,7 +63,7 @@ struct Moves {
 }  // namespace
 
 // Panel of NB columns at kb, rows kb.. n-1, thread t holding rows t + PT q.
-// Pivot: largest |entry| (compared in FP32), rows moved at the end as the
+// Pivot: largest |entry| (by pivot_key), rows moved at the end as the
 // sequence of interchanges would.
 template <typename T, int NB, int RPT>
 __global__ void __launch_bounds__(PT) k_lu_panel(T *LUall, const int64_t *loff, const int *tn, int *pivall,
@@ -93,7 +102,7 @@ __global__ void __launch_bounds__(PT) k_lu_panel(T *LUall, const int64_t *loff, 
 #pragma unroll
       for (int q = 0; q < RPT; q++)
         if (!(used >> q & 1)) {
-          const unsigned k = __float_as_uint((float)a[q][j]) & 0x7fffffffu;
+          const unsigned k = pivot_key(a[q][j]);
           if (qb < 0 || k > key) key = k, qb = q;
         }
       // a thread with no row left offers nothing (zero keys of real rows win)
