@@ -179,8 +179,9 @@ void sweep_chunk_attributes();
 // Set the shared-memory attributes of every sweep kernel on the current device.
 void sweep_kernel_attributes();
 // Top blocks: mode 0 solves with the LU factors or, with Winv = U^{-1} L^{-1}
-// and groups of at most 4 columns, multiplies by it; mode 1 multiplies by the
-// block.
+// and groups of at most 4 columns, multiplies by it (and, several problems,
+// several groups or orders past 1024, corrects the result by its residual);
+// mode 1 multiplies by the block.
 template <typename T>
 void launch_top(int mode, const T *LU, const int64_t *loff, const int *piv, const int64_t *top, const int64_t *toff,
                 const int *tn, int nprob, int ntop_total, T *v, int64_t n, int nr, int groups, T *work,

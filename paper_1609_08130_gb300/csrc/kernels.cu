@@ -3973,8 +3973,8 @@ __global__ void __launch_bounds__(256) k_top_mul_wide(const T *LUall, const int6
   }
 }
 
-// y = P v_top (the pivoted gather), then v_top = W y with one warp per row,
-// all problems' rows in one grid; grid.y: groups of NR columns.
+// y = P v_top (the pivoted gather), then products with one warp per row, all
+// problems' rows in one grid; grid.y: groups of NR columns.
 template <typename T, int NR>
 __global__ void __launch_bounds__(256) k_top_gather(const int *piv, const int64_t *top, const int64_t *toff, int nprob,
                                                     int ntot, const T *v, int64_t vstride, T *y, int64_t wstride) {
@@ -3985,32 +3985,55 @@ __global__ void __launch_bounds__(256) k_top_gather(const int *piv, const int64_
 #pragma unroll
   for (int c = 0; c < NR; c++) y[blockIdx.y * wstride + (int64_t)e * NR + c] = x[c];
 }
-template <typename T, int NR>
-__global__ void __launch_bounds__(256) k_top_gemv(const T *Wall, const int64_t *loff, const int64_t *topall,
-                                                  const int64_t *toff, int nprob, int ntot, const T *y,
-                                                  int64_t wstride, T *v, int64_t vstride) {
+// The products of a solve: rows of W (row-major, as L\U) against the gathered
+// y, or of L\U against the solution so far.  z: beside y in the work array.
+//   TOP_SOLVE    v_top = W y
+//   TOP_FIRST    z = W y
+//   TOP_U        v_top = U z
+//   TOP_RESIDUAL y -= L v_top
+//   TOP_CORRECT  v_top = z + W y
+// A product with the inverse leaves a forward error some times that of
+// triangular solves when the block is ill-conditioned (first-kind matrices,
+// n = 1500 and 2000: FP64 4.2e-13 and 2.8e-13 against 6.5e-14 and 3.9e-14, FP32
+// 2.0e-4 against 5.3e-5 at 1500), so where those were taken before, the
+// solution is corrected once by its residual L U z - y: three launches more
+// instead of 2 n row steps.
+enum { TOP_SOLVE, TOP_FIRST, TOP_U, TOP_RESIDUAL, TOP_CORRECT };
+template <typename T, int NR, int STEP>
+__global__ void __launch_bounds__(256) k_top_gemv(const T *Aall, const int64_t *loff, const int64_t *topall,
+                                                  const int64_t *toff, int nprob, int ntot, T *y, int64_t wstride,
+                                                  T *v, int64_t vstride) {
   const int lane = threadIdx.x & 31, e = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (e >= ntot) return;
   const int p = problem_of(toff, nprob, e);
   const int64_t o = toff[p];
-  const int n = (int)(toff[p + 1] - o);
-  y += blockIdx.y * wstride + o * NR;
+  const int n = (int)(toff[p + 1] - o), i = (int)(e - o);
+  y += blockIdx.y * wstride;
   v += blockIdx.y * vstride;
-  const T *Wi = Wall + loff[p] + (int64_t)(e - o) * n;
+  T *z = y + (int64_t)ntot * NR;
+  const T *Ai = Aall + loff[p] + (int64_t)i * n;
   T acc[NR];
 #pragma unroll
   for (int c = 0; c < NR; c++) acc[c] = (T)0;
+  const int l0 = STEP == TOP_U ? i : 0, l1 = STEP == TOP_RESIDUAL ? i : n;
 #pragma unroll 4
-  for (int kk = lane; kk < n; kk += 32) {
-    const T w = Wi[kk];
+  for (int l = l0 + lane; l < l1; l += 32) {
+    const T w = Ai[l];
+    const T *x = STEP == TOP_RESIDUAL ? v + topall[o + l] * NR : (STEP == TOP_U ? z : y) + (o + l) * NR;
 #pragma unroll
-    for (int c = 0; c < NR; c++) acc[c] += w * y[kk * NR + c];
+    for (int c = 0; c < NR; c++) acc[c] += w * x[c];
   }
 #pragma unroll
   for (int c = 0; c < NR; c++) acc[c] = warp_sum(acc[c]);
-  if (lane == 0)
+  if (lane == 0) {
+    T *ve = v + topall[e] * NR, *ye = y + (int64_t)e * NR, *ze = z + (int64_t)e * NR;
 #pragma unroll
-    for (int c = 0; c < NR; c++) v[topall[e] * NR + c] = acc[c];
+    for (int c = 0; c < NR; c++) {
+      if (STEP == TOP_FIRST) ze[c] = acc[c];
+      else if (STEP == TOP_RESIDUAL) ye[c] -= acc[c] + ve[c];  // L has a unit diagonal
+      else ve[c] = STEP == TOP_CORRECT ? ze[c] + acc[c] : acc[c];
+    }
+  }
 }
 
 template <typename T, int NR>
@@ -4021,12 +4044,24 @@ static void launch_top_nr(int mode, const T *LU, const int64_t *loff, const int 
   if (mode == 0) {
     k_top_gather<T, NR><<<dim3((unsigned)((ntop + 255) / 256), groups), 256, 0, st>>>(piv, top, toff, nprob, ntop, v,
                                                                                      vstride, work, wstride);
-    k_top_gemv<T, NR><<<rows, 256, 0, st>>>(Winv, loff, top, toff, nprob, ntop, work, wstride, v, vstride);
+    auto run = [&](auto kern, const T *A) {
+      kern<<<rows, 256, 0, st>>>(A, loff, top, toff, nprob, ntop, work, wstride, v, vstride);
+      count_launch();
+    };
+    if (nprob == 1 && ntop <= 1024 && groups == 1) {
+      run(k_top_gemv<T, NR, TOP_SOLVE>, Winv);
+    } else {
+      run(k_top_gemv<T, NR, TOP_FIRST>, Winv);
+      run(k_top_gemv<T, NR, TOP_U>, LU);
+      run(k_top_gemv<T, NR, TOP_RESIDUAL>, LU);
+      run(k_top_gemv<T, NR, TOP_CORRECT>, Winv);
+    }
+    count_launch();
   } else {
     for (int half = 0; half < 2; half++)
       k_top_mul<T, NR><<<rows, 256, 0, st>>>(half, LU, loff, piv, top, toff, nprob, ntop, v, vstride, work, wstride);
+    count_launch(2);
   }
-  count_launch(2);
 }
 
 template <typename T>
