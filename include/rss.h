@@ -409,13 +409,12 @@ rss_status rss_box_features(const rss_factorization *f, float *feat, int32_t *ra
  * fastest for the rest of the process and re-runs it, so factorizations
  * with the same key compute the same result.  Disabled per factorization by
  * RSS_FLAG_NO_AUTOTUNE.  *nbytes in/out as in rss_tree_query.
- * An FP32 factor with eps >= 5e-7 and boxes of at most 512 DOFs has one more
- * form of the ID, from the rows' exact Gram matrix on the tensor cores (the
- * same truncation, ranks equal up to ties): it is timed once per key beside
- * these shapes and taken where it is faster than all of them.  It is not in
- * the table; a shape fixed by rss_autotune_set is always used as set.  With
- * RSS_FLAG_NO_AUTOTUNE, and for boxes wider than 256, such a factor takes it
- * without timing. */
+ * An FP32 factor with eps >= 5e-7 has one more form of the ID, from the rows'
+ * exact Gram matrix on the tensor cores (the same truncation, ranks equal up
+ * to ties).  It takes it on every level whose widest box has 13 to 512 DOFs,
+ * with or without a table: a rule of sizes, so that no timing and no table
+ * changes the factor's form.  The table's shapes are what it takes on the other
+ * levels, and what factors of smaller eps and FP64 factors take. */
 rss_status rss_autotune_table(int32_t *buf, size_t *nbytes);
 
 /* rss_autotune_set -- fix the shape used for one key (e.g. a table saved

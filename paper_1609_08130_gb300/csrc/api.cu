@@ -1160,17 +1160,15 @@ static int shape_hint(int c) {
 struct TuneEntry {
   int shape;            // index into kTuneShapes
   float us[kNShapes];   // time of each candidate, microseconds; 0 if not a candidate
-  float gram_us;        // time of the Gram form on the same phase; 0 if not timed
-  bool pinned;          // set by the caller (rss_autotune_set): this shape and no other
 };
 static std::mutex g_tune_m;
 static std::map<std::tuple<int, int, int>, TuneEntry> g_tune;
 
-// gram: the exact-Gram form of the ID (id_gram.cu), when the factor may take
-// it; timed once per key beside the Householder shapes and used where it is
-// faster than all of them (a 512^2 grid's leaf phase of 1024 boxes 0.27 ms
-// against 1.2 ms, its phases of 4-64 boxes 0.09 against 0.4 ms), unless the
-// caller pinned a shape.  The widths that have no key take it by rule.
+// gram: the exact-Gram form of the ID (id_gram.cu), where the factor takes it
+// (run_factor's rule): by sizes and tolerance only, whatever the table holds, so
+// that every process takes it for the same phases and a table saved in one and
+// set in another gives the same factor.  A key is timed all the same when it is
+// first met, for the factors of smaller tolerances that share it.
 template <typename T, typename Launch, typename Gram>
 static void tuned_id_launch(Factor<T> &F, int bmax, int nbox, Launch &&launch, bool have_gram, Gram &&gram) {
   const bool tunable = bmax > 0 && bmax <= 256 && !(F.flags & RSS_FLAG_NO_AUTOTUNE);
@@ -1187,56 +1185,49 @@ static void tuned_id_launch(Factor<T> &F, int bmax, int nbox, Launch &&launch, b
   while ((2 << bucket) <= nbox) bucket++;
   const int width = bmax <= 64 ? 64 : (bmax <= 128 ? 128 : 256);
   const auto key = std::make_tuple((int)sizeof(T), width, bucket);
-  TuneEntry te{-1, {}, 0.f, false};
+  int shape = -1;
   {
     std::lock_guard<std::mutex> lk(g_tune_m);
     auto it = g_tune.find(key);
-    if (it != g_tune.end()) te = it->second;
+    if (it != g_tune.end()) shape = it->second.shape;
   }
-  const bool time_gram = have_gram && !te.pinned && te.gram_us == 0.f;
-  if (te.shape < 0 || time_gram) {
+  if (shape < 0) {
+    TuneEntry te{-1, {}};
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
-    auto timed = [&](auto &&fn) {
+    float best = 0.f;
+    for (int ci = 0; ci < kNShapes; ci++) {
+      const int tpc = kTuneShapes[ci][0], g = kTuneShapes[ci][1], ctas = kTuneShapes[ci][2];
+      if (!shape_fits(width, tpc, g, kTuneShapes[ci][3])) continue;  // the kernels' thread limits
+      if (ctas > 1 && width == 256 && tpc != 2) continue;  // the widest class: two threads per column
+      set_id_groups(shape_hint(ci));
       float ms = 0.f;
       for (int rep = 0; rep < 2; rep++) {  // the second launch is timed
         CK(cudaEventRecord(e0, F.st));
-        fn();
+        launch();
         CK(cudaEventRecord(e1, F.st));
         CK(cudaEventSynchronize(e1));
         CK(cudaEventElapsedTime(&ms, e0, e1));
       }
-      return std::max(1e3f * ms, 1e-3f);
-    };
-    if (te.shape < 0) {
-      float best = 0.f;
-      for (int ci = 0; ci < kNShapes; ci++) {
-        const int tpc = kTuneShapes[ci][0], g = kTuneShapes[ci][1], ctas = kTuneShapes[ci][2];
-        if (!shape_fits(width, tpc, g, kTuneShapes[ci][3])) continue;  // the kernels' thread limits
-        if (ctas > 1 && width == 256 && tpc != 2) continue;  // the widest class: two threads per column
-        set_id_groups(shape_hint(ci));
-        te.us[ci] = timed(launch);
-        if (te.shape < 0 || te.us[ci] < best) {
-          best = te.us[ci];
-          te.shape = ci;
-        }
+      te.us[ci] = std::max(1e3f * ms, 1e-3f);
+      if (te.shape < 0 || te.us[ci] < best) {
+        best = te.us[ci];
+        te.shape = ci;
       }
     }
-    if (time_gram) te.gram_us = timed(gram);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     std::lock_guard<std::mutex> lk(g_tune_m);
     auto ins = g_tune.insert({key, te});
-    TuneEntry &have = ins.first->second;  // another thread may have tuned the key first
-    if (have.gram_us == 0.f && !have.pinned) have.gram_us = te.gram_us;
-    te = have;
+    shape = ins.first->second.shape;  // another thread may have tuned the key first
   }
-  if (have_gram && !te.pinned && te.gram_us < te.us[te.shape]) {
+  if (have_gram) {
+    set_id_groups(0);
     gram();
     return;
   }
-  set_id_groups(shape_hint(te.shape));
+  set_id_groups(shape_hint(shape));
   launch();
   set_id_groups(0);
 }
@@ -2000,7 +1991,7 @@ template <typename T> static void run_factor(Factor<T> &F) {
     // quantisation): partial sums of the largest phase
     bool have_gram = false;
     if constexpr (std::is_same<T, float>::value) {
-      have_gram = !large && F.eps >= ID_GRAM_EPS && H.bmax <= ID_GRAM_BMAX;
+      have_gram = !large && F.eps >= ID_GRAM_EPS && H.bmax >= ID_GRAM_BMIN && H.bmax <= ID_GRAM_BMAX;
       if (have_gram) {
         int64_t need = 0;
         for (auto &p : ph) need = std::max(need, id_gram_scratch_bytes(p.second, H.bmax, ring_max + F.px.np));
@@ -3557,7 +3548,7 @@ rss_status rss_autotune_set(int elem_bytes, int width, int phase_class, int tpc,
         (width == 256 && ctas > 1 && tpc != 2))
       throw Fail{RSS_EINVAL, "rss_autotune_set: bad arguments"};
     std::lock_guard<std::mutex> lk(g_tune_m);
-    TuneEntry te{shape, {}, 0.f, true};
+    TuneEntry te{shape, {}};
     g_tune[std::make_tuple(elem_bytes, width, phase_class)] = te;
   });
 }

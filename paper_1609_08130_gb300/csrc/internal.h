@@ -119,11 +119,16 @@ struct IdMultiScratch {
 };
 void set_id_multi(const IdMultiScratch &m);
 // The FP32 factor's ID from the exact Gram matrix of its rows (id_gram.cu):
-// tolerances from ID_GRAM_EPS up (five times the quantisation), boxes up to
-// ID_GRAM_BMAX wide (one CTA's threads run the pivoted Cholesky), scratch
-// (id_gram_scratch_bytes for a phase of nbox boxes, m rows) up to 4 GB.
+// tolerances from ID_GRAM_EPS up (five times the quantisation), levels whose
+// widest box has ID_GRAM_BMIN DOFs or more and at most ID_GRAM_BMAX (one CTA's
+// threads run the pivoted Cholesky), scratch (id_gram_scratch_bytes for a phase
+// of nbox boxes, m rows) up to 4 GB.  Where the lower line lies: a block is
+// padded to 64 columns, so for the narrowest boxes in large phases the
+// Householder form is faster (ID class, 128^2 boxes of 9: 5.3 against 5.9 ms, of
+// 4: 4.3 against 5.1; of 16: slower than Gram's 6.7), for all others 1.5 to 7
+// times slower (64^2 grid 4.0 against 1.14, 512^2 16.5 / 4.5, 32^3 58 / 7.7).
 constexpr double ID_GRAM_EPS = 5e-7;
-constexpr int ID_GRAM_BMAX = 512;
+constexpr int ID_GRAM_BMIN = 13, ID_GRAM_BMAX = 512;
 constexpr int64_t ID_GRAM_SCRATCH = (int64_t)4 << 30;
 int64_t id_gram_scratch_bytes(int nbox, int bmax, int m);
 void launch_id_gram(const LevelDev<float> &lv, FBox<float> *boxes, const int *box_list, int nbox, int bmax,
