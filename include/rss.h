@@ -271,7 +271,9 @@ rss_status rss_sqrt_apply(const rss_factorization *f, const double *x, double *y
  * (s a power of two; exact up to FP64 rounding), direct summation over all
  * pairs otherwise (in sums of three FP32 numbers, about 56 bits a term,
  * flushed into FP64 sums: an error no larger than that of a plain FP64 sum).
- * Device buffers, n x nrhs column-major. */
+ * A direct sum allocates nothing: its scratch, 192 bytes a point for passes of
+ * 16 columns, is the factor's (the convolution's is allocated by the first
+ * call).  Device buffers, n x nrhs column-major. */
 rss_status rss_matvec(const rss_factorization *f, const double *x, double *y, int nrhs);
 
 /* rss_sync -- wait for the factor's stream, then report an error the device

@@ -912,7 +912,11 @@ template <typename T> struct Factor : FactorBase {
   mutable bool grid_ready = false;
   int mv_ntile = 0;
   DBuf d_mv_ts, d_mv_te, d_mv_sb, d_mv_se;
-  DBuf d_mv_split;  // the points in FP32 parts (direct summation only)
+  // direct summation only: the points in FP32 parts, and room for the parts of
+  // MV_COLS columns, which rss_matvec fills and reads in launches queued
+  // together under mv_m (calls from several threads share the stream)
+  DBuf d_mv_split, d_mv_x;
+  mutable std::mutex mv_m;
   // rank proposal: the network (borrowed during rss_factor only), the
   // features of every box (MLP_NFEAT each, box order) and storage accounting
   // sweeps: work items (box, chunk) of every phase, per-box counters and
@@ -1430,6 +1434,7 @@ template <typename T> static void run_factor(Factor<T> &F) {
   detect_grid(F);
   if (F.grid_side == 0 && n > 0) {
     F.d_mv_split.alloc((size_t)matvec_split_bytes(n, dim), st);
+    F.d_mv_x.alloc((size_t)matvec_x_bytes(n, MV_COLS, F.mv_ntile), st);
     matvec_split(F.P.x, n, dim, F.d_mv_split.p, st);
     check_launch("point parts");
   }
@@ -2459,15 +2464,12 @@ template <typename T> static void apply_A_impl(const Factor<T> &F, const double 
                       ptr<int64_t>(F.d_mv_ts), ptr<int64_t>(F.d_mv_te), ptr<int64_t>(F.d_mv_sb),
                       ptr<int64_t>(F.d_mv_se), F.d_mv_split.p, F.st);
   } else {
-    // at most 32 columns at a time, so that the scratch stays a small part of
-    // the caller's vectors; stream-ordered, so calls do not share it
-    DBuf xbuf;
-    xbuf.alloc((size_t)matvec_x_bytes(F.n, std::min(nrhs, 32), F.mv_ntile), F.st);
-    for (int c = 0; c < nrhs; c += 32)
+    std::lock_guard<std::mutex> lk(F.mv_m);
+    for (int c = 0; c < nrhs; c += MV_COLS)
       launch_matvec(ptr<double>(F.d_x), F.dim, F.K, F.P.wdof, ptr<int64_t>(F.d_perm), x + (int64_t)c * F.n,
-                    y + (int64_t)c * F.n, F.n, std::min(nrhs - c, 32), F.mv_ntile, ptr<int64_t>(F.d_mv_ts),
+                    y + (int64_t)c * F.n, F.n, std::min(nrhs - c, MV_COLS), F.mv_ntile, ptr<int64_t>(F.d_mv_ts),
                     ptr<int64_t>(F.d_mv_te), ptr<int64_t>(F.d_mv_sb), ptr<int64_t>(F.d_mv_se), F.d_mv_split.p,
-                    xbuf.p, F.st);
+                    F.d_mv_x.p, F.st);
   }
   check_launch("residual operator");
 }

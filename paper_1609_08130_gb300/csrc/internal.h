@@ -218,6 +218,9 @@ void launch_permute(int dir, const int64_t *perm, const double *in, T *out_or_in
 // y = A x by direct summation in sums of three FP32 numbers (matvec.cu), FP64
 // in and out.  split: the points' parts (matvec_split, matvec_split_bytes); xbuf:
 // matvec_x_bytes of scratch.
+// Columns a pass of the direct sum: two groups of eight in one launch, 192 bytes of
+// scratch a point.
+constexpr int MV_COLS = 16;
 int64_t matvec_split_bytes(int64_t n, int dim);
 int64_t matvec_x_bytes(int64_t n, int nrhs, int ntile);
 void matvec_split(const double *x_tree, int64_t n, int dim, void *split, cudaStream_t st);
