@@ -184,14 +184,21 @@ rss_status rss_factor_batched(int nprob, const double *const *pts, const int64_t
                               double eps, int leaf_size, const rss_options *opts, rss_factorization **out);
 
 /* rss_apply -- y = F x (Eq. 3.10).  x, y: device, n x nrhs column-major,
- * original point order; may not alias.  nrhs >= 1. */
+ * original point order; may not alias.  nrhs >= 1.
+ * rss_apply, rss_solve and what is built on them keep working space with the
+ * factor until rss_free, grown by the first call with that many columns:
+ * vectors of up to 64 columns, and for more than four columns partial sums of up
+ * to a quarter of the factor's storage (a sixty-fourth for every four columns).
+ * rss_stats does not count it. */
 rss_status rss_apply(const rss_factorization *f, const double *x, double *y, int nrhs);
 
 /* rss_solve -- x = F^{-1} b (Eq. 3.11).  b, x: device, n x nrhs column-major;
  * may not alias.  nrhs >= 1. */
 rss_status rss_solve(const rss_factorization *f, const double *b, double *x, int nrhs);
 
-/* rss_solve_noalloc -- x = F^{-1} b, the same result as rss_solve, for callers
+/* rss_solve_noalloc -- x = F^{-1} b, rss_solve's result (to rounding: calls of
+ * more than four columns go through the one-CTA-per-box sweeps, which are several
+ * times slower than rss_solve's groups of four), for callers
  * that must not have the library allocate device memory during the call:
  * programs that hand all device memory to their own allocator up front, or
  * that keep a fixed memory budget inside a hot loop and cannot afford an
@@ -200,9 +207,8 @@ rss_status rss_solve(const rss_factorization *f, const double *b, double *x, int
  * variant never does.  The paper has no counterpart to this entry point.
  *   Working space is one fixed 16 MiB array in device memory that exists
  *   once per device from the moment the library is loaded until the process
- *   exits.  The columns are solved in passes (as rss_solve does, at most as
- *   many columns as the sweep kernels' shared memory takes, and fewer if the
- *   array needs it); a pass of c columns keeps n x c plus 2 * ntop * c
+ *   exits.  The columns are solved in passes (at most as many columns as
+ *   those kernels' shared memory takes, and fewer if the array needs it); a pass of c columns keeps n x c plus 2 * ntop * c
  *   entries there, in the factor's precision (4 bytes for a RSS_MIXED
  *   factor, 8 for RSS_FP64).  If a single column does not fit (about 4.19 M
  *   points for RSS_MIXED, 2.09 M for RSS_FP64, less twice the top-block
@@ -211,7 +217,8 @@ rss_status rss_solve(const rss_factorization *f, const double *b, double *x, int
  *   The first call made with a given device current looks up the array's
  *   device address (cudaGetSymbolAddress) and raises the sweep kernels'
  *   shared-memory limits on that device; make that first call before any
- *   stream capture begins.
+ *   stream capture begins.  What a captured call refers to stays in place until
+ *   rss_free, whatever other calls the factor serves meanwhile.
  *   Every call uses the same array: calls whose work overlaps on the GPU
  *   (different streams, different host threads) race and give wrong
  *   results.  Calls serialised on one stream are safe.

@@ -1,7 +1,7 @@
 // tc.cuh -- inline-PTX helpers for the 5th-generation tensor cores of sm_103a
 // (tcgen05: MMA with operands in shared memory and the accumulator in tensor
 // memory), mbarriers and the async-proxy fence.  Used by the FP32 Schur
-// update (schur_tc.cu).
+// update (schur_tc.cu) and the Gram form of the ID (id_gram.cu).
 //
 // Operand layout: "K-major, no swizzle" -- a tile of R rows x K columns of
 // 32-bit elements is stored as K/8 slabs of R x 8; inside a slab, core

@@ -3,12 +3,12 @@
 //
 // Right-looking blocked LU, every problem's block in each launch (grid
 // dimension), a panel per step:
-//   k_lu_panel  one CTA per problem: a thread holds its rows of the panel in
-//               registers; a column step is one barrier (every warp publishes
-//               its best row, every warp picks the winner by a reduction over
-//               the warps' keys); rows are moved once at the end;
-//   k_lu_trsm   the panel's row moves on the other columns, U12;
-//   k_lu_gemm   A22 -= L21 U12.
+//   k_top_panel  one CTA per problem: a thread holds its rows of the panel in
+//                registers; a column step is one barrier (every warp publishes
+//                its best row, every warp picks the winner by a reduction over
+//                the warps' keys); rows are moved once at the end;
+//   k_top_trsm   the panel's row moves on the other columns, U12;
+//   k_top_trail  A22 -= L21 U12.
 // Each launch is a programmatic dependent of the one before.  Bound: the chain
 // of n column steps.  Measured, LU and inverse: FP32 n = 305 1.29 -> 0.46 ms (a
 // panel in shared memory with three barriers a column before), n = 1600
@@ -67,8 +67,8 @@ struct Moves {
 // Pivot: largest |entry| (by pivot_key), rows moved at the end as the
 // sequence of interchanges would.
 template <typename T, int NB, int RPT>
-__global__ void __launch_bounds__(PT) k_lu_panel(T *LUall, const int64_t *loff, const int *tn, int *pivall,
-                                                 const int64_t *toff, int kb, Moves *moves, int *err) {
+__global__ void __launch_bounds__(PT) k_top_panel(T *LUall, const int64_t *loff, const int *tn, int *pivall,
+                                                  const int64_t *toff, int kb, Moves *moves, int *err) {
   constexpr int NW = PT / 32, VW = Pack<T>::N;
   __shared__ unsigned s_key[2][NW];
   __shared__ int s_idx[2][NW], s_prow[NB], s_at[PT * RPT], s_where[PT * RPT];
@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(PT) k_lu_panel(T *LUall, const int64_t *loff, 
         if (c < nb) o[c] = a[q][c];
     }
   }
-  // the moves, for k_lu_trsm, and on the permutation
+  // the moves, for k_top_trsm, and on the permutation
   Moves &M = moves[p];
   int dst = -1, src = 0, pv = 0;
   if (tid < 2 * nb) {
@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(PT) k_lu_panel(T *LUall, const int64_t *loff, 
 // The panel's row moves on every column outside it (all loads of a column
 // before its stores), then U12 = L11^{-1} A12 right of it; a thread per column.
 template <typename T, int NB>
-__global__ void __launch_bounds__(64) k_lu_trsm(T *LUall, const int64_t *loff, const int *tn, int kb,
+__global__ void __launch_bounds__(64) k_top_trsm(T *LUall, const int64_t *loff, const int *tn, int kb,
                                                 const Moves *moves) {
   __shared__ T s_l[NB][NB + 1];
   __shared__ T s_v[2 * NB][64];
@@ -263,7 +263,7 @@ __global__ void __launch_bounds__(64) k_lu_trsm(T *LUall, const int64_t *loff, c
 
 // A22 -= L21 U12 (64 x 64 tiles, inner dimension NB)
 template <typename T, int NB>
-__global__ void __launch_bounds__(256) k_lu_gemm(T *LUall, const int64_t *loff, const int *tn, int kb) {
+__global__ void __launch_bounds__(256) k_top_trail(T *LUall, const int64_t *loff, const int *tn, int kb) {
   __shared__ T Ls[NB][64 + 1], Us[NB][64 + 1];
   pdl_enter();
   const int p = blockIdx.z, n = tn[p];
@@ -328,13 +328,13 @@ static void launch_pdl(K kernel, dim3 grid, int threads, size_t smem, cudaStream
 template <typename T, int NB, int RPT>
 static void lu_step(T *LU, const int64_t *loff, int *piv, const int64_t *toff, const int *tn, int nprob, int maxn,
                     int kb, Moves *moves, int *err, cudaStream_t st) {
-  launch_pdl(k_lu_panel<T, NB, RPT>, dim3(nprob), PT, 0, st, LU, loff, tn, piv, toff, kb, moves, err);
+  launch_pdl(k_top_panel<T, NB, RPT>, dim3(nprob), PT, 0, st, LU, loff, tn, piv, toff, kb, moves, err);
   if (maxn <= NB) return;
-  launch_pdl(k_lu_trsm<T, NB>, dim3((maxn + 63) / 64, nprob), 64, 0, st, LU, loff, tn, kb, (const Moves *)moves);
+  launch_pdl(k_top_trsm<T, NB>, dim3((maxn + 63) / 64, nprob), 64, 0, st, LU, loff, tn, kb, (const Moves *)moves);
   const int rem = maxn - kb - NB;
   if (rem > 0) {
     const int t = (rem + 63) / 64;
-    launch_pdl(k_lu_gemm<T, NB>, dim3(t, t, nprob), 256, 0, st, LU, loff, tn, kb);
+    launch_pdl(k_top_trail<T, NB>, dim3(t, t, nprob), 256, 0, st, LU, loff, tn, kb);
   }
 }
 
