@@ -306,10 +306,15 @@ def run_reference(args, rank, world):
 
 
 # DRAM bytes (read + write) per launch of a kernel class from an ncu capture,
-# valid only for the kernel source it was taken on (sha-256 of kernels.cu).
-# Entry: class -> {"bytes_per_launch": ..., "kernels_sha256": ...}; none is held
-# for the current source.
-NCU_TRAFFIC = {}
+# valid only for the kernel source it was taken on (sha-256 of "source",
+# kernels.cu where none is named).
+NCU_TRAFFIC = {
+    # the ID's DRAM bytes per phase of the 512^2 step: a capture of both ID
+    # kernels in every phase of the 256^2 factorization, scaled by box count
+    # per depth
+    "id": {"bytes_per_launch": 80.9e6, "source": "id_gram.cu",
+           "kernels_sha256": "696ea74f066694281bb1e0a1aa637f08dcb7ae5633ca9c48aa4b3a6f502583d4"},
+}
 
 
 def ncu_traffic(cls):
@@ -317,7 +322,7 @@ def ncu_traffic(cls):
     t = NCU_TRAFFIC.get(cls)
     if t is None:
         return None
-    src = os.path.join(ROOT, "paper_1609_08130_gb300", "csrc", "kernels.cu")
+    src = os.path.join(ROOT, "paper_1609_08130_gb300", "csrc", t.get("source", "kernels.cu"))
     with open(src, "rb") as fh:
         if hashlib.sha256(fh.read()).hexdigest() != t["kernels_sha256"]:
             return None
