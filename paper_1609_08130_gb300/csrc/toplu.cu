@@ -386,8 +386,9 @@ __global__ void __launch_bounds__(64) k_diag_inverse(const T *LUall, const int64
 #pragma unroll
     for (int i = 0; i < DB; i++) {
       T s = (T)(i == lane);
+      if (i < nb)  // rows past the block are the identity's
 #pragma unroll
-      for (int l = 0; l < i; l++) s -= s_a[i][l] * x[l];
+        for (int l = 0; l < i; l++) s -= s_a[i][l] * x[l];
       x[i] = s;
       o[i * DB + lane] = s;
     }
@@ -395,10 +396,13 @@ __global__ void __launch_bounds__(64) k_diag_inverse(const T *LUall, const int64
 #pragma unroll
     for (int i = DB - 1; i >= 0; i--) {
       T s = (T)(i == lane);
+      if (i < nb) {
 #pragma unroll
-      for (int l = DB - 1; l > i; l--) s -= s_a[i][l] * x[l];
-      x[i] = s / s_a[i][i];
-      o[DB * DB + i * DB + lane] = x[i];
+        for (int l = DB - 1; l > i; l--) s -= s_a[i][l] * x[l];
+        s /= s_a[i][i];
+      }
+      x[i] = s;
+      o[DB * DB + i * DB + lane] = s;
     }
   }
 }
