@@ -2021,6 +2021,8 @@ template <typename T> static void run_factor(Factor<T> &F) {
       check_launch("id");
       F.prof.end(pi, st);
       pi = F.prof.begin(KC_ELIM, st, base + p.first, p.second);
+      if (F.flags & RSS_FLAG_HYBRID)
+        launch_mean_blocks<T>(view, ptr<FBox<T>>(F.d_boxes), bl, p.second, H.bmax, st);
       auto elim_launch = [&] {
         launch_elim<T>(view, ptr<FBox<T>>(F.d_boxes), bl, p.second, large ? -H.bmax : H.bmax, ptr<T>(gel), el_stride,
                        ovf, st, ptr<int>(F.d_err), njmax_lvl);

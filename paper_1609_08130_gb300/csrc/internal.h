@@ -135,6 +135,9 @@ void launch_id_gram(const LevelDev<float> &lv, FBox<float> *boxes, const int *bo
                     int ring_max, const Points &P, const KernelParams &K, const ProxyParams &px,
                     const float *proxy_unit, double eps, void *scratch, cudaStream_t st, int *err);
 template <typename T>
+void launch_mean_blocks(const LevelDev<T> &lv, const FBox<T> *boxes, const int *box_list, int nbox, int bmax,
+                        cudaStream_t st);
+template <typename T>
 void launch_elim(const LevelDev<T> &lv, FBox<T> *boxes, const int *box_list, int nbox, int bmax,
                  T *scratch, int64_t scratch_stride, const Overflow<T> &ovf, cudaStream_t st, int *err, int njmax);
 template <typename T>

@@ -3148,6 +3148,34 @@ __global__ void __launch_bounds__(NT) k_elim_inv(const FBox<float> *boxes, const
     for (int i = tid; i < r; i += NT) fb.Xi[i + (int64_t)fb.piv[c0 + c] * r] = x[c * ld + i];
 }
 
+// The own pair block of every box of a phase replaced by the mean of it and its
+// transpose.  For RS-WS: a weak step's Schur update is symmetric only as far as
+// X_RR^{-1} is, and the elimination reads one half of the block (first-kind
+// matrices, FP32: apply error 1.8e-5 without, 6e-6 with, 9e-6 when both halves were
+// eliminated; geometric means of 20 problems).
+template <typename T>
+__global__ void __launch_bounds__(NT) k_mean_block(LevelDev<T> lv, const FBox<T> *boxes, const int *box_list) {
+  const FBox<T> &fb = boxes[box_list[blockIdx.x]];
+  const int b = fb.b;
+  T *A = lv.pool + lv.pair_off[(int64_t)fb.cell * lv.NB + code5(0, 0, 0, lv.dim)];
+  for (int e = blockIdx.y * NT + threadIdx.x; e < b * b; e += gridDim.y * NT) {
+    const int i = e % b, j = e / b;
+    if (i <= j) continue;
+    T *x = A + i + (int64_t)j * b, *y = A + j + (int64_t)i * b;
+    const T m = (T)0.5 * (*x + *y);
+    *x = m;
+    *y = m;
+  }
+}
+
+template <typename T>
+void launch_mean_blocks(const LevelDev<T> &lv, const FBox<T> *boxes, const int *box_list, int nbox, int bmax,
+                        cudaStream_t st) {
+  if (nbox == 0) return;
+  k_mean_block<T><<<dim3(nbox, std::min(64, bmax * bmax / (4 * NT) + 1)), NT, 0, st>>>(lv, boxes, box_list);
+  count_launch();
+}
+
 // Shape of the next k_elim2 launch on this thread: (split << 4) | CTAs per
 // box, or 0 for the built-in choice.  Set by the host's autotuner.
 static thread_local int elim_shape_hint = 0;
@@ -4209,6 +4237,7 @@ void launch_permute(int dir, const int64_t *perm, const double *in, T *tv, doubl
                              const KernelParams &, const ProxyParams &, const T *, double, T *, int64_t, bool,       \
                              cudaStream_t,                                                                   \
                              int *);                                                                          \
+  template void launch_mean_blocks<T>(const LevelDev<T> &, const FBox<T> *, const int *, int, int, cudaStream_t); \
   template void launch_elim<T>(const LevelDev<T> &, FBox<T> *, const int *, int, int, T *, int64_t,            \
                                const Overflow<T> &, cudaStream_t, int *, int);                                \
   template void launch_schur<T>(const LevelDev<T> &, const FBox<T> *, const int *, int, int, const T *, int64_t, \
