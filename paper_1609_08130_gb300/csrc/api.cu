@@ -875,6 +875,8 @@ template <typename T> struct Factor : FactorBase {
   std::vector<int64_t> h_toff, h_loff;
   DBuf d_top, d_topLU, d_toppiv, d_tn, d_toff, d_loff;
   DBuf d_topinv;  // U^{-1} L^{-1} of the top blocks (orders up to top_lu_limit), else empty
+  DBuf d_topnorm; // and its, L's and U's norms, three a problem
+  mutable int top_plain = -1;  // 1: no block needs its solves corrected; -1: not looked at
   mutable DBuf d_work, d_topwork;
   // Cholesky factors of the diagonal blocks for the generalized square root
   // (rss_sqrt_apply), built on its first use
@@ -2198,10 +2200,11 @@ template <typename T> static void run_factor(Factor<T> &F) {
       check_launch("top lu");
       // the solves multiply by U^{-1} L^{-1} instead of two triangular sweeps
       F.d_topinv.alloc((size_t)F.h_loff[np] * sizeof(T) + 16, st);
+      F.d_topnorm.alloc(sizeof(unsigned) * 3 * (size_t)np, st);
       d_diag.alloc((size_t)top_inverse_scratch_elems(np, maxt) * sizeof(T), st, 1);
       F.factor_bytes += F.h_loff[np] * (int64_t)sizeof(T);
       launch_top_inverse<T>(ptr<T>(F.d_topLU), ptr<int64_t>(F.d_loff), ptr<int>(F.d_tn), np, maxt, ptr<T>(F.d_topinv),
-                            ptr<T>(d_diag), st);
+                            ptr<T>(d_diag), ptr<unsigned>(F.d_topnorm), st);
       check_launch("top inverse");
     } else if (np == 1) {
       DBuf d_panel;  // column-major copy of the current panel
@@ -2283,6 +2286,24 @@ template <typename T> static int group_columns(const Factor<T> &F, int nrhs) {
   return 4;
 }
 
+// The norms of the top blocks' factors if the solves by the inverse may need
+// their correction (launch_top), else null: not for one problem of up to 1024
+// DOFs and one group, where the inverse has always been taken, and not where the
+// norms of every block rule it out.  A factor that answers asynchronously
+// leaves that to the kernels, the others read the norms once.
+template <typename T> static const unsigned *top_correction(const Factor<T> &F, int groups) {
+  if (!F.d_topinv.p || (F.nprob == 1 && F.ntop <= 1024 && groups == 1)) return nullptr;
+  if (F.top_plain < 0 && !F.async()) {
+    std::vector<float> q(3 * (size_t)F.nprob);
+    CK(cudaMemcpyAsync(q.data(), F.d_topnorm.p, sizeof(float) * q.size(), cudaMemcpyDeviceToHost, F.st));
+    CK(cudaStreamSynchronize(F.st));
+    bool plain = true;
+    for (int p = 0; p < F.nprob; p++) plain &= q[3 * p] * q[3 * p + 1] * q[3 * p + 2] <= TOP_PLAIN;
+    F.top_plain = plain;
+  }
+  return F.top_plain == 1 ? nullptr : ptr<unsigned>(F.d_topnorm);
+}
+
 // One phase of a sweep over `groups` groups of nr columns.
 template <typename T>
 static void sweep_phase(const Factor<T> &F, int mode, const Phase &p, T *v, int nr, int groups, cudaStream_t st) {
@@ -2325,7 +2346,7 @@ static void enqueue_sweeps(const Factor<T> &F, const double *in, double *out, T 
   pi = begin(KC_TOP, 0, 0, 0, nt * nt * sz + 2.0 * nt * nrhs * sz, 2.0 * nt * nt * nrhs);
   launch_top<T>(solve ? 0 : 1, ptr<T>(F.d_topLU), ptr<int64_t>(F.d_loff), ptr<int>(F.d_toppiv), ptr<int64_t>(F.d_top),
                 ptr<int64_t>(F.d_toff), ptr<int>(F.d_tn), F.nprob, F.ntop, v, F.n, nr, groups, ptr<T>(F.d_topwork), st,
-                F.d_topinv.p ? ptr<T>(F.d_topinv) : nullptr);
+                F.d_topinv.p ? ptr<T>(F.d_topinv) : nullptr, solve ? top_correction(F, groups) : nullptr);
   end(pi);
   for (auto it = F.phases.rbegin(); it != F.phases.rend(); ++it) {
     pi = begin(KC_SWEEP, it->first, it->count, nrhs);
@@ -2854,7 +2875,7 @@ static void solve_noalloc(const Factor<T> &F, const double *b, double *x, int nr
     for (const Phase &p : F.phases) sweep_phase<T>(F, SWEEP_SOLVE_FWD, p, v, nc, 1, st);
     launch_top<T>(0, ptr<T>(F.d_topLU), ptr<int64_t>(F.d_loff), ptr<int>(F.d_toppiv), ptr<int64_t>(F.d_top),
                   ptr<int64_t>(F.d_toff), ptr<int>(F.d_tn), F.nprob, F.ntop, v, F.n, nc, 1, topwork, st,
-                  F.d_topinv.p ? ptr<T>(F.d_topinv) : nullptr);
+                  F.d_topinv.p ? ptr<T>(F.d_topinv) : nullptr, top_correction(F, 1));
     for (auto it = F.phases.rbegin(); it != F.phases.rend(); ++it) sweep_phase<T>(F, SWEEP_SOLVE_BWD, *it, v, nc, 1, st);
     launch_permute<T>(1, ptr<int64_t>(F.d_perm), nullptr, v, xc, F.n, nc, nc, st);
     check_launch("rss_solve_noalloc");

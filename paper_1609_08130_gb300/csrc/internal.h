@@ -187,16 +187,19 @@ void sweep_chunk_attributes();
 // Set the shared-memory attributes of every sweep kernel on the current device.
 void sweep_kernel_attributes();
 // Top blocks: mode 0 solves with the LU factors or, with Winv = U^{-1} L^{-1}
-// and groups of at most 4 columns, multiplies by it (and, several problems,
-// several groups or orders past 1024, corrects the result by its residual);
-// mode 1 multiplies by the block.
+// and groups of at most 4 columns, multiplies by it; with norms
+// (launch_top_inverse's) the result of every block whose three numbers' product
+// is above TOP_PLAIN is corrected by its residual.  Mode 1 multiplies by the
+// block.
+constexpr float TOP_PLAIN = 1e4f;
 template <typename T>
 void launch_top(int mode, const T *LU, const int64_t *loff, const int *piv, const int64_t *top, const int64_t *toff,
                 const int *tn, int nprob, int ntop_total, T *v, int64_t n, int nr, int groups, T *work,
-                cudaStream_t st, const T *Winv = nullptr);
+                cudaStream_t st, const T *Winv = nullptr, const unsigned *norms = nullptr);
 // Top blocks up to top_lu_limit (toplu.cu): the LU of every problem's block
 // (maxn: the largest order; scratch: top_lu_scratch_bytes) and
-// W = U^{-1} L^{-1} at the same offsets (D: top_inverse_scratch_elems of T).
+// W = U^{-1} L^{-1} at the same offsets (D: top_inverse_scratch_elems of T;
+// norms: three numbers a problem).
 int top_lu_limit(int elem);
 int64_t top_lu_scratch_bytes(int nprob);
 int64_t top_inverse_scratch_elems(int nprob, int maxn);
@@ -205,7 +208,7 @@ void launch_top_lu(T *LU, const int64_t *loff, int *piv, const int64_t *toff, co
                    void *scratch, cudaStream_t st, int *err);
 template <typename T>
 void launch_top_inverse(const T *LU, const int64_t *loff, const int *tn, int nprob, int maxn, T *W, T *D,
-                        cudaStream_t st);
+                        unsigned *norms, cudaStream_t st);
 template <typename T>
 void launch_lu_batched(T *LU, const int64_t *loff, int *piv, const int64_t *toff, const int *tn, int nprob,
                        cudaStream_t st, int *err);

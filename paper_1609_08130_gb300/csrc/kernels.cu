@@ -4026,12 +4026,17 @@ __global__ void __launch_bounds__(256) k_top_gather(const int *piv, const int64_
 // n = 1500 and 2000: FP64 4.2e-13 and 2.8e-13 against 6.5e-14 and 3.9e-14, FP32
 // 2.0e-4 against 5.3e-5 at 1500), so where those were taken before, the
 // solution is corrected once by its residual L U z - y: three launches more
-// instead of 2 n row steps.
+// instead of 2 n row steps.  Blocks whose norms (largest row sums) rule that loss
+// out keep the product: |W| |L| |U| is 2 to 2300 for second-kind matrices at eps
+// 1e-6 (64^2 to 512^2, 32^3, scattered points; error of solve after apply with and
+// without the correction 4.5e-16 and 4.5e-16 on the 100^2 grid, 5.3e-16 with
+// triangular solves), 5e5 and more for first-kind ones.  The FP64 solve of 16
+// columns at n = 1500 spends 100 us on the correction's products.
 enum { TOP_SOLVE, TOP_FIRST, TOP_U, TOP_RESIDUAL, TOP_CORRECT };
 template <typename T, int NR, int STEP>
 __global__ void __launch_bounds__(256) k_top_gemv(const T *Aall, const int64_t *loff, const int64_t *topall,
                                                   const int64_t *toff, int nprob, int ntot, T *y, int64_t wstride,
-                                                  T *v, int64_t vstride) {
+                                                  T *v, int64_t vstride, const unsigned *norms) {
   const int lane = threadIdx.x & 31, e = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (e >= ntot) return;
   const int p = problem_of(toff, nprob, e);
@@ -4040,11 +4045,17 @@ __global__ void __launch_bounds__(256) k_top_gemv(const T *Aall, const int64_t *
   y += blockIdx.y * wstride;
   v += blockIdx.y * vstride;
   T *z = y + (int64_t)ntot * NR;
+  bool plain = false;
+  if (STEP == TOP_U || STEP == TOP_RESIDUAL || STEP == TOP_CORRECT) {
+    const unsigned *q = norms + 3 * p;
+    plain = __uint_as_float(q[0]) * __uint_as_float(q[1]) * __uint_as_float(q[2]) <= TOP_PLAIN;
+    if (plain && STEP != TOP_CORRECT) return;
+  }
   const T *Ai = Aall + loff[p] + (int64_t)i * n;
   T acc[NR];
 #pragma unroll
   for (int c = 0; c < NR; c++) acc[c] = (T)0;
-  const int l0 = STEP == TOP_U ? i : 0, l1 = STEP == TOP_RESIDUAL ? i : n;
+  const int l0 = STEP == TOP_U ? i : 0, l1 = plain ? 0 : STEP == TOP_RESIDUAL ? i : n;
 #pragma unroll 4
   for (int l = l0 + lane; l < l1; l += 32) {
     const T w = Ai[l];
@@ -4068,16 +4079,16 @@ __global__ void __launch_bounds__(256) k_top_gemv(const T *Aall, const int64_t *
 template <typename T, int NR>
 static void launch_top_nr(int mode, const T *LU, const int64_t *loff, const int *piv, const int64_t *top,
                           const int64_t *toff, int nprob, int ntop, T *v, int64_t vstride, int groups, T *work,
-                          int64_t wstride, const T *Winv, cudaStream_t st) {
+                          int64_t wstride, const T *Winv, const unsigned *norms, cudaStream_t st) {
   const dim3 rows((unsigned)((ntop + 7) / 8), groups);
   if (mode == 0) {
     k_top_gather<T, NR><<<dim3((unsigned)((ntop + 255) / 256), groups), 256, 0, st>>>(piv, top, toff, nprob, ntop, v,
                                                                                      vstride, work, wstride);
     auto run = [&](auto kern, const T *A) {
-      kern<<<rows, 256, 0, st>>>(A, loff, top, toff, nprob, ntop, work, wstride, v, vstride);
+      kern<<<rows, 256, 0, st>>>(A, loff, top, toff, nprob, ntop, work, wstride, v, vstride, norms);
       count_launch();
     };
-    if (nprob == 1 && ntop <= 1024 && groups == 1) {
+    if (!norms) {
       run(k_top_gemv<T, NR, TOP_SOLVE>, Winv);
     } else {
       run(k_top_gemv<T, NR, TOP_FIRST>, Winv);
@@ -4096,12 +4107,12 @@ static void launch_top_nr(int mode, const T *LU, const int64_t *loff, const int 
 template <typename T>
 void launch_top(int mode, const T *LU, const int64_t *loff, const int *piv, const int64_t *top, const int64_t *toff,
                 const int *tn, int nprob, int ntop_total, T *v, int64_t n, int nr, int groups, T *work,
-                cudaStream_t st, const T *Winv) {
+                cudaStream_t st, const T *Winv, const unsigned *norms) {
   if (ntop_total == 0 || nprob == 0) return;
   const int64_t vs = n * nr, ws = (int64_t)2 * ntop_total * nr;
   if (nr <= 4 && (mode == 1 || Winv)) {
 #define RSS_TOP_NR(N) \
-  case N: launch_top_nr<T, N>(mode, LU, loff, piv, top, toff, nprob, ntop_total, v, vs, groups, work, ws, Winv, st); break;
+  case N: launch_top_nr<T, N>(mode, LU, loff, piv, top, toff, nprob, ntop_total, v, vs, groups, work, ws, Winv, norms, st); break;
     switch (nr) { RSS_TOP_NR(1) RSS_TOP_NR(2) RSS_TOP_NR(3) RSS_TOP_NR(4) }
 #undef RSS_TOP_NR
     return;
@@ -4249,7 +4260,8 @@ void launch_permute(int dir, const int64_t *perm, const double *in, T *tv, doubl
   template void launch_chol_apply<T>(const FBox<T> *, int, const int64_t *, const int64_t *, const int *, int,     \
                                      const T *, const int64_t *, T *, int, int, int, cudaStream_t);              \
   template void launch_top<T>(int, const T *, const int64_t *, const int *, const int64_t *, const int64_t *,     \
-                              const int *, int, int, T *, int64_t, int, int, T *, cudaStream_t, const T *);   \
+                              const int *, int, int, T *, int64_t, int, int, T *, cudaStream_t, const T *,    \
+                              const unsigned *);                                                              \
   template void launch_lu_batched<T>(T *, const int64_t *, int *, const int64_t *, const int *, int, cudaStream_t, \
                                      int *);                                                                  \
   template void launch_permute<T>(int, const int64_t *, const double *, T *, double *, int64_t, int, int,     \

@@ -484,13 +484,31 @@ __global__ void __launch_bounds__(256) k_top_inverse(const T *LUall, const int64
   }
 }
 
+// Largest row sums of |W|, |L| and |U| of every problem (as FP32 bits), a warp per
+// row: their product bounds what a solve by W loses against triangular solves.
+template <typename T>
+__global__ void __launch_bounds__(256) k_top_norms(const T *LUall, const T *Wall, const int64_t *loff, const int *tn,
+                                                   unsigned *norms) {
+  const int p = blockIdx.y, n = tn[p], lane = threadIdx.x & 31, i = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (i >= n) return;
+  const T *a = LUall + loff[p] + (int64_t)i * n, *w = Wall + loff[p] + (int64_t)i * n;
+  T sw = (T)0, sl = (T)0, su = (T)0;
+  for (int l = lane; l < n; l += 32) {
+    sw += fabs(w[l]);
+    (l < i ? sl : su) += fabs(a[l]);
+  }
+  const float v[3] = {(float)warp_sum(sw), (float)warp_sum(sl) + 1.f, (float)warp_sum(su)};
+  if (lane == 0)
+    for (int q = 0; q < 3; q++) atomicMax(norms + 3 * p + q, __float_as_uint(v[q]) & 0x7fffffffu);
+}
+
 int64_t top_inverse_scratch_elems(int nprob, int maxn) {
   return (int64_t)nprob * ((maxn + DB - 1) / DB) * (2 * DB * DB);
 }
 
 template <typename T>
 void launch_top_inverse(const T *LU, const int64_t *loff, const int *tn, int nprob, int maxn, T *W, T *D,
-                        cudaStream_t st) {
+                        unsigned *norms, cudaStream_t st) {
   if (maxn == 0 || nprob == 0) return;
   const int maxblk = (maxn + DB - 1) / DB;
   launch_pdl(k_diag_inverse<T>, dim3(maxblk, nprob), 64, 0, st, LU, loff, tn, maxblk, D);
@@ -504,12 +522,16 @@ void launch_top_inverse(const T *LU, const int64_t *loff, const int *tn, int npr
   if (cols >= 8 * 152 && sizeof(T) == 4) run(k_top_inverse<T, 8>, 8);
   else if (cols >= 4 * 152) run(k_top_inverse<T, 4>, 4);
   else run(k_top_inverse<T, 2>, 2);
+  cudaMemsetAsync(norms, 0, sizeof(unsigned) * 3 * (size_t)nprob, st);
+  k_top_norms<T><<<dim3((maxn + 7) / 8, nprob), 256, 0, st>>>(LU, W, loff, tn, norms);
+  count_launch();
 }
 
 #define RSS_INST(T)                                                                                                 \
   template void launch_top_lu<T>(T *, const int64_t *, int *, const int64_t *, const int *, int, int, void *,       \
                                  cudaStream_t, int *);                                                              \
-  template void launch_top_inverse<T>(const T *, const int64_t *, const int *, int, int, T *, T *, cudaStream_t);
+  template void launch_top_inverse<T>(const T *, const int64_t *, const int *, int, int, T *, T *, unsigned *,         \
+                                      cudaStream_t);
 RSS_INST(float)
 RSS_INST(double)
 

@@ -67,3 +67,17 @@ def test_several_problems(pkg, prec):
     z, off = _solve(f, np.concatenate(bs, axis=1)), np.cumsum([0] + sizes)
     r = [_gmean_ratio(z[:, o:o + n], _solve(g, b), x) for g, b, x, o, n in zip(single, bs, xs, off, sizes)]
     assert np.exp(np.mean(np.log(r))) <= 0.5
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("dim,kind", [(2, 0), (3, 1)])
+def test_well_conditioned_blocks_keep_the_plain_product(pkg, prec, dim, kind):
+    """Second-kind matrices: a wide call gives each column the bits of a narrow
+    one, since neither corrects anything."""
+    n = 700
+    f = pkg.Factorization(torch.from_numpy(inputs.random_points(97, n, dim)).cuda(), kind, 0.0, leaf=1024,
+                          prec=pkg.FP64 if prec == "fp64" else pkg.MIXED)
+    assert f.stats()["ntop"] == n
+    b = inputs.rhs(98, n, 9)
+    wide = _solve(f, b)
+    assert all(np.array_equal(wide[c], _solve(f, b[c])) for c in range(9))
